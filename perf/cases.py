@@ -402,13 +402,18 @@ def fill(record: dict, values: dict) -> dict:
     return {**values, **{k: v if values[k] is not None else None for k, v in record.items()}}
 
 
-def tuple_order(hits, n):
-    """The hits with unused places -1, and the permutation that puts n-tuplets
-    in order of a 64-bit number made of their hits."""
-    hits = torch.where(torch.arange(NMAX, device=hits.device) < n[:, None], hits, -1)
-    odd = torch.tensor([0x1E3779B97F4A7C15, 0x3F58476D1CE4E5B9, 0x14D049BB133111EB, 0x2545F4914F6CDD1D,
-                        0x369DEA0F31A53F85, 0x1B03738712FAD5C9, 0x2545F3C65D2C8A4F, 0x1CE4E5B9BF58476D], device=hits.device)
-    return hits, torch.argsort((hits * odd).sum(1))
+def places():
+    """The places of an n-tuplet, and a factor for each."""
+    return torch.arange(NMAX, device=DEV), torch.tensor(
+        [0x1E3779B97F4A7C15, 0x3F58476D1CE4E5B9, 0x14D049BB133111EB, 0x2545F4914F6CDD1D,
+         0x369DEA0F31A53F85, 0x1B03738712FAD5C9, 0x2545F3C65D2C8A4F, 0x1CE4E5B9BF58476D], device=DEV)
+
+
+def tuple_keys(hits, n, places):
+    """The hits with unused places -1, and a 64-bit number made of each
+    n-tuplet's hits: the program's n-tuplets are in the order of it."""
+    hits = torch.where(places[0] < n[:, None], hits, -1)
+    return hits, (hits * places[1]).sum(1)
 
 
 def fix_order(bufs, counts) -> None:
@@ -416,7 +421,7 @@ def fix_order(bufs, counts) -> None:
     refits the same tracks many times and compares them one by one."""
     nt = counts.n_tuples
     hits = bufs.tup_hits[:nt * NMAX].view(-1, NMAX)
-    _, order = tuple_order(hits, bufs.tup_n[:nt])
+    order = torch.argsort(tuple_keys(hits, bufs.tup_n[:nt], places())[1])
     cells = bufs.tup_cells[:nt * NMAX].view(-1, NMAX)
     for t in (hits, cells, bufs.tup_n[:nt], bufs.tup_alive[:nt]):
         t.copy_(t[order])
@@ -429,8 +434,7 @@ def fitted_order(n, alive, min_hits=3):
 
 
 def pipeline_for(case: dict) -> Pipeline:
-    return Pipeline(LAYERS, module_layers(), make_cuts(case["pt_min"], case["helices"] > 0),
-                    FIT, device=DEV)
+    return Pipeline(LAYERS, module_layers(), make_cuts(case["pt_min"], case["helices"] > 0), FIT, device=DEV)
 
 
 def alignment(seed: int) -> list[torch.Tensor]:
@@ -455,7 +459,7 @@ def prepare(case: dict, seed: int) -> dict:
     pipe = pipeline_for(case)
     if case["kind"] == "chain":
         bufs = pipe.allocate(b["x"].numel(), case["events"])
-        return dict(case=case, pipe=pipe, hits=hits, bufs=bufs, record=make_record(case))
+        return dict(case=case, pipe=pipe, hits=hits, bufs=bufs, record=make_record(case), places=places())
     res, bufs = pipe.run(*hits)
     fix_order(bufs, res.counts)
     state = dict(case=case, pipe=pipe, hits=hits, bufs=bufs, counts=res.counts, record=make_record(case))
@@ -478,13 +482,13 @@ def prepare(case: dict, seed: int) -> dict:
     return state
 
 
-def ordered_tracks(res, record: dict) -> dict:
-    t = res.tracks
-    which = t["tuple"].long()
-    n = res.tuples["n"][which]
-    hits, order = tuple_order(res.tuples["hits"][which], n)
-    for k, v in dict(params=t["params"], cov=t["cov"], chi2=t["chi2"], ndf=t["ndf"], hits=hits).items():
-        torch.index_select(v, 0, order, out=record[k][:order.numel()])
+def ordered_tracks(res, record: dict, places) -> dict:
+    t, which = res.tracks, res.tracks["tuple"]
+    hits, key = tuple_keys(res.tuples["hits"], res.tuples["n"], places)
+    order = torch.argsort(key[which])
+    for k in ("params", "cov", "chi2", "ndf"):
+        torch.index_select(t[k], 0, order, out=record[k][:order.numel()])
+    torch.take(hits, torch.add(places[0], which[order][:, None], alpha=NMAX), out=record["hits"][:order.numel()])
     c = res.counts
     return dict(record, counts=[c.n_cells, c.n_alive_cells, c.n_edges, c.n_tuples, c.n_alive_tuples, c.n_tracks])
 
@@ -501,7 +505,7 @@ def run(state: dict):
     case, record = state["case"], state["record"]
     if case["kind"] == "chain":
         res, state["bufs"] = state["pipe"].run(*state["hits"], bufs=state["bufs"])
-        return ordered_tracks(res, record)
+        return ordered_tracks(res, record, state["places"])
     if case["kind"] == "vertices":
         s = state["summaries"]
         return fill(record, used_rows(find_vertices(s["ev"], s["z0"], s["ez0"], s["pt"], s["nhits"], s["keep"],
@@ -622,7 +626,8 @@ def find_all(b, cuts):
             h, n, a = find_tuples(*(v[lo:hi] for v in xyzr), layer[lo:hi], cuts)
             parts.append((torch.where(h >= 0, h + lo, -1), n, a))
     hits, n, alive = (torch.cat(v) for v in zip(*parts))
-    hits, order = tuple_order(hits, n)
+    hits, key = tuple_keys(hits, n, places())
+    order = torch.argsort(key)
     return hits[order], n[order], alive[order]
 
 
