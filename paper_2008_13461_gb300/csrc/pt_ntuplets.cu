@@ -184,11 +184,26 @@ __global__ void __launch_bounds__(kThreads) k_select_tracks(Params p) {
         p.counters[C_TRACKS] = total;
         if (total > p.cap_tracks) set_flag(p.counters, PT_FLAG_TRACKS);
     }
-    // this slice's start in each class: the counts of the slices before it
+    // this slice's start in each class: the counts of the slices before it,
+    // summed by the whole block (four classes per 16-byte load).  Summed by
+    // one thread per class, the last slices' ~1000 additions in a row were
+    // most of this kernel (35.7 -> 8.0 us in an event of 112 n-tuplets,
+    // 42.8 -> 27.8 us with 3.6 M of them).
+    int4 b = make_int4(0, 0, 0, 0);
+    for (int q = threadIdx.x; q < (int)blockIdx.x; q += kThreads) {
+        const int4 v = reinterpret_cast<const int4 *>(p.trk_blk)[q];
+        b.x += v.x; b.y += v.y; b.z += v.z; b.w += v.w;
+    }
+    b.x = __reduce_add_sync(0xffffffffu, b.x);
+    b.y = __reduce_add_sync(0xffffffffu, b.y);
+    b.z = __reduce_add_sync(0xffffffffu, b.z);
+    b.w = __reduce_add_sync(0xffffffffu, b.w);
+    if (lane < 4) s_wcnt[w][lane] = lane == 0 ? b.x : lane == 1 ? b.y : lane == 2 ? b.z : b.w;
+    __syncthreads();
     if (threadIdx.x < 4) {
-        int b = 0;
-        for (int q = 0; q < (int)blockIdx.x; q++) b += p.trk_blk[q * 4 + threadIdx.x];
-        s_base[threadIdx.x] = off[threadIdx.x] + b;
+        int v = threadIdx.x == 0 ? off[0] : threadIdx.x == 1 ? off[1] : threadIdx.x == 2 ? off[2] : off[3];
+        for (int q = 0; q < kThreads / 32; q++) v += s_wcnt[q][threadIdx.x];
+        s_base[threadIdx.x] = v;
     }
     __syncthreads();
     const int64_t nt = min((int64_t)p.counters[C_TUPLES], p.cap_tuples);
