@@ -232,9 +232,9 @@ pt_status check_common(void *ws, size_t ws_bytes, const pt_hits *h, const pt_con
     return PT_OK;
 }
 
-int grid_for(const pt_config *cfg) {
-    int sms = num_sms();
-    return (sms > 0 ? sms : 1) * cfg->tuning.blocks_per_sm;
+Grid grid_for(const pt_config *cfg) {
+    const int sms = num_sms();
+    return {sms > 0 ? sms : 1, cfg->tuning.blocks_per_sm};
 }
 
 pt_status launched() { return cudaGetLastError() == cudaSuccess ? PT_OK : PT_ERR_CUDA; }
@@ -273,7 +273,7 @@ pt_status pt_build_doublets(void *ws, size_t ws_bytes, const pt_hits *hits, cons
     if (cudaMemsetAsync(p.bin_cnt, 0, sizeof(int32_t) * (size_t)(L.n_bins + 1), s) != cudaSuccess)
         return PT_ERR_CUDA;
     if (cudaMemsetAsync(p.in_live, 0, sizeof(int32_t) * (size_t)hits->n_hits, s) != cudaSuccess) return PT_ERR_CUDA;
-    const int grid = grid_for(cfg);
+    const Grid grid = grid_for(cfg);
     launch_binning(p, grid, s);
     launch_doublets(p, cfg->tuning.doublet_lanes, grid, s);
     // alignment within eps (sin) implies |u^ - v^| <= 2 sin(asin(eps)/2) <= eps pi/2;
@@ -347,13 +347,13 @@ pt_status pt_fit_tracks(void *ws, size_t ws_bytes, const pt_hits *hits, const pt
     p.trk_chi2 = tracks->chi2;
     p.trk_ndf = tracks->ndf;
     p.trk_tuple = tracks->tuple;
-    const int grid = grid_for(cfg);
+    const Grid grid = grid_for(cfg);
     cudaStream_t s = (cudaStream_t)stream;
     // the selection counts afresh on every call
     if (cudaMemsetAsync(p.counters + C_TRACKS, 0, sizeof(int32_t), s) != cudaSuccess ||
         cudaMemsetAsync(p.counters + C_TRK_CNT, 0, sizeof(int32_t) * 8, s) != cudaSuccess)
         return PT_ERR_CUDA;
-    launch_select(p, grid, s);
+    launch_select(p, s);
     launch_fit(p, grid, s);
     return launched();
 }

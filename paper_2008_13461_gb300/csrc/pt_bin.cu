@@ -175,14 +175,14 @@ __global__ void __launch_bounds__(kThreads) k_bin_fill(Params p) {
     }
 }
 
-void launch_binning(const Params &p, int grid, cudaStream_t s) {
+void launch_binning(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_bin_count", s);
-        k_bin_count<<<grid, kThreads, 0, s>>>(p);
+        k_bin_count<<<g.blocks(8), kThreads, 0, s>>>(p);
     }
     launch_scan(p.bin_cnt, p.n_bins, p.scan_part, s);
     KernelTimer t("k_bin_fill", s);
-    k_bin_fill<<<grid, kThreads, 0, s>>>(p);
+    k_bin_fill<<<g.blocks(8), kThreads, 0, s>>>(p);
 }
 
 }  // namespace ptk

@@ -297,13 +297,13 @@ __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
     }
 }
 
-void launch_connect(const Params &p, int grid, cudaStream_t s) {
+void launch_connect(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_connect", s);
-        k_connect<<<grid * (kThreads / (32 * kCaWarps)), 32 * kCaWarps, 0, s>>>(p);
+        k_connect<<<g.blocks(10), 32 * kCaWarps, 0, s>>>(p);
     }
     KernelTimer t("k_connect_exact", s);
-    k_connect_exact<<<grid / 8 + 1, 128, 0, s>>>(p);
+    k_connect_exact<<<g.blocks(4), 128, 0, s>>>(p);
 }
 
 }  // namespace ptk

@@ -274,9 +274,10 @@ __global__ void __launch_bounds__(kThreads) k_doublets_exact(Params p) {
         doublets_hit<G, true>(p, p.hit_bin[k], lane, 0xffffffffu, 0, s_inner[grp], s_pair[grp], s_row[grp], kBuf);
 }
 
-void launch_doublets(const Params &p, int lanes, int grid, cudaStream_t s) {
+void launch_doublets(const Params &p, int lanes, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_doublets", s);
+        const int grid = g.blocks(5);
         switch (lanes) {
         case 4: k_doublets<4><<<grid, kThreads, 0, s>>>(p); break;
         case 8: k_doublets<8><<<grid, kThreads, 0, s>>>(p); break;
@@ -285,7 +286,7 @@ void launch_doublets(const Params &p, int lanes, int grid, cudaStream_t s) {
         }
     }
     KernelTimer t("k_doublets_exact", s);
-    k_doublets_exact<<<grid / 4 + 1, kThreads, 0, s>>>(p);
+    k_doublets_exact<<<g.blocks(2), kThreads, 0, s>>>(p);
 }
 
 }  // namespace ptk

@@ -521,26 +521,26 @@ __global__ void __launch_bounds__(kThreads) k_fit(Params p) {
 }
 
 template <typename R>
-void launch_fit_r(const Params &p, int grid, cudaStream_t s) {
+void launch_fit_r(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_fit<3>", s);
-        k_fit<3, R><<<grid, kThreads, 0, s>>>(p);
+        k_fit<3, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_fit<4>", s);
-        k_fit<4, R><<<grid, kThreads, 0, s>>>(p);
+        k_fit<4, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_fit<5>", s);
-        k_fit<5, R><<<grid, kThreads, 0, s>>>(p);
+        k_fit<5, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
     }
     KernelTimer t("k_fit<6..8>", s);
-    k_fit<6, R><<<grid, kThreads, 0, s>>>(p);
+    k_fit<6, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
 }
 
-void launch_fit(const Params &p, int grid, cudaStream_t s) {
-    if (p.fit.solve_fp32) launch_fit_r<float>(p, grid, s);
-    else launch_fit_r<double>(p, grid, s);
+void launch_fit(const Params &p, const Grid &g, cudaStream_t s) {
+    if (p.fit.solve_fp32) launch_fit_r<float>(p, g, s);
+    else launch_fit_r<double>(p, g, s);
 }
 
 }  // namespace ptk

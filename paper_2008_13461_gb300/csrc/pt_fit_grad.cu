@@ -700,22 +700,22 @@ __global__ void __launch_bounds__(kThreads) k_align_grad(int n, const float *x, 
 
 }  // namespace
 
-void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, float *gx, float *gy, float *gz, int grid,
+void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, float *gx, float *gy, float *gz, const Grid &g,
                      cudaStream_t s) {
     {
         KernelTimer t("k_fit_grad<3>", s);
-        k_fit_grad<3><<<grid, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<3><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<4>", s);
-        k_fit_grad<4><<<grid, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<4><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<5>", s);
-        k_fit_grad<5><<<grid, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<5><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     KernelTimer t("k_fit_grad<6..8>", s);
-    k_fit_grad<6><<<grid, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+    k_fit_grad<6><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
 }
 
 void launch_align(int n, const float *x, const float *y, const float *z, const int32_t *module, const float *centre,

@@ -21,16 +21,26 @@ class KernelTimer {
     cudaEvent_t a_;
 };
 
+// Size of a persistent grid: `resident` blocks per SM (what the kernel's
+// registers and shared memory let an SM hold), or the tuning's factor when
+// that is smaller.  More blocks than are resident only start, find the queue
+// or the range used up, and end: 5-10 us of empty waves per kernel in the
+// smallest events with a grid of 24 blocks per SM whatever the kernel.
+struct Grid {
+    int sms, factor;
+    int blocks(int resident) const { return sms * (factor < resident ? factor : resident); }
+};
+
 void launch_scan(int32_t *a, int64_t n, int32_t *part, cudaStream_t s);
-void launch_binning(const Params &p, int grid, cudaStream_t s);
-void launch_doublets(const Params &p, int lanes, int grid, cudaStream_t s);
-void launch_fishbone(const Params &p, float unit_thr, float du, int grid, cudaStream_t s);
-void launch_connect(const Params &p, int grid, cudaStream_t s);
-void launch_ntuplets(const Params &p, int grid, cudaStream_t s);
-void launch_select(const Params &p, int grid, cudaStream_t s);
-void launch_fit(const Params &p, int grid, cudaStream_t s);
-void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, float *gx, float *gy, float *gz, int grid,
-                     cudaStream_t s);
+void launch_binning(const Params &p, const Grid &g, cudaStream_t s);
+void launch_doublets(const Params &p, int lanes, const Grid &g, cudaStream_t s);
+void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, cudaStream_t s);
+void launch_connect(const Params &p, const Grid &g, cudaStream_t s);
+void launch_ntuplets(const Params &p, const Grid &g, cudaStream_t s);
+void launch_select(const Params &p, cudaStream_t s);
+void launch_fit(const Params &p, const Grid &g, cudaStream_t s);
+void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, float *gx, float *gy, float *gz,
+                     const Grid &g, cudaStream_t s);
 void launch_ambiguities(const int32_t *hits, const int32_t *cells, const uint8_t *n, const int32_t *track_tuple,
                         int32_t n_tracks, const float *chi2, const float *tip, int32_t tip_stride, int32_t n_cells,
                         int32_t n_hits, uint32_t *scratch, uint8_t *keep, int grid, cudaStream_t s);

@@ -112,7 +112,7 @@ extern "C" pt_status pt_bin_hits_noalloc(const pt_hits *hits, const pt_geometry 
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return PT_ERR_CUDA;
-    launch_binning(p, sms * 8, s);
+    launch_binning(p, Grid{sms, 8}, s);
     if (cudaMemcpyAsync(flags, p.counters + C_FLAGS, sizeof(int32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return PT_ERR_CUDA;
     return cudaGetLastError() == cudaSuccess ? PT_OK : PT_ERR_CUDA;

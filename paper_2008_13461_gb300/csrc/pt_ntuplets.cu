@@ -238,8 +238,7 @@ __global__ void __launch_bounds__(kThreads) k_select_tracks(Params p) {
     }
 }
 
-void launch_select(const Params &p, int grid, cudaStream_t s) {
-    (void)grid;
+void launch_select(const Params &p, cudaStream_t s) {
     {
         KernelTimer t("k_count_tracks", s);
         k_count_tracks<<<kSelBlocks, kThreads, 0, s>>>(p);
@@ -248,21 +247,21 @@ void launch_select(const Params &p, int grid, cudaStream_t s) {
     k_select_tracks<<<kSelBlocks, kThreads, 0, s>>>(p);
 }
 
-void launch_ntuplets(const Params &p, int grid, cudaStream_t s) {
+void launch_ntuplets(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_edge_records", s);
-        k_edge_records<<<grid, kThreads, 0, s>>>(p);
+        k_edge_records<<<g.blocks(8), kThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_dfs", s);
-        k_dfs<<<grid, kThreads, 0, s>>>(p);
+        k_dfs<<<g.blocks(5), kThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_clean_max", s);
-        k_clean_max<<<grid, kThreads, 0, s>>>(p);
+        k_clean_max<<<g.blocks(8), kThreads, 0, s>>>(p);
     }
     KernelTimer t("k_clean_keep", s);
-    k_clean_keep<<<grid, kThreads, 0, s>>>(p);
+    k_clean_keep<<<g.blocks(6), kThreads, 0, s>>>(p);
 }
 
 }  // namespace ptk
