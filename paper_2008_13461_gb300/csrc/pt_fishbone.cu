@@ -24,8 +24,11 @@
 // share the work: many small warps take chunks of 32 outer hits from a queue
 // and list the outer hits with more cells, which medium (up to 320 cells)
 // and large warps (up to 512) then take one at a time; an exact pass takes
-// the rest (undecided tests, more cells) with a pairwise loop over global
-// memory beyond 512.
+// the rest (undecided tests, more cells), sorted in shared memory like the
+// others up to 1024 cells, which pT > 0.3 GeV events reach (0.2% of their
+// hits), with a pairwise loop over global memory beyond: that loop from 512
+// cells on took 2.15 of the 8.8 ms of a batch of 24 such events, against
+// 0.07 ms now.
 //
 // The same pass prepares the CA connection: it writes the live cells of o
 // ordered by a bucket of their R-z slope key relative to o (with the inner
@@ -383,30 +386,35 @@ __device__ __forceinline__ void add_alive(const Params &p, int v) {
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(p.counters + C_ALIVE_CELLS, v);
 }
 
-// Small warps: take chunks of 32 consecutive binned hits from a queue, load
+// Small warps: take chunks of consecutive binned hits from a queue, load
 // their cell counts together, work through those with 1..M cells and list
 // the ones with more: up to kFbMidMax cells from the front of the list
-// array, more from its back.
+// array, more from its back.  A warp walks its chunk's hits in turn, so a
+// chunk is 32 hits only where that leaves every resident warp several chunks:
+// with 32 whatever the size, one PU200 event (30.8 k hits) kept 962 of 4864
+// warps busy (454 -> 75 us with chunks by size; a PU50 event 158 -> 19 us, a
+// batch of 32 of them 279 -> 194 us).
 constexpr int kFbSmallMax = 192;
 constexpr int kFbMidMax = 320;
 
 template <int W, int M, int NB, int kMinBlocks>
-__global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p, float unit_thr, float du) {
+__global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p, float unit_thr, float du,
+                                                                    int chunk_log2) {
     __shared__ FbSmem<W, M, NB, true> sm;
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     int my_alive = 0;
     const int n_binned = p.bin_cnt[p.n_bins];
-    const int n_chunks = (n_binned + 31) >> 5;
+    const int n_chunks = (n_binned + (1 << chunk_log2) - 1) >> chunk_log2;
     for (;;) {
         int ch = 0;
         if (lane == 0) ch = atomicAdd(p.counters + C_FB_NEXT, 1);
         ch = __shfl_sync(0xffffffffu, ch, 0);
         if (ch >= n_chunks) break;
-        const int ol = (ch << 5) + lane;
+        const int o0 = ch << chunk_log2, ol = o0 + lane;
         int nl = 0, bl = 0;
-        if (ol < n_binned) {
+        if (lane < (1 << chunk_log2) && ol < n_binned) {
             nl = p.in_cnt[ol];
             bl = p.in_off[ol];
         }
@@ -430,10 +438,9 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
             todo &= todo - 1;
             const int n = __shfl_sync(0xffffffffu, nl, t);
             const int b = __shfl_sync(0xffffffffu, bl, t);
-            const int a = fishbone_hit<W, M, NB, false, false, true>(p, (ch << 5) + t, n, b, lane, w, unit_thr, du,
-                                                                     sm);
+            const int a = fishbone_hit<W, M, NB, false, false, true>(p, o0 + t, n, b, lane, w, unit_thr, du, sm);
             if (a >= 0) my_alive += a;
-            else list_pending(p, (ch << 5) + t, lane);
+            else list_pending(p, o0 + t, lane);
         }
     }
     add_alive(p, my_alive);
@@ -481,8 +488,11 @@ __global__ void __launch_bounds__(32 * W) k_fishbone_exact(Params p, float unit_
 
 void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, cudaStream_t s) {
     {
+        // at least four chunks for each resident warp
+        int chunk_log2 = 0;
+        while (chunk_log2 < 5 && (p.n_hits >> (chunk_log2 + 1)) >= 4 * 8 * g.blocks(4)) chunk_log2++;
         KernelTimer t("k_fishbone_small", s);
-        k_fishbone_small<8, kFbSmallMax, 256, 4><<<g.blocks(4), 256, 0, s>>>(p, unit_thr, du);
+        k_fishbone_small<8, kFbSmallMax, 256, 4><<<g.blocks(4), 256, 0, s>>>(p, unit_thr, du, chunk_log2);
     }
     {
         KernelTimer t("k_fishbone_medium", s);
@@ -493,7 +503,7 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
         k_fishbone_large<2, 512, 1024, true, true><<<g.blocks(5), 64, 0, s>>>(p, unit_thr, du);
     }
     KernelTimer t("k_fishbone_exact", s);
-    k_fishbone_exact<2, 512, 1024><<<g.blocks(5), 64, 0, s>>>(p, unit_thr, du);
+    k_fishbone_exact<1, 1024, 1024><<<g.blocks(6), 32, 0, s>>>(p, unit_thr, du);
 }
 
 }  // namespace ptk
