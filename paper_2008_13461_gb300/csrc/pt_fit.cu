@@ -499,8 +499,17 @@ __device__ void fit_track(const Params &p, int64_t k, int32_t t) {
 // of track indices (see k_select_tracks), which each kernel walks.  R: the
 // precision of the normal equations (double, or float for the all-float32
 // variant).
+//
+// Blocks of two warps: the float64 pipe of one SM is shared by a block's
+// warps, and the tracks of a small event fill only a few blocks (blocks of
+// eight warps: k_fit<5> 49 -> 31 us, k_fit<4> 43 -> 34 us, k_fit<3> 26 -> 20
+// us for the 87 k tracks of 32 PU50 events; 461 -> 455 us for 2.3 M triplets).
+// Four times the resident blocks (two for five hits): with a single wave,
+// 474 us for the 2.3 M triplets.
+constexpr int kFitThreads = 64;
+
 template <int N, typename R>
-__global__ void __launch_bounds__(kThreads) k_fit(Params p) {
+__global__ void __launch_bounds__(kFitThreads) k_fit(Params p) {
     constexpr int c = N - 3;
     int64_t k0 = 0;
 #pragma unroll
@@ -524,18 +533,18 @@ template <typename R>
 void launch_fit_r(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_fit<3>", s);
-        k_fit<3, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
+        k_fit<3, R><<<g.sms * 56, kFitThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_fit<4>", s);
-        k_fit<4, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
+        k_fit<4, R><<<g.sms * 44, kFitThreads, 0, s>>>(p);
     }
     {
         KernelTimer t("k_fit<5>", s);
-        k_fit<5, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
+        k_fit<5, R><<<g.sms * 16, kFitThreads, 0, s>>>(p);
     }
     KernelTimer t("k_fit<6..8>", s);
-    k_fit<6, R><<<g.sms * g.factor, kThreads, 0, s>>>(p);
+    k_fit<6, R><<<g.sms * 4, kFitThreads, 0, s>>>(p);
 }
 
 void launch_fit(const Params &p, const Grid &g, cudaStream_t s) {

@@ -626,8 +626,13 @@ __device__ void grad_track(const Params &p, int32_t t, const float *gp, float gc
 }
 
 // One kernel per hit count, over the track range of that count.
+// Blocks of two warps, as in the fit (4 warps: 1486 -> 1408 us for 1 M
+// triplets, whose 170 registers let an SM hold 10 warps of these, 8 of
+// those), in four waves of resident blocks (with one, 1710 us).
+constexpr int kGradThreads = 64;
+
 template <int N>
-__global__ void __launch_bounds__(128) k_fit_grad(Params p, const float *gpar, const float *gchi, float *gx, float *gy,
+__global__ void __launch_bounds__(kGradThreads) k_fit_grad(Params p, const float *gpar, const float *gchi, float *gx, float *gy,
                                                   float *gz) {
     if (upstream_overflow(p, PT_FLAG_CELLS | PT_FLAG_TUPLES | PT_FLAG_TRACKS)) return;
     constexpr int c = N - 3;
@@ -704,18 +709,18 @@ void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, floa
                      cudaStream_t s) {
     {
         KernelTimer t("k_fit_grad<3>", s);
-        k_fit_grad<3><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<3><<<g.sms * 20, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<4>", s);
-        k_fit_grad<4><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<4><<<g.sms * 16, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<5>", s);
-        k_fit_grad<5><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        k_fit_grad<5><<<g.sms * 8, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
     }
     KernelTimer t("k_fit_grad<6..8>", s);
-    k_fit_grad<6><<<g.sms * g.factor, 128, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+    k_fit_grad<6><<<g.sms * 4, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
 }
 
 void launch_align(int n, const float *x, const float *y, const float *z, const int32_t *module, const float *centre,
