@@ -145,9 +145,35 @@ __global__ void __launch_bounds__(kThreads) k_scan_apply(int32_t *a, int64_t n, 
     }
 }
 
+// the same for n <= kScanItems: one block, one kernel
+__global__ void __launch_bounds__(kThreads) k_scan_small(int32_t *a, int n) {
+    __shared__ int sw[kThreads / 32];
+    int v[kPerThread], s = 0;
+#pragma unroll
+    for (int k = 0; k < kPerThread; k++) {
+        const int i = threadIdx.x * kPerThread + k;
+        v[k] = i < n ? a[i] : 0;
+        s += v[k];
+    }
+    int total;
+    int e = block_exclusive_scan(s, sw, total);
+#pragma unroll
+    for (int k = 0; k < kPerThread; k++) {
+        const int i = threadIdx.x * kPerThread + k;
+        if (i < n) a[i] = e;
+        e += v[k];
+    }
+    if (threadIdx.x == 0) a[n] = total;
+}
+
 void launch_scan(int32_t *a, int64_t n, int32_t *part, cudaStream_t s) {
     const int nb = (int)((n + kScanItems - 1) / kScanItems);
-    if (nb > 0) {
+    if (nb <= 1) {       // (the vertex finder's events: 17 us in three kernels, 6 us in one)
+        KernelTimer t("k_scan_small", s);
+        k_scan_small<<<1, kThreads, 0, s>>>(a, (int)n);
+        return;
+    }
+    {
         KernelTimer t("k_scan_reduce", s);
         k_scan_reduce<<<nb, kThreads, 0, s>>>(a, n, part);
     }
@@ -155,10 +181,8 @@ void launch_scan(int32_t *a, int64_t n, int32_t *part, cudaStream_t s) {
         KernelTimer t("k_scan_partials", s);
         k_scan_partials<<<1, kThreads, 0, s>>>(part, nb, a + n);
     }
-    if (nb > 0) {
-        KernelTimer t("k_scan_apply", s);
-        k_scan_apply<<<nb, kThreads, 0, s>>>(a, n, part);
-    }
+    KernelTimer t("k_scan_apply", s);
+    k_scan_apply<<<nb, kThreads, 0, s>>>(a, n, part);
 }
 
 __global__ void __launch_bounds__(kThreads) k_bin_fill(Params p) {

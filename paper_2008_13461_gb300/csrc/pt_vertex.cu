@@ -25,10 +25,12 @@
 //
 // GPU form: a counting sort groups the eligible tracks by event; one block of
 // 1024 threads per event then sorts its tracks by (z0, index) in shared
-// memory (bitonic), so that every track's compatible tracks lie in a window
-// around it; densities and links come from window scans (one thread per
-// track), roots from pointer jumping, candidates from a second sort of
-// (root, position) keys.  The candidates' fits and 2-means splits, the
+// memory, so that every track's compatible tracks lie in a window around it;
+// densities and links come from window scans (two threads per track, one to
+// each side), roots from pointer jumping, candidates from a counting sort of
+// the tracks by root.  The sort by z0 is a counting sort too (by z0 tile, a
+// tile's few entries ranked by comparing them with each other); where a tile
+// is crowded a bitonic sort takes over.  The candidates' fits and 2-means splits, the
 // float64 part, then run one warp per candidate over the candidates of all
 // events at once (shuffle reductions), so that every SM takes part; a last
 // block per event orders its vertices and labels their tracks.
@@ -44,7 +46,11 @@ constexpr int kPosMask = kVtxMax - 1;
 constexpr int kSideBit = 30;                 // 2-means side of a member, kept in its key
 constexpr int kVtxCap = PT_VTX_MAX_VERTICES; // vertex candidates / vertices per event
 constexpr int kVtxThreads = 1024;
-constexpr size_t kVtxDynSmem = 3 * sizeof(int32_t) * kVtxMax;
+constexpr int kZTiles = 4096;                // z0 tiles of the counting sort, over +-kZHalf
+constexpr float kZHalf = 24.0f;              //   (beyond, the outermost tiles)
+constexpr int kVtxSplit = 10000;             // tracks per event from which the windows run over all SMs
+constexpr int kCrowd = 256;                  // entries of a tile that are still ranked pairwise
+constexpr size_t kVtxDynSmem = sizeof(int32_t) * (3 * kVtxMax + kZTiles);
 constexpr int kKmeansRounds = 20;
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -55,12 +61,16 @@ struct VtxArgs {
     pt_vertex_tracks in;
     pt_vertex_cuts cuts;
     // scratch; arrays "by sorted position" hold each event's tracks at its ev_off
-    int32_t *ev_off, *ev_cur, *order, *rho, *root;
-    double2 *wz;                     // (1 / ez0^2, z0) in float64 by sorted position
-    int32_t *key;                    // (root, position) keys, grouped by root; the members of the candidates
+    int32_t *ev_off, *ev_cur, *order, *rho, *root;   // order: key before its groups are put
+                                                     //   in order, then ~vertex of each member
+    float4 *rec;                     // (z0, ez0, track index as int bits, -), grouped by event
+    double2 *wz;                     // (1 / ez0^2, z0) in float64 by sorted position (in rec's place: each
+                                     //   event's records are used up when its first weight is written)
+    float2 *ze;                      // (z0, ez0) by sorted position
+    int32_t *key;                    // sorted positions grouped by root; the members of the candidates
     int32_t *sid;                    // track index by sorted position
     int32_t *nc, *nv;                // per event: candidates, provisional vertices
-    int32_t *cq, *cn, *cv0, *cv1;    // per event and candidate (kVtxCap each): first key, members, its vertices
+    int32_t *cq, *cn;                // per event and candidate (kVtxCap each): first key, members
     double *vz, *vsp;                // per event and provisional vertex (kVtxCap each): z, sum of pT^2
     float *vez, *vc2;                //   its error and chi2
     int32_t *vnt, *vkey;             //   its tracks and (2 * first key + part)
@@ -101,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_vtx_fill(VtxArgs a) {
         int slot = 0;
         if (ok && lane == leader) slot = atomicAdd(a.ev_cur + e, __popc(grp));
         slot = __shfl_sync(kFull, slot, leader) + __popc(grp & ((1u << lane) - 1u));
-        if (ok) a.order[a.ev_off[e] + slot] = i;
+        if (ok) a.rec[a.ev_off[e] + slot] = make_float4(a.in.z0[i], a.in.ez0[i], __int_as_float(i), 0.f);
     }
 }
 
@@ -111,93 +121,202 @@ __device__ __forceinline__ bool chi2_ok(float dz, float ep2, float eq, float c2m
     return __fmul_rn(dz, dz) < __fmul_rn(c2m, __fadd_rn(ep2, __fmul_rn(eq, eq)));
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);    // every lane ends with the same bits
-    return v;
+// Warp-wide sums (every lane ends with the same bits).  The float64 pipe
+// takes ~19 cycles for one instruction of a warp, so four sums share their
+// additions: after each of the first two exchanges a lane carries on half of
+// them, in the same pairing of lanes as a butterfly for each alone.
+__device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(kFull, v); }
+
+__device__ __forceinline__ void warp_sum4(double &a, double &b, double &c, double &d) {
+    const int lane = threadIdx.x & 31;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    // lanes with bit 16 clear keep a, b; the others c, d
+    double x = (h16 ? c : a) + __shfl_xor_sync(kFull, h16 ? a : c, 16);
+    double y = (h16 ? d : b) + __shfl_xor_sync(kFull, h16 ? b : d, 16);
+    // bit 8 clear: the first of the two; set: the second
+    double v = (h8 ? y : x) + __shfl_xor_sync(kFull, h8 ? x : y, 8);
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0);
+    b = __shfl_sync(kFull, v, 8);
+    c = __shfl_sync(kFull, v, 16);
+    d = __shfl_sync(kFull, v, 24);
 }
 
-__device__ __forceinline__ int warp_sum(int v) {
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    return v;
+__device__ __forceinline__ void warp_sum2(double &a, double &b) {
+    const bool h16 = threadIdx.x & 16;
+    double v = (h16 ? b : a) + __shfl_xor_sync(kFull, h16 ? a : b, 16);
+    for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    a = __shfl_sync(kFull, v, 0);
+    b = __shfl_sync(kFull, v, 16);
 }
 
-struct WSums {
-    double sw, swz;
+// a / b and c / d in one division's instructions
+__device__ __forceinline__ void warp_div2(double a, double b, double c, double d, double &q0, double &q1) {
+    const bool h16 = threadIdx.x & 16;
+    const double q = (h16 ? c : a) / (h16 ? d : b);
+    q0 = __shfl_sync(kFull, q, 0);
+    q1 = __shfl_sync(kFull, q, 16);
+}
+
+// The members of a candidate, lane k mod 32 holding member k: weight and z0
+// (wz: in float64 by sorted position, computed once per track) and the side
+// of a partition.  Up to 32 kMemCache of them stay in registers, so that
+// the rounds of a 2-means split wait for no loads; in a larger candidate
+// they are read again each time and the sides are kept in the keys' side
+// bits (mk).
+constexpr int kMemCache = 8;
+
+struct Sides {
+    double sw0, swz0, sw1, swz1;
+    int n1;
+};
+
+struct Members {
+    int32_t *mk;
+    const double2 *wz;
     int n;
+    bool cached;
+    double2 v[kMemCache];
+    unsigned side;
+
+    // f(member, weight and z0, side) -> side, for every member of the lane
+    template <class F>
+    __device__ __forceinline__ void each(F f) {
+        const int lane = threadIdx.x & 31;
+        if (cached) {
+#pragma unroll
+            for (int i = 0; i < kMemCache; i++) {
+                if (32 * i >= n) break;
+                if (lane + 32 * i < n) {
+                    const unsigned u = f(lane + 32 * i, v[i], (int)((side >> i) & 1));
+                    side = (side & ~(1u << i)) | u << i;
+                }
+            }
+        } else {
+            for (int k = lane; k < n; k += 32) {
+                const int32_t kk = mk[k];
+                const int u = f(k, wz[kk & kPosMask], (kk >> kSideBit) & 1);
+                mk[k] = (kk & ~(1 << kSideBit)) | (u << kSideBit);
+            }
+        }
+    }
+
+    __device__ __forceinline__ Sides sums() {
+        Sides s = {0.0, 0.0, 0.0, 0.0, 0};
+        each([&](int, const double2 &m, int u) {
+            if (u) {
+                s.sw1 += m.x;
+                s.swz1 += m.x * m.y;
+                s.n1++;
+            } else {
+                s.sw0 += m.x;
+                s.swz0 += m.x * m.y;
+            }
+            return u;
+        });
+        warp_sum4(s.sw0, s.swz0, s.sw1, s.swz1);
+        s.n1 = warp_sum(s.n1);
+        return s;
+    }
+
+    // chi2 of the members on side sel about z, and the sum of their pT^2
+    // (pt(k): member k's pT); sel < 0: every member
+    template <class Pt>
+    __device__ __forceinline__ void chi2_pt2(int sel, double z, Pt pt, double &chi2, double &pt2) {
+        double c = 0.0, p = 0.0;
+        each([&](int k, const double2 &m, int u) {
+            if (sel < 0 || u == sel) {
+                const double d = m.y - z, t = pt(k);
+                c += m.x * d * d;
+                p += t * t;
+            }
+            return u;
+        });
+        warp_sum2(c, p);
+        chi2 = c;
+        pt2 = p;
+    }
 };
 
-// Weighted sums over the members mk[0, n) of a candidate (one warp); sel < 0:
-// every member, else those whose side bit equals sel.  wz: each track's
-// weight 1/ez0^2 and z0 in float64 by sorted position, computed once per
-// track (the float64 pipe is the slow one on this GPU, and a division, or a
-// conversion to float64, costs many of its cycles).
-__device__ __forceinline__ WSums member_sums(const int32_t *mk, int n, int sel, const double2 *wz) {
-    double sw = 0.0, swz = 0.0;
-    int c = 0;
-    for (int k = threadIdx.x & 31; k < n; k += 32) {
-        const int32_t kk = mk[k];
-        if (sel >= 0 && ((kk >> kSideBit) & 1) != sel) continue;
-        const double2 v = wz[kk & kPosMask];
-        sw += v.x;
-        swz += v.x * v.y;
-        c++;
-    }
-    return WSums{warp_sum(sw), warp_sum(swz), warp_sum(c)};
+// (float)(1 / sqrt(s)): by one Newton step from a float32 seed where s is
+// well inside its range (relative error ~1e-14 before the rounding)
+__device__ __forceinline__ float error_of_weight(double s) {
+    if (!(s > 1e-30 && s < 1e30)) return (float)(1.0 / sqrt(s));
+    const double y = (double)rsqrtf((float)s);
+    return (float)(y * (1.5 - 0.5 * s * y * y));
 }
 
-__device__ __forceinline__ double member_chi2(const int32_t *mk, int n, int sel, double z, const double2 *wz) {
-    double c = 0.0;
-    for (int k = threadIdx.x & 31; k < n; k += 32) {
-        const int32_t kk = mk[k];
-        if (sel >= 0 && ((kk >> kSideBit) & 1) != sel) continue;
-        const double2 v = wz[kk & kPosMask];
-        const double d = v.y - z;
-        c += v.x * d * d;
-    }
-    return warp_sum(c);
-}
-
-__device__ __forceinline__ double member_sumpt2(const VtxArgs &a, const int32_t *mk, int n, int sel,
-                                                const int32_t *sid) {
-    // (sid: the event's track index by sorted position)
-    double s = 0.0;
-    for (int k = threadIdx.x & 31; k < n; k += 32) {
-        const int32_t kk = mk[k];
-        if (sel >= 0 && ((kk >> kSideBit) & 1) != sel) continue;
-        const double t = a.in.pt[sid[kk & kPosMask]];
-        s += t * t;
-    }
-    return warp_sum(s);
-}
-
-// sort elements: (z0, track index) in order of both, or plain int keys
-struct ZId {
+// sort element: z0 and record, in order of (z0, track index)
+struct ZRec {
     float z;
-    int id;
+    int rec;
 };
-__device__ __forceinline__ bool elem_gt(const ZId &a, const ZId &b) { return a.z > b.z || (a.z == b.z && a.id > b.id); }
-__device__ __forceinline__ bool elem_gt(int a, int b) { return a > b; }
-__device__ __forceinline__ ZId elem_shfl_xor(const ZId &e, int j) {
-    return {__shfl_xor_sync(0xffffffffu, e.z, j), __shfl_xor_sync(0xffffffffu, e.id, j)};
+__device__ __forceinline__ int track_of(const float4 *rec, int r) { return r < kVtxMax ? __float_as_int(rec[r].z) : r; }
+__device__ __forceinline__ bool elem_gt(const ZRec &a, const ZRec &b, const float4 *rec) {
+    return a.z > b.z || (a.z == b.z && track_of(rec, a.rec) > track_of(rec, b.rec));
 }
-__device__ __forceinline__ int elem_shfl_xor(int e, int j) { return __shfl_xor_sync(0xffffffffu, e, j); }
+
+// z0 tile: monotone in z0 (the track's place among equal tiles is found by
+// comparing the values)
+__device__ __forceinline__ int z_tile(float z) {
+    return min(max((int)((z + kZHalf) * (kZTiles / (2.0f * kZHalf))), 0), kZTiles - 1);
+}
+
+// Exclusive prefix sums of a[0, n) in place (the whole block), and whether
+// any entry was above kCrowd.  warp: 32 ints.
+__device__ __forceinline__ bool block_starts(int32_t *a, int n, int32_t *warp) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, per = (n + kVtxThreads - 1) / kVtxThreads;
+    const int i0 = min((int)threadIdx.x * per, n), i1 = min(i0 + per, n);
+    int sum = 0;
+    bool crowded = false;
+    for (int i = i0; i < i1; i++) {
+        sum += a[i];
+        crowded |= a[i] > kCrowd;
+    }
+    int incl = sum;
+    for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += t;
+    }
+    if (lane == 31) warp[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        const int v = warp[lane];
+        int x = v;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int t = __shfl_up_sync(kFull, x, d);
+            if (lane >= d) x += t;
+        }
+        warp[lane] = x - v;
+    }
+    __syncthreads();
+    int run = warp[w] + incl - sum;
+    for (int i = i0; i < i1; i++) {
+        const int v = a[i];
+        a[i] = run;
+        run += v;
+    }
+    return __syncthreads_or(crowded) != 0;
+}
 
 // Ascending bitonic sort of P entries (P a power of two, at least 32; the
-// block a multiple of 32 threads).  Position p is handled by thread p mod
+// block a multiple of 32 threads); padding entries have records from kVtxMax
+// on and an infinite z0.  Position p is handled by thread p mod
 // blockDim, so the partners of the stages at distance 16 or less are lanes
 // of one warp: those stages of each merge run in registers with shuffles,
 // one barrier per merge instead of one per stage.
-template <class E, class Load, class Store>
-__device__ __forceinline__ void bitonic(int P, Load load, Store store) {
+__device__ __forceinline__ void bitonic(int P, float *sz, int32_t *srec, const float4 *rec) {
     for (int k = 2; k <= P; k <<= 1) {
         for (int j = k >> 1; j >= 32; j >>= 1) {
             for (int p = threadIdx.x; p < P; p += blockDim.x) {
                 const int q = p ^ j;
                 if (q > p) {
-                    const E a = load(p), b = load(q);
-                    if (elem_gt(a, b) == ((p & k) == 0)) {
-                        store(p, b);
-                        store(q, a);
+                    const ZRec a = {sz[p], srec[p]}, b = {sz[q], srec[q]};
+                    if (elem_gt(a, b, rec) == ((p & k) == 0)) {
+                        sz[p] = b.z;
+                        srec[p] = b.rec;
+                        sz[q] = a.z;
+                        srec[q] = a.rec;
                     }
                 }
             }
@@ -205,113 +324,240 @@ __device__ __forceinline__ void bitonic(int P, Load load, Store store) {
         }
         // whole warps take part: P and blockDim are multiples of 32
         for (int p = threadIdx.x; p < P; p += blockDim.x) {
-            E e = load(p);
+            ZRec e = {sz[p], srec[p]};
             const bool up = (p & k) == 0;
             for (int j = min(k >> 1, 16); j > 0; j >>= 1) {
-                const E o = elem_shfl_xor(e, j);
+                const ZRec o = {__shfl_xor_sync(kFull, e.z, j), __shfl_xor_sync(kFull, e.rec, j)};
                 // the lower of a pair keeps the smaller entry in an ascending
                 // run and the larger in a descending one
-                if (((p & j) == 0) == up ? elem_gt(e, o) : elem_gt(o, e)) e = o;
+                if (((p & j) == 0) == up ? elem_gt(e, o, rec) : elem_gt(o, e, rec)) e = o;
             }
-            store(p, e);
+            sz[p] = e.z;
+            srec[p] = e.rec;
         }
         __syncthreads();
     }
 }
 
-// Per event: sort, densities, links, roots, candidates (one block).
+// Densities: the compatible tracks of the track at position p of an event's
+// sorted tracks [0, cnt) lie in the window |z0 - z0_p| < dz_cut (rounded
+// differences are monotonic along the sorted order); those on one side.
+template <class Z, class Ez>
+__device__ __forceinline__ int side_density(int p, int dir, int cnt, Z z, Ez ez, float dzc, float c2m) {
+    const float zp = z(p), ep = ez(p), ep2 = __fmul_rn(ep, ep);
+    int r = 0;
+    for (int q = p + dir; q >= 0 && q < cnt; q += dir) {
+        const float dz = __fsub_rn(zp, z(q));
+        if (!(fabsf(dz) < dzc)) break;
+        r += chi2_ok(dz, ep2, ez(q), c2m);
+    }
+    return r;
+}
+
+// Links: the nearest compatible track of higher rank on one side (-1: none)
+// and its distance; the sorted position orders equal densities and equal
+// distances by (z0, index).
+template <class Z, class Ez, class Rho>
+__device__ __forceinline__ int side_link(int p, int dir, int cnt, Z z, Ez ez, Rho rho, float dzc, float c2m, float &bd) {
+    const float zp = z(p), ep = ez(p), ep2 = __fmul_rn(ep, ep);
+    const int rp = rho(p);
+    int best = -1;
+    bd = __int_as_float(0x7f800000);
+    for (int q = p + dir; q >= 0 && q < cnt; q += dir) {
+        const float dz = __fsub_rn(zp, z(q)), ad = fabsf(dz);
+        // distances do not shrink along the window, so nothing nearer
+        // follows; at an equal one the smaller position wins
+        if (!(ad < dzc) || ad > bd) break;
+        const int rq = rho(q);
+        if (!(rq > rp || (rq == rp && q < p))) continue;
+        if (!chi2_ok(dz, ep2, ez(q), c2m)) continue;
+        if (best < 0 || q < best) best = q;
+        bd = ad;
+    }
+    return best;
+}
+
+// the nearer of the two sides' links of a track, whose lanes are neighbours
+__device__ __forceinline__ int join_sides(int best, float bd) {
+    const int ob = __shfl_xor_sync(kFull, best, 1);
+    const float od = __shfl_xor_sync(kFull, bd, 1);
+    return ob >= 0 && (best < 0 || od < bd || (od == bd && ob < best)) ? ob : best;
+}
+
+__device__ __forceinline__ double2 weight_and_z(float2 ze) {
+    const double e = ze.y;
+    return make_double2(1.0 / (e * e), (double)ze.x);
+}
+
+// Densities (kLinks = false; and the fits' weights) or links (true) of the
+// sorted tracks of all events, over every SM: two neighbouring lanes take a
+// track, one to each side.
+template <bool kLinks>
+__global__ void __launch_bounds__(kThreads) k_vtx_window(VtxArgs a) {
+    const int total = a.ev_off[a.n_events];
+    const float dzc = a.cuts.dz_cut, c2m = a.cuts.chi2_max;
+    const int64_t items = (2 * (int64_t)total + 31) & ~31;
+    for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items; it += (int64_t)gridDim.x * blockDim.x) {
+        const int g = (int)(it >> 1), dir = (it & 1) ? 1 : -1;
+        bool ok = g < total;
+        int base = 0, cnt = 0;
+        if (ok) {
+            int lo = 0, hi = a.n_events - 1;                 // the event of position g
+            while (lo < hi) {
+                const int m = (lo + hi + 1) >> 1;
+                if (__ldg(a.ev_off + m) <= g) lo = m;
+                else hi = m - 1;
+            }
+            base = __ldg(a.ev_off + lo);
+            cnt = __ldg(a.ev_off + lo + 1) - base;
+            ok = cnt <= kVtxMax;                             // (a larger one was not sorted)
+        }
+        const float2 *ze = a.ze + base;
+        int *rho = a.rho + base;
+        const auto z = [&](int q) { return ze[q].x; };
+        const auto ez = [&](int q) { return ze[q].y; };
+        if (!kLinks) {
+            int r = ok ? side_density(g - base, dir, cnt, z, ez, dzc, c2m) : 0;
+            r += __shfl_xor_sync(kFull, r, 1);
+            if (ok && dir > 0) rho[g - base] = 1 + r;
+            if (ok && dir < 0) a.wz[g] = weight_and_z(ze[g - base]);
+        } else {
+            float bd = 0.f;
+            int best = ok ? side_link(g - base, dir, cnt, z, ez, [&](int q) { return rho[q]; }, dzc, c2m, bd) : -1;
+            best = join_sides(best, bd);
+            if (ok && dir > 0) a.root[g] = best < 0 ? g - base : best;
+        }
+    }
+}
+
+// Per event (one block): sort, densities, links, roots, candidates
+// (kVtxAll), or only the sort (kVtxSort) or only the roots and candidates
+// (kVtxRoots), the windows in between run by k_vtx_window over every SM.
+//
+// One SM works on an event, so the length of its chain of phases counts:
+// with two bitonic sorts and one thread per track and window, 24 PU200 events
+// of 4950 eligible tracks took 381 us and one PU50 event of 449 took 31 us;
+// with the counting sorts and two lanes per track 225 and 17 us, and the
+// first 106 us with the windows over every SM.
+enum VtxPart { kVtxAll, kVtxSort, kVtxRoots };
+
+template <VtxPart kPart>
 __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
     extern __shared__ __align__(16) unsigned char vsm[];
     float *sz = reinterpret_cast<float *>(vsm);                   // z0 by sorted position
-    int32_t *sid = reinterpret_cast<int32_t *>(sz + kVtxMax);     // track index by sorted position
-    int32_t *key = sid + kVtxMax;                                 // root << kPosBits | position
+    int32_t *sid = reinterpret_cast<int32_t *>(sz + kVtxMax);     // track index by sorted position, then rho
+    int32_t *key = sid + kVtxMax;                                 // z0 errors, then roots, then keys
+    int32_t *tile = key + kVtxMax;
     __shared__ int s_nc;
+    __shared__ int32_t s_warp[32];
 
     const int e = blockIdx.x, tid = threadIdx.x;
     const int base = a.ev_off[e], cnt = a.ev_off[e + 1] - base;
-    if (tid == 0) {
+    if (kPart != kVtxSort && tid == 0) {
         a.nc[e] = 0;
         a.nv[e] = 0;
+        s_nc = 0;
     }
     if (cnt > kVtxMax) {                                          // uniform over the block
-        if (tid == 0) set_status(a, PT_VTX_EVENT_TOO_LARGE);
+        if (kPart != kVtxSort && tid == 0) set_status(a, PT_VTX_EVENT_TOO_LARGE);
         return;
     }
-    if (tid == 0) s_nc = 0;
-    int P = 32;
-    while (P < cnt) P <<= 1;
-    for (int p = tid; p < P; p += blockDim.x) {
-        if (p < cnt) {
-            const int i = a.order[base + p];
-            sz[p] = a.in.z0[i];
-            sid[p] = i;
-        } else {
-            sz[p] = __int_as_float(0x7f800000);
-            sid[p] = 0x7fffffff;
+    int32_t *gsid = a.sid + base, *root = a.root + base;
+    float2 *ze = a.ze + base;
+    if constexpr (kPart != kVtxRoots) {
+        const float4 *rec = a.rec + base;
+        for (int t = tid; t < kZTiles; t += blockDim.x) tile[t] = 0;
+        __syncthreads();
+        // four records of a thread in flight at a time
+        for (int p0 = tid; p0 < cnt; p0 += 4 * kVtxThreads) {
+            float z[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (p0 + i * kVtxThreads < cnt) z[i] = rec[p0 + i * kVtxThreads].x;
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (p0 + i * kVtxThreads < cnt) atomicAdd(&tile[z_tile(z[i])], 1);
         }
-    }
-    __syncthreads();
-    bitonic<ZId>(
-        P, [&](int p) { return ZId{sz[p], sid[p]}; },
-        [&](int p, const ZId &e) {
-            sz[p] = e.z;
-            sid[p] = e.id;
-        });
-
-    const float dzc = a.cuts.dz_cut, c2m = a.cuts.chi2_max;
-    int32_t *rho = a.rho + base, *root = a.root + base;
-    // the z0 errors by sorted position, in the key array until the keys are
-    // built, and the weights 1/ez0^2 of the vertex fits
-    float *sez = reinterpret_cast<float *>(key);
-    double2 *wz = a.wz + base;
-    for (int p = tid; p < cnt; p += blockDim.x) {
-        const float ez = a.in.ez0[sid[p]];
-        sez[p] = ez;
-        const double e = ez;
-        wz[p] = make_double2(1.0 / (e * e), (double)sz[p]);
-        a.sid[base + p] = sid[p];
-    }
-    __syncthreads();
-    // densities: the compatible tracks lie in the window |z0 - z0_p| < dz_cut
-    // (rounded differences are monotonic along the sorted order)
-    for (int p = tid; p < cnt; p += blockDim.x) {
-        const float zp = sz[p], ep = sez[p], ep2 = __fmul_rn(ep, ep);
-        int r = 1;
-        for (int q = p - 1; q >= 0; q--) {
-            const float dz = __fsub_rn(zp, sz[q]);
-            if (!(fabsf(dz) < dzc)) break;
-            r += chi2_ok(dz, ep2, sez[q], c2m);
-        }
-        for (int q = p + 1; q < cnt; q++) {
-            const float dz = __fsub_rn(zp, sz[q]);
-            if (!(fabsf(dz) < dzc)) break;
-            r += chi2_ok(dz, ep2, sez[q], c2m);
-        }
-        rho[p] = r;
-    }
-    __syncthreads();
-    // links to the nearest compatible track of higher rank; the sorted
-    // position orders equal densities and equal distances by (z0, index)
-    for (int p = tid; p < cnt; p += blockDim.x) {
-        const float zp = sz[p];
-        const int rp = rho[p];
-        const float ep = sez[p], ep2 = __fmul_rn(ep, ep);
-        int best = -1;
-        float bd = 0.f;
-        for (int dir = -1; dir <= 1; dir += 2)
-            for (int q = p + dir; q >= 0 && q < cnt; q += dir) {
-                const float dz = __fsub_rn(zp, sz[q]), ad = fabsf(dz);
-                if (!(ad < dzc)) break;
-                const int rq = rho[q];
-                if (!(rq > rp || (rq == rp && q < p))) continue;
-                if (!chi2_ok(dz, ep2, sez[q], c2m)) continue;
-                if (best < 0 || ad < bd || (ad == bd && q < best)) {
-                    best = q;
-                    bd = ad;
-                }
+        __syncthreads();
+        auto put = [&](int at, int r) {
+            const float4 v = rec[r];
+            ze[at] = make_float2(v.x, v.y);
+            gsid[at] = __float_as_int(v.z);
+        };
+        if (!block_starts(tile, kZTiles, s_warp)) {
+            // by tile, any order inside (tile[] becomes each tile's end), then
+            // every entry's place among its tile's
+            for (int p0 = tid; p0 < cnt; p0 += 4 * kVtxThreads) {
+                float z[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (p0 + i * kVtxThreads < cnt) z[i] = rec[p0 + i * kVtxThreads].x;
+#pragma unroll
+                for (int i = 0; i < 4; i++)
+                    if (p0 + i * kVtxThreads < cnt) {
+                        const int q = atomicAdd(&tile[z_tile(z[i])], 1);
+                        sz[q] = z[i];
+                        sid[q] = p0 + i * kVtxThreads;
+                    }
             }
-        root[p] = best < 0 ? p : best;
+            __syncthreads();
+            for (int p = tid; p < cnt; p += blockDim.x) {
+                const ZRec me = {sz[p], sid[p]};
+                const int t = z_tile(me.z), q0 = t > 0 ? tile[t - 1] : 0, q1 = tile[t];
+                int at = q0;
+                for (int q = q0; q < q1; q++) at += elem_gt(me, ZRec{sz[q], sid[q]}, rec);
+                put(at, me.rec);
+            }
+        } else {
+            int P = 32;
+            while (P < cnt) P <<= 1;
+            for (int p = tid; p < P; p += blockDim.x) {
+                sz[p] = p < cnt ? rec[p].x : __int_as_float(0x7f800000);
+                sid[p] = p < cnt ? p : kVtxMax + p;
+            }
+            __syncthreads();
+            bitonic(P, sz, sid, rec);
+            for (int p = tid; p < cnt; p += blockDim.x) put(p, sid[p]);
+        }
+        if constexpr (kPart == kVtxSort) return;
+        __syncthreads();
     }
+    int32_t *rho = a.rho + base;
+    if constexpr (kPart == kVtxAll) {
+        // z0, its error (in the key array until the roots are known) and the
+        // densities by sorted position
+        const float dzc = a.cuts.dz_cut, c2m = a.cuts.chi2_max;
+        float *sez = reinterpret_cast<float *>(key);
+        rho = sid;
+        for (int p = tid; p < cnt; p += blockDim.x) {
+            const float2 v = ze[p];
+            sz[p] = v.x;
+            sez[p] = v.y;
+            a.wz[base + p] = weight_and_z(v);
+        }
+        __syncthreads();
+        const auto z = [&](int q) { return sz[q]; };
+        const auto ez = [&](int q) { return sez[q]; };
+        const int items = (2 * cnt + 31) & ~31;                   // whole warps
+        for (int it = tid; it < items; it += blockDim.x) {
+            const int p = it >> 1, dir = (it & 1) ? 1 : -1;
+            int r = p < cnt ? side_density(p, dir, cnt, z, ez, dzc, c2m) : 0;
+            r += __shfl_xor_sync(kFull, r, 1);
+            if (p < cnt && dir > 0) rho[p] = 1 + r;
+        }
+        __syncthreads();
+        for (int it = tid; it < items; it += blockDim.x) {
+            const int p = it >> 1, dir = (it & 1) ? 1 : -1;
+            float bd = 0.f;
+            int best = p < cnt ? side_link(p, dir, cnt, z, ez, [&](int q) { return rho[q]; }, dzc, c2m, bd) : -1;
+            best = join_sides(best, bd);
+            if (p < cnt && dir > 0) root[p] = best < 0 ? p : best;
+        }
+        __syncthreads();
+    }
+    for (int p = tid; p < cnt; p += blockDim.x) key[p] = root[p];
+    int32_t *start = reinterpret_cast<int32_t *>(sz);             // by root: count, start, then end of its group
+    for (int p = tid; p < cnt; p += blockDim.x) start[p] = 0;
     __syncthreads();
     // roots by pointer jumping; a racing read sees an old or a new value, both
     // ancestors, so the iteration still converges (path lengths halve)
@@ -319,9 +565,9 @@ __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
     for (int it = 0; it < 2 * kPosBits + 4 && !done; it++) {
         bool ch = false;
         for (int p = tid; p < cnt; p += blockDim.x) {
-            const int r = root[p], rr = root[r];
+            const int r = key[p], rr = key[r];
             if (rr != r) {
-                root[p] = rr;
+                key[p] = rr;
                 ch = true;
             }
         }
@@ -331,128 +577,179 @@ __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
         if (tid == 0) set_status(a, PT_VTX_INTERNAL);
         return;
     }
-    // group the tracks by root: sort the (root, position) keys
-    for (int p = tid; p < P; p += blockDim.x) key[p] = p < cnt ? (root[p] << kPosBits | p) : 0x7fffffff;
+    // group the tracks by root (k_vtx_fit puts a group's members in order of
+    // position); a group whose root has rho > 1 and at least min_tracks
+    // tracks is a candidate
+    for (int p = tid; p < cnt; p += blockDim.x) {
+        const int r = key[p];
+        atomicAdd(&start[r], 1);
+        root[p] = r;
+    }
     __syncthreads();
-    bitonic<int>(
-        P, [&](int p) { return key[p]; }, [&](int p, int e) { key[p] = e; });
-    // candidates: groups whose root has rho > 1 and at least min_tracks tracks
-    for (int q = tid; q < cnt; q += blockDim.x) {
-        const int r = key[q] >> kPosBits;
-        if (q > 0 && (key[q - 1] >> kPosBits) == r) continue;
-        int n = 1;
-        while (q + n < cnt && (key[q + n] >> kPosBits) == r) n++;
-        if (rho[r] > 1 && n >= a.cuts.min_tracks) {
-            const int c = atomicAdd(&s_nc, 1);
-            if (c < kVtxCap) {
-                a.cq[e * kVtxCap + c] = q;
-                a.cn[e * kVtxCap + c] = n;
-            } else {
-                set_status(a, PT_VTX_TOO_MANY);
-            }
+    block_starts(start, cnt, s_warp);
+    for (int p = tid; p < cnt; p += blockDim.x) {
+        if (key[p] != p) continue;
+        const int q = start[p], n = (p + 1 < cnt ? start[p + 1] : cnt) - q;
+        if (rho[p] <= 1 || n < a.cuts.min_tracks) continue;
+        const int c = atomicAdd(&s_nc, 1);
+        if (c < kVtxCap) {
+            a.cq[e * kVtxCap + c] = q;
+            a.cn[e * kVtxCap + c] = n;
+        } else {
+            set_status(a, PT_VTX_TOO_MANY);
         }
     }
-    for (int q = tid; q < cnt; q += blockDim.x) a.key[base + q] = key[q];
+    __syncthreads();
+    int32_t *order = a.order + base;
+    for (int p = tid; p < cnt; p += blockDim.x) order[atomicAdd(&start[key[p]], 1)] = p;
     __syncthreads();
     if (tid == 0) a.nc[e] = min(s_nc, kVtxCap);
 }
 
-// The candidates of all events, one warp each: fit, 2-means split,
-// provisional vertices (grid: candidates / warps per block x events).
+// The candidates of all events, one warp each: members in order, fit,
+// 2-means split, provisional vertices (grid: candidates / warps per block x
+// events).  What bounds it is the float64 pipe and the longest split: with a
+// butterfly per sum, a division per centre, the members read again in every
+// round and the outputs summed anew, 24 PU200 events (194 vertices of 25
+// tracks each, up to 192) took 122 us; 66 us now.
 constexpr int kFitWarps = 8;
 
 __global__ void __launch_bounds__(32 * kFitWarps) k_vtx_fit(VtxArgs a) {
     const int e = blockIdx.y, c = blockIdx.x * kFitWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= a.nc[e]) return;                                     // uniform over the warp
-    const int base = a.ev_off[e];
-    int32_t *key = a.key + base;
+    const int base = a.ev_off[e], cnt = a.ev_off[e + 1] - base;
     const int32_t *sid = a.sid + base;
     const double2 *wz = a.wz + base;
-    {
-        const int q = a.cq[e * kVtxCap + c], n = a.cn[e * kVtxCap + c];
-        int32_t *mk = key + q;
-        const WSums all = member_sums(mk, n, -1, wz);
-        const double z = all.swz / all.sw;
-        const double chi2 = member_chi2(mk, n, -1, z, wz);
-        bool split = false;
-        if (n > 1 && chi2 / (double)(n - 1) > (double)a.cuts.split_chi2) {
-            int hi = 0;
-            for (int k = lane; k < n; k += 32) {
-                const int32_t kk = mk[k];
-                const int s = wz[kk & kPosMask].y >= z;
-                mk[k] = (kk & ~(1 << kSideBit)) | (s << kSideBit);
-                hi += s;
-            }
-            hi = warp_sum(hi);
-            __syncwarp();
-            if (hi > 0 && hi < n) {
-                WSums s0 = member_sums(mk, n, 0, wz), s1 = member_sums(mk, n, 1, wz);
-                double c0 = s0.swz / s0.sw, c1 = s1.swz / s1.sw;
-                int up = 0;
-                bool have = false;
-                for (int round = 0; round < kKmeansRounds; round++) {
-                    bool diff = false;
-                    up = 0;
-                    for (int k = lane; k < n; k += 32) {
-                        const int32_t kk = mk[k];
-                        const double zz = wz[kk & kPosMask].y;
-                        const int u = fabs(zz - c1) < fabs(zz - c0);      // ties: the lower centre
-                        diff |= u != ((kk >> kSideBit) & 1);
-                        mk[k] = (kk & ~(1 << kSideBit)) | (u << kSideBit);
-                        up += u;
-                    }
-                    up = warp_sum(up);
-                    diff = __any_sync(kFull, diff);
-                    __syncwarp();
-                    if (have && !diff) break;
-                    have = true;
-                    if (up == 0 || up == n) break;
-                    s0 = member_sums(mk, n, 0, wz);
-                    s1 = member_sums(mk, n, 1, wz);
-                    c0 = s0.swz / s0.sw;
-                    c1 = s1.swz / s1.sw;
-                }
-                split = up >= a.cuts.min_tracks && n - up >= a.cuts.min_tracks;
-            }
+    const int q = a.cq[e * kVtxCap + c], n = a.cn[e * kVtxCap + c];
+    int32_t *mk = a.key + base + q;
+    // the members in order of position: by comparing them with each other,
+    // or, where that is more work, by a pass over the event's roots
+    const int32_t *un = a.order + base + q;
+    if ((int64_t)n * n <= 2 * (int64_t)cnt) {
+        for (int k = lane; k < n; k += 32) {
+            const int p = un[k];
+            int at = 0;
+            for (int j = 0; j < n; j++) at += un[j] < p;
+            mk[at] = p;
         }
-        for (int part = 0; part < (split ? 2 : 1); part++) {
-            const int sel = split ? part : -1;
-            const WSums s = member_sums(mk, n, sel, wz);
-            const double zv = s.swz / s.sw;
-            const double c2v = member_chi2(mk, n, sel, zv, wz);
-            const double sp = member_sumpt2(a, mk, n, sel, sid);
-            int v = 0;
-            if (lane == 0) {
-                v = atomicAdd(a.nv + e, 1);
-                if (v < kVtxCap) {
-                    const int o = e * kVtxCap + v;
-                    a.vz[o] = zv;
-                    a.vez[o] = (float)(1.0 / sqrt(s.sw));
-                    a.vc2[o] = (float)c2v;
-                    a.vnt[o] = s.n;
-                    a.vsp[o] = sp;
-                    a.vkey[o] = 2 * q + part;
-                } else {
-                    set_status(a, PT_VTX_TOO_MANY);
-                }
-                if (part == 0) a.cv0[e * kVtxCap + c] = v;
-                else a.cv1[e * kVtxCap + c] = v;
-                if (!split) a.cv1[e * kVtxCap + c] = -1;
+    } else {
+        const int32_t *root = a.root + base;
+        const int r = root[un[0]];
+        int at = 0;
+        for (int p0 = lane; p0 - lane < cnt; p0 += 256) {
+            int v[8];                                             // eight loads in flight
+#pragma unroll
+            for (int i = 0; i < 8; i++) v[i] = p0 + 32 * i < cnt ? root[p0 + 32 * i] : -1;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+                const unsigned m = __ballot_sync(kFull, v[i] == r);
+                if (v[i] == r) mk[at + __popc(m & ((1u << lane) - 1u))] = p0 + 32 * i;
+                at += __popc(m);
             }
         }
     }
+    __syncwarp();
+    Members m;
+    m.mk = mk;
+    m.wz = wz;
+    m.n = n;
+    m.cached = n <= 32 * kMemCache;
+    m.side = 0;
+    if (m.cached) {
+#pragma unroll
+        for (int i = 0; i < kMemCache; i++)
+            if (lane + 32 * i < n) m.v[i] = wz[mk[lane + 32 * i]];
+    }
+    const auto pt = [&](int k) { return (double)a.in.pt[sid[mk[k] & kPosMask]]; };
+    const Sides all = m.sums();                                   // (all on side 0 yet)
+    const double z = all.swz0 / all.sw0;
+    double chi2, pt2;
+    m.chi2_pt2(-1, z, pt, chi2, pt2);
+    // chi2 / (n - 1) > split_chi2, the quotient taken only near the cut
+    const double lim = (double)a.cuts.split_chi2 * (double)(n - 1);
+    bool split = false;
+    if (n > 1 && (chi2 > lim * (1.0 + 1e-12) ||
+                  (!(chi2 < lim * (1.0 - 1e-12)) && chi2 / (double)(n - 1) > (double)a.cuts.split_chi2))) {
+        int hi = 0;
+        m.each([&](int, const double2 &v, int) {
+            const int u = v.y >= z;
+            hi += u;
+            return u;
+        });
+        hi = warp_sum(hi);
+        if (hi > 0 && hi < n) {
+            Sides s = m.sums();
+            double c0, c1;
+            warp_div2(s.swz0, s.sw0, s.swz1, s.sw1, c0, c1);
+            int up = 0;
+            bool have = false;
+            for (int round = 0; round < kKmeansRounds; round++) {
+                bool diff = false;
+                up = 0;
+                m.each([&](int, const double2 &v, int was) {
+                    const int u = fabs(v.y - c1) < fabs(v.y - c0);          // ties: the lower centre
+                    diff |= u != was;
+                    up += u;
+                    return u;
+                });
+                up = warp_sum(up);
+                diff = __any_sync(kFull, diff);
+                if (have && !diff) break;
+                have = true;
+                if (up == 0 || up == n) break;
+                s = m.sums();
+                warp_div2(s.swz0, s.sw0, s.swz1, s.sw1, c0, c1);
+            }
+            split = up >= a.cuts.min_tracks && n - up >= a.cuts.min_tracks;
+        }
+    }
+    Sides s = all;
+    double z0 = z, z1 = 0.0;
+    if (split) {
+        s = m.sums();
+        warp_div2(s.swz0, s.sw0, s.swz1, s.sw1, z0, z1);
+    }
+    int vtx[2] = {0, 0};
+    for (int part = 0; part < (split ? 2 : 1); part++) {
+        const double zv = part ? z1 : z0, sw = part ? s.sw1 : s.sw0;
+        if (split) m.chi2_pt2(part, zv, pt, chi2, pt2);
+        const float ez = error_of_weight(sw);
+        int v = 0;
+        if (lane == 0) {
+            v = atomicAdd(a.nv + e, 1);
+            if (v < kVtxCap) {
+                const int o = e * kVtxCap + v;
+                a.vz[o] = zv;
+                a.vez[o] = ez;
+                a.vc2[o] = (float)chi2;
+                a.vnt[o] = split ? (part ? s.n1 : n - s.n1) : n;
+                a.vsp[o] = pt2;
+                a.vkey[o] = 2 * q + part;
+            } else {
+                set_status(a, PT_VTX_TOO_MANY);
+            }
+        }
+        vtx[part] = __shfl_sync(kFull, v, 0);
+    }
+    // the vertex of every member, as its complement (members of no candidate
+    // keep their position there, which is not negative)
+    int32_t *mv = a.order + base + q;
+    m.each([&](int k, const double2 &, int u) {
+        mv[k] = ~(split && u ? vtx[1] : vtx[0]);
+        return u;
+    });
 }
 
 // Per event: the vertices by sum of pT^2 (then z, then the key), their
 // outputs and the vertex of every member track (one block).
-constexpr int kOrderThreads = 256;
+constexpr int kOrderThreads = 1024;
 
 __global__ void __launch_bounds__(kOrderThreads) k_vtx_order(VtxArgs a) {
     __shared__ double s_z[kVtxCap], s_sp[kVtxCap];
     __shared__ int s_vkey[kVtxCap], s_rank[kVtxCap];
-    const int e = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    const int base = a.ev_off[e];
-    const int nv = min(a.nv[e], kVtxCap), nc = a.nc[e];
+    const int e = blockIdx.x, tid = threadIdx.x;
+    const int base = a.ev_off[e], cnt = a.nv[e] > 0 ? a.ev_off[e + 1] - base : 0;     // (none if not clustered)
+    const int nv = min(a.nv[e], kVtxCap);
     const int32_t *key = a.key + base, *sid = a.sid + base;
     for (int v = tid; v < nv; v += blockDim.x) {
         s_z[v] = a.vz[e * kVtxCap + v];
@@ -461,11 +758,16 @@ __global__ void __launch_bounds__(kOrderThreads) k_vtx_order(VtxArgs a) {
     }
     __syncthreads();
     for (int v = tid; v < nv; v += blockDim.x) {
+        // sums of pT^2 are not negative, so their bits order like them: the
+        // float64 pipe stays out of this loop over all vertices
         const double sv = s_sp[v], zv = s_z[v];
+        const long long bv = __double_as_longlong(sv);
         const int kv = s_vkey[v];
         int r = 0;
-        for (int u = 0; u < nv; u++)
-            r += s_sp[u] > sv || (s_sp[u] == sv && (s_z[u] < zv || (s_z[u] == zv && s_vkey[u] < kv)));
+        for (int u = 0; u < nv; u++) {
+            const long long bu = __double_as_longlong(s_sp[u]);
+            r += bu > bv || (bu == bv && (s_z[u] < zv || (s_z[u] == zv && s_vkey[u] < kv)));
+        }
         s_rank[v] = r;
         if (r < a.max_vertices) {
             const int64_t o = (int64_t)e * a.max_vertices + r;
@@ -482,14 +784,11 @@ __global__ void __launch_bounds__(kOrderThreads) k_vtx_order(VtxArgs a) {
         if (nv > a.max_vertices) set_status(a, PT_VTX_TOO_MANY);
     }
     __syncthreads();
-    for (int c = wid; c < nc; c += nw) {
-        const int q = a.cq[e * kVtxCap + c], n = a.cn[e * kVtxCap + c];
-        const int v0 = a.cv0[e * kVtxCap + c], v1 = a.cv1[e * kVtxCap + c];
-        for (int k = lane; k < n; k += 32) {
-            const int32_t kk = key[q + k];
-            const int v = (v1 >= 0 && ((kk >> kSideBit) & 1)) ? v1 : v0;
-            if (v < nv && s_rank[v] < a.max_vertices) a.out.track_vertex[sid[kk & kPosMask]] = s_rank[v];
-        }
+    const int32_t *mv = a.order + base;
+    for (int j = tid; j < cnt; j += blockDim.x) {
+        const int v = ~mv[j];
+        if (v >= 0 && v < nv && s_rank[v] < a.max_vertices)
+            a.out.track_vertex[sid[key[j] & kPosMask]] = s_rank[v];
     }
 }
 
@@ -519,7 +818,7 @@ __global__ void __launch_bounds__(kThreads) k_track_summary(int32_t n_tracks, co
 
 // Scratch layout (byte offsets, each array 16-byte aligned).
 struct VtxLayout {
-    size_t ev_off, ev_cur, part, order, rho, root, wz, key, sid, nc, nv, cq, cn, cv0, cv1, vz, vsp, vez, vc2, vnt,
+    size_t ev_off, ev_cur, part, order, rho, root, wz, ze, key, sid, nc, nv, cq, cn, vz, vsp, vez, vc2, vnt,
         vkey, total;
 };
 
@@ -539,14 +838,13 @@ VtxLayout vertex_layout(int32_t n_tracks, int32_t n_events) {
     L.rho = take(4 * nt);
     L.root = take(4 * nt);
     L.wz = take(16 * nt);
+    L.ze = take(8 * nt);
     L.key = take(4 * nt);
     L.sid = take(4 * nt);
     L.nc = take(4 * ne);
     L.nv = take(4 * ne);
     L.cq = take(4 * ncap);
     L.cn = take(4 * ncap);
-    L.cv0 = take(4 * ncap);
-    L.cv1 = take(4 * ncap);
     L.vz = take(8 * ncap);
     L.vsp = take(8 * ncap);
     L.vez = take(4 * ncap);
@@ -577,14 +875,14 @@ pt_status launch_vertices(const pt_vertex_tracks &in, int32_t n_tracks, int32_t 
     a.rho = (int32_t *)(w + L.rho);
     a.root = (int32_t *)(w + L.root);
     a.wz = (double2 *)(w + L.wz);
+    a.rec = (float4 *)(w + L.wz);
+    a.ze = (float2 *)(w + L.ze);
     a.key = (int32_t *)(w + L.key);
     a.sid = (int32_t *)(w + L.sid);
     a.nc = (int32_t *)(w + L.nc);
     a.nv = (int32_t *)(w + L.nv);
     a.cq = (int32_t *)(w + L.cq);
     a.cn = (int32_t *)(w + L.cn);
-    a.cv0 = (int32_t *)(w + L.cv0);
-    a.cv1 = (int32_t *)(w + L.cv1);
     a.vz = (double *)(w + L.vz);
     a.vsp = (double *)(w + L.vsp);
     a.vez = (float *)(w + L.vez);
@@ -592,12 +890,21 @@ pt_status launch_vertices(const pt_vertex_tracks &in, int32_t n_tracks, int32_t 
     a.vnt = (int32_t *)(w + L.vnt);
     a.vkey = (int32_t *)(w + L.vkey);
     a.out = out;
+    // Windows in kernels of their own where the events are large: for track
+    // summaries of which a third are eligible, one block against four kernels
+    // measured 35 / 49 us at 3400 tracks per event, 50 / 57 us at 5100 and
+    // 67 / 62 us at 6800; for fitted PU200 events (48,600 tracks, a tenth
+    // eligible) 225 / 106 us.  The line lies between, where either costs the
+    // other at most ~15 us.
+    const bool split = n_tracks / n_events > kVtxSplit;
     // per device and call (cheap; no shared state between threads or devices)
-    if (cudaFuncSetAttribute(k_vtx_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVtxDynSmem) !=
-        cudaSuccess)
+    auto big_smem = [](void (*k)(VtxArgs)) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVtxDynSmem) == cudaSuccess;
+    };
+    if (!(split ? big_smem(k_vtx_group<kVtxSort>) && big_smem(k_vtx_group<kVtxRoots>) : big_smem(k_vtx_group<kVtxAll>)))
         return PT_ERR_CUDA;
-    if (cudaMemsetAsync(a.ev_off, 0, sizeof(int32_t) * ((size_t)n_events + 1), s) != cudaSuccess ||
-        cudaMemsetAsync(a.ev_cur, 0, sizeof(int32_t) * ((size_t)n_events + 1), s) != cudaSuccess ||
+    // (ev_off and ev_cur are neighbours in the scratch)
+    if (cudaMemsetAsync(a.ev_off, 0, L.part - L.ev_off, s) != cudaSuccess ||
         cudaMemsetAsync(out.status, 0, sizeof(int32_t), s) != cudaSuccess)
         return PT_ERR_CUDA;
     {
@@ -609,9 +916,24 @@ pt_status launch_vertices(const pt_vertex_tracks &in, int32_t n_tracks, int32_t 
         KernelTimer t("k_vtx_fill", s);
         k_vtx_fill<<<grid, kThreads, 0, s>>>(a);
     }
-    {
+    if (split) {
+        {
+            KernelTimer t("k_vtx_sort", s);
+            k_vtx_group<kVtxSort><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+        }
+        {
+            KernelTimer t("k_vtx_density", s);
+            k_vtx_window<false><<<2 * grid, kThreads, 0, s>>>(a);
+        }
+        {
+            KernelTimer t("k_vtx_link", s);
+            k_vtx_window<true><<<2 * grid, kThreads, 0, s>>>(a);
+        }
+        KernelTimer t("k_vtx_roots", s);
+        k_vtx_group<kVtxRoots><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+    } else {
         KernelTimer t("k_vtx_group", s);
-        k_vtx_group<<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+        k_vtx_group<kVtxAll><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
     }
     {
         KernelTimer t("k_vtx_fit", s);
