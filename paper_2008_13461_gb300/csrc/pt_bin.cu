@@ -19,6 +19,7 @@ __device__ __forceinline__ bool on_grid(float v) {
 // (warp-aggregated: __match_any_sync groups them, the lowest lane adds the
 // group's size and shares the old count).
 __global__ void __launch_bounds__(kThreads) k_bin_count(Params p) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const int stride = gridDim.x * blockDim.x;
     for (int h0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); h0 < p.n_hits; h0 += stride) {
@@ -97,6 +98,7 @@ constexpr int kPerThread = kScanItems / kThreads;   // 16
 // Exclusive scan of a[0 .. n) in place, a[n] = total, in three kernels:
 // per-block sums, a one-block scan of those, per-block scans plus offset.
 __global__ void __launch_bounds__(kThreads) k_scan_reduce(const int32_t *a, int64_t n, int32_t *part) {
+    pdl_enter();
     __shared__ int sw[kThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPerThread;
     int s = 0;
@@ -111,6 +113,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_reduce(const int32_t *a, int6
 }
 
 __global__ void __launch_bounds__(kThreads) k_scan_partials(int32_t *part, int nblocks, int32_t *total_out) {
+    pdl_enter();
     __shared__ int sw[kThreads / 32];
     int carry = 0;
     for (int b0 = 0; b0 < nblocks; b0 += kThreads) {
@@ -125,6 +128,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_partials(int32_t *part, int n
 }
 
 __global__ void __launch_bounds__(kThreads) k_scan_apply(int32_t *a, int64_t n, const int32_t *part) {
+    pdl_enter();
     __shared__ int sw[kThreads / 32];
     int64_t base = (int64_t)blockIdx.x * kScanItems + (int64_t)threadIdx.x * kPerThread;
     int v[kPerThread];
@@ -147,6 +151,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_apply(int32_t *a, int64_t n, 
 
 // the same for n <= kScanItems: one block, one kernel
 __global__ void __launch_bounds__(kThreads) k_scan_small(int32_t *a, int n) {
+    pdl_enter();
     __shared__ int sw[kThreads / 32];
     int v[kPerThread], s = 0;
 #pragma unroll
@@ -170,22 +175,23 @@ void launch_scan(int32_t *a, int64_t n, int32_t *part, cudaStream_t s) {
     const int nb = (int)((n + kScanItems - 1) / kScanItems);
     if (nb <= 1) {       // (the vertex finder's events: 17 us in three kernels, 6 us in one)
         KernelTimer t("k_scan_small", s);
-        k_scan_small<<<1, kThreads, 0, s>>>(a, (int)n);
+        launch_pdl(k_scan_small, 1, kThreads, 0, s, a, (int)n);
         return;
     }
     {
         KernelTimer t("k_scan_reduce", s);
-        k_scan_reduce<<<nb, kThreads, 0, s>>>(a, n, part);
+        launch_pdl(k_scan_reduce, nb, kThreads, 0, s, a, n, part);
     }
     {
         KernelTimer t("k_scan_partials", s);
-        k_scan_partials<<<1, kThreads, 0, s>>>(part, nb, a + n);
+        launch_pdl(k_scan_partials, 1, kThreads, 0, s, part, nb, a + n);
     }
     KernelTimer t("k_scan_apply", s);
-    k_scan_apply<<<nb, kThreads, 0, s>>>(a, n, part);
+    launch_pdl(k_scan_apply, nb, kThreads, 0, s, a, n, part);
 }
 
 __global__ void __launch_bounds__(kThreads) k_bin_fill(Params p) {
+    pdl_enter();
     const int stride = gridDim.x * blockDim.x;
     const int per_event = PT_N_LAYERS * p.n_phi * p.n_t;
     for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < p.n_hits; h += stride) {
@@ -202,11 +208,11 @@ __global__ void __launch_bounds__(kThreads) k_bin_fill(Params p) {
 void launch_binning(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_bin_count", s);
-        k_bin_count<<<g.blocks(8), kThreads, 0, s>>>(p);
+        launch_pdl(k_bin_count, g.blocks(8), kThreads, 0, s, p);
     }
     launch_scan(p.bin_cnt, p.n_bins, p.scan_part, s);
     KernelTimer t("k_bin_fill", s);
-    k_bin_fill<<<g.blocks(8), kThreads, 0, s>>>(p);
+    launch_pdl(k_bin_fill, g.blocks(8), kThreads, 0, s, p);
 }
 
 }  // namespace ptk

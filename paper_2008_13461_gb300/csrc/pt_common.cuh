@@ -120,6 +120,11 @@ struct Params {
 };
 
 // ---------------------------------------------------------------- utilities
+// First statement of every kernel (launch_pdl): waits until the kernel
+// before it on the stream has finished and its writes are visible.  No kernel
+// may end without it: the next one waits only for its direct predecessor.
+__device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void set_flag(int32_t *counters, uint32_t f) {
     atomicOr(reinterpret_cast<unsigned int *>(counters + C_FLAGS), f);
 }

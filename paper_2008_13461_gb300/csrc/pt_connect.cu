@@ -161,6 +161,7 @@ __device__ __forceinline__ int scan_cell(const Params &p, int x, Emit &&emit) {
 }
 
 __global__ void __launch_bounds__(32 * kCaWarps, 10) k_connect(Params p) {
+    pdl_enter();
     constexpr int kPer = 32 * kCaChunk;
     __shared__ int32_t s_q[kCaWarps][kCaQueue][kPer];   // accepted inner cells per chunk position
     __shared__ int32_t s_m[kCaWarps][kPer];             // edges per chunk position (-1: no live cell,
@@ -275,6 +276,7 @@ __global__ void __launch_bounds__(32 * kCaWarps, 10) k_connect(Params p) {
 // The cells with an undecided candidate (a few hundred), one thread each,
 // with the exact predicates; each reserves its own edges.
 __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
+    pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int n = (int)min((int64_t)p.counters[C_CA_PENDING], p.cap_cells);
     const int32_t *list = reinterpret_cast<const int32_t *>(p.ck);
@@ -300,10 +302,10 @@ __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
 void launch_connect(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_connect", s);
-        k_connect<<<g.blocks(10), 32 * kCaWarps, 0, s>>>(p);
+        launch_pdl(k_connect, g.blocks(10), 32 * kCaWarps, 0, s, p);
     }
     KernelTimer t("k_connect_exact", s);
-    k_connect_exact<<<g.blocks(4), 128, 0, s>>>(p);
+    launch_pdl(k_connect_exact, g.blocks(4), 128, 0, s, p);
 }
 
 }  // namespace ptk

@@ -228,6 +228,7 @@ __device__ __forceinline__ bool doublets_hit(const Params &p, int o, int lane, u
 // layer pair (the exact pass repeats a few of them and does not count).
 template <int G>
 __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
+    pdl_enter();
     constexpr int kGroups = kThreads / G;
     constexpr int kBuf = 32 * G;   // 40 KB of shared memory per block for every G
     __shared__ int32_t s_inner[kGroups][kBuf];
@@ -264,6 +265,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
 // the hits dealt round the blocks first, so that they spread over the SMs
 // and no warp runs two hits' exact fallbacks one after the other.
 __global__ void __launch_bounds__(kThreads) k_doublets_exact(Params p) {
+    pdl_enter();
     constexpr int G = 32, kGroups = kThreads / G, kBuf = 32 * G;
     __shared__ int32_t s_inner[kGroups][kBuf];
     __shared__ uint8_t s_pair[kGroups][kBuf];
@@ -279,14 +281,14 @@ void launch_doublets(const Params &p, int lanes, const Grid &g, cudaStream_t s) 
         KernelTimer t("k_doublets", s);
         const int grid = g.blocks(5);
         switch (lanes) {
-        case 4: k_doublets<4><<<grid, kThreads, 0, s>>>(p); break;
-        case 8: k_doublets<8><<<grid, kThreads, 0, s>>>(p); break;
-        case 16: k_doublets<16><<<grid, kThreads, 0, s>>>(p); break;
-        default: k_doublets<32><<<grid, kThreads, 0, s>>>(p); break;
+        case 4: launch_pdl(k_doublets<4>, grid, kThreads, 0, s, p); break;
+        case 8: launch_pdl(k_doublets<8>, grid, kThreads, 0, s, p); break;
+        case 16: launch_pdl(k_doublets<16>, grid, kThreads, 0, s, p); break;
+        default: launch_pdl(k_doublets<32>, grid, kThreads, 0, s, p); break;
         }
     }
     KernelTimer t("k_doublets_exact", s);
-    k_doublets_exact<<<g.blocks(2), kThreads, 0, s>>>(p);
+    launch_pdl(k_doublets_exact, g.blocks(2), kThreads, 0, s, p);
 }
 
 }  // namespace ptk

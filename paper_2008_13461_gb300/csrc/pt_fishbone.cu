@@ -400,6 +400,7 @@ constexpr int kFbMidMax = 320;
 template <int W, int M, int NB, int kMinBlocks>
 __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p, float unit_thr, float du,
                                                                     int chunk_log2) {
+    pdl_enter();
     __shared__ FbSmem<W, M, NB, true> sm;
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -450,6 +451,7 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
 // the list at the back of the array).
 template <int W, int M, int NB, bool kFromBack, bool C>
 __global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_thr, float du) {
+    pdl_enter();
     __shared__ FbSmem<W, M, NB, C> sm;
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -474,6 +476,7 @@ __global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_
 // predicate and the pairwise loop for any number of cells.
 template <int W, int M, int NB>
 __global__ void __launch_bounds__(32 * W) k_fishbone_exact(Params p, float unit_thr, float du) {
+    pdl_enter();
     __shared__ FbSmem<W, M, NB, true> sm;
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -492,18 +495,18 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
         int chunk_log2 = 0;
         while (chunk_log2 < 5 && (p.n_hits >> (chunk_log2 + 1)) >= 4 * 8 * g.blocks(4)) chunk_log2++;
         KernelTimer t("k_fishbone_small", s);
-        k_fishbone_small<8, kFbSmallMax, 256, 4><<<g.blocks(4), 256, 0, s>>>(p, unit_thr, du, chunk_log2);
+        launch_pdl(k_fishbone_small<8, kFbSmallMax, 256, 4>, g.blocks(4), 256, 0, s, p, unit_thr, du, chunk_log2);
     }
     {
         KernelTimer t("k_fishbone_medium", s);
-        k_fishbone_large<4, kFbMidMax, 512, false, false><<<g.blocks(6), 128, 0, s>>>(p, unit_thr, du);
+        launch_pdl(k_fishbone_large<4, kFbMidMax, 512, false, false>, g.blocks(6), 128, 0, s, p, unit_thr, du);
     }
     {
         KernelTimer t("k_fishbone_large", s);
-        k_fishbone_large<2, 512, 1024, true, true><<<g.blocks(5), 64, 0, s>>>(p, unit_thr, du);
+        launch_pdl(k_fishbone_large<2, 512, 1024, true, true>, g.blocks(5), 64, 0, s, p, unit_thr, du);
     }
     KernelTimer t("k_fishbone_exact", s);
-    k_fishbone_exact<1, 1024, 1024><<<g.blocks(6), 32, 0, s>>>(p, unit_thr, du);
+    launch_pdl(k_fishbone_exact<1, 1024, 1024>, g.blocks(6), 32, 0, s, p, unit_thr, du);
 }
 
 }  // namespace ptk

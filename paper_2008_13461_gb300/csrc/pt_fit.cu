@@ -510,6 +510,7 @@ constexpr int kFitThreads = 64;
 
 template <int N, typename R>
 __global__ void __launch_bounds__(kFitThreads) k_fit(Params p) {
+    pdl_enter();
     constexpr int c = N - 3;
     int64_t k0 = 0;
 #pragma unroll
@@ -533,18 +534,18 @@ template <typename R>
 void launch_fit_r(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_fit<3>", s);
-        k_fit<3, R><<<g.sms * 56, kFitThreads, 0, s>>>(p);
+        launch_pdl(k_fit<3, R>, g.sms * 56, kFitThreads, 0, s, p);
     }
     {
         KernelTimer t("k_fit<4>", s);
-        k_fit<4, R><<<g.sms * 44, kFitThreads, 0, s>>>(p);
+        launch_pdl(k_fit<4, R>, g.sms * 44, kFitThreads, 0, s, p);
     }
     {
         KernelTimer t("k_fit<5>", s);
-        k_fit<5, R><<<g.sms * 16, kFitThreads, 0, s>>>(p);
+        launch_pdl(k_fit<5, R>, g.sms * 16, kFitThreads, 0, s, p);
     }
     KernelTimer t("k_fit<6..8>", s);
-    k_fit<6, R><<<g.sms * 4, kFitThreads, 0, s>>>(p);
+    launch_pdl(k_fit<6, R>, g.sms * 4, kFitThreads, 0, s, p);
 }
 
 void launch_fit(const Params &p, const Grid &g, cudaStream_t s) {

@@ -634,6 +634,7 @@ constexpr int kGradThreads = 64;
 template <int N>
 __global__ void __launch_bounds__(kGradThreads) k_fit_grad(Params p, const float *gpar, const float *gchi, float *gx, float *gy,
                                                   float *gz) {
+    pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS | PT_FLAG_TUPLES | PT_FLAG_TRACKS)) return;
     constexpr int c = N - 3;
     int64_t k0 = 0;
@@ -661,6 +662,7 @@ __global__ void __launch_bounds__(kGradThreads) k_fit_grad(Params p, const float
 __global__ void __launch_bounds__(kThreads) k_align(int n, const float *x, const float *y, const float *z,
                                                     const int32_t *module, const float *centre, const float *shift,
                                                     const float *rot, float *xo, float *yo, float *zo) {
+    pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int mm = module[i];
         const float rx = x[i] - centre[3 * mm], ry = y[i] - centre[3 * mm + 1], rz = z[i] - centre[3 * mm + 2];
@@ -679,6 +681,7 @@ __global__ void __launch_bounds__(kThreads) k_align_grad(int n, const float *x, 
                                                          const float *gxa, const float *gya, const float *gza,
                                                          float *gx, float *gy, float *gz, float *gshift,
                                                          float *grot) {
+    pdl_enter();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int mm = module[i];
         const float ax = gxa[i], ay = gya[i], az = gza[i];
@@ -709,31 +712,31 @@ void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, floa
                      cudaStream_t s) {
     {
         KernelTimer t("k_fit_grad<3>", s);
-        k_fit_grad<3><<<g.sms * 20, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<3>, g.sms * 20, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<4>", s);
-        k_fit_grad<4><<<g.sms * 16, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<4>, g.sms * 16, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<5>", s);
-        k_fit_grad<5><<<g.sms * 8, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<5>, g.sms * 8, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     KernelTimer t("k_fit_grad<6..8>", s);
-    k_fit_grad<6><<<g.sms * 4, kGradThreads, 0, s>>>(p, gpar, gchi, gx, gy, gz);
+    launch_pdl(k_fit_grad<6>, g.sms * 4, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
 }
 
 void launch_align(int n, const float *x, const float *y, const float *z, const int32_t *module, const float *centre,
                   const float *shift, const float *rot, float *xo, float *yo, float *zo, int grid, cudaStream_t s) {
     KernelTimer t("k_align", s);
-    k_align<<<grid, kThreads, 0, s>>>(n, x, y, z, module, centre, shift, rot, xo, yo, zo);
+    launch_pdl(k_align, grid, kThreads, 0, s, n, x, y, z, module, centre, shift, rot, xo, yo, zo);
 }
 
 void launch_align_grad(int n, const float *x, const float *y, const float *z, const int32_t *module,
                        const float *centre, const float *rot, const float *gxa, const float *gya, const float *gza,
                        float *gx, float *gy, float *gz, float *gshift, float *grot, int grid, cudaStream_t s) {
     KernelTimer t("k_align_grad", s);
-    k_align_grad<<<grid, kThreads, 0, s>>>(n, x, y, z, module, centre, rot, gxa, gya, gza, gx, gy, gz, gshift, grot);
+    launch_pdl(k_align_grad, grid, kThreads, 0, s, n, x, y, z, module, centre, rot, gxa, gya, gza, gx, gy, gz, gshift, grot);
 }
 
 }  // namespace ptk

@@ -21,6 +21,7 @@ __device__ __forceinline__ bool root_layer(int L) { return L == 0 || L == 1 || L
 // each step back along a path is one dependent load: the source, its own
 // incoming-edge range, and its inner hit (input index) with the root flag.
 __global__ void __launch_bounds__(kThreads) k_edge_records(Params p) {
+    pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int64_t ne = min((int64_t)p.counters[C_EDGES], p.cap_edges);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (int64_t)gridDim.x * blockDim.x) {
@@ -92,6 +93,7 @@ __device__ __forceinline__ void dfs_level(const Params &p, DfsPath &pa, int firs
 // neighbour) starts the search: the leaf and the edge's source are the
 // path's first two cells, searched back from there.
 __global__ void __launch_bounds__(kThreads) k_dfs(Params p) {
+    pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int64_t ne = min((int64_t)p.counters[C_EDGES], p.cap_edges);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(kThreads) k_dfs(Params p) {
 
 // L(c) = longest n-tuplet containing cell c
 __global__ void __launch_bounds__(kThreads) k_clean_max(Params p) {
+    pdl_enter();
     const int64_t nt = min((int64_t)p.counters[C_TUPLES], p.cap_tuples);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) {
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(kThreads) k_clean_max(Params p) {
 
 // keep an n-tuplet unless one of its cells belongs to a longer one
 __global__ void __launch_bounds__(kThreads) k_clean_keep(Params p) {
+    pdl_enter();
     const int64_t nt = min((int64_t)p.counters[C_TUPLES], p.cap_tuples);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int kept = 0;
@@ -153,6 +157,7 @@ __device__ __forceinline__ int track_class_of(const Params &p, int64_t t) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_count_tracks(Params p) {
+    pdl_enter();
     __shared__ int s_cnt[4];
     if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -171,6 +176,7 @@ __global__ void __launch_bounds__(kThreads) k_count_tracks(Params p) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_select_tracks(Params p) {
+    pdl_enter();
     __shared__ int s_base[4];
     __shared__ int s_wcnt[kThreads / 32][4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -241,27 +247,27 @@ __global__ void __launch_bounds__(kThreads) k_select_tracks(Params p) {
 void launch_select(const Params &p, cudaStream_t s) {
     {
         KernelTimer t("k_count_tracks", s);
-        k_count_tracks<<<kSelBlocks, kThreads, 0, s>>>(p);
+        launch_pdl(k_count_tracks, kSelBlocks, kThreads, 0, s, p);
     }
     KernelTimer t("k_select_tracks", s);
-    k_select_tracks<<<kSelBlocks, kThreads, 0, s>>>(p);
+    launch_pdl(k_select_tracks, kSelBlocks, kThreads, 0, s, p);
 }
 
 void launch_ntuplets(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_edge_records", s);
-        k_edge_records<<<g.blocks(8), kThreads, 0, s>>>(p);
+        launch_pdl(k_edge_records, g.blocks(8), kThreads, 0, s, p);
     }
     {
         KernelTimer t("k_dfs", s);
-        k_dfs<<<g.blocks(5), kThreads, 0, s>>>(p);
+        launch_pdl(k_dfs, g.blocks(5), kThreads, 0, s, p);
     }
     {
         KernelTimer t("k_clean_max", s);
-        k_clean_max<<<g.blocks(8), kThreads, 0, s>>>(p);
+        launch_pdl(k_clean_max, g.blocks(8), kThreads, 0, s, p);
     }
     KernelTimer t("k_clean_keep", s);
-    k_clean_keep<<<g.blocks(6), kThreads, 0, s>>>(p);
+    launch_pdl(k_clean_keep, g.blocks(6), kThreads, 0, s, p);
 }
 
 }  // namespace ptk

@@ -27,6 +27,7 @@ struct AmbArgs {
 };
 
 __global__ void __launch_bounds__(kThreads) k_amb_cells(AmbArgs a) {
+    pdl_enter();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_tracks; k += gridDim.x * blockDim.x) {
         const int t = a.track_tuple[k];
         const int n = a.n[t];
@@ -39,6 +40,7 @@ __global__ void __launch_bounds__(kThreads) k_amb_cells(AmbArgs a) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_amb_hits(AmbArgs a) {
+    pdl_enter();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_tracks; k += gridDim.x * blockDim.x) {
         const int t = a.track_tuple[k];
         const int n = a.n[t];
@@ -60,6 +62,7 @@ __global__ void __launch_bounds__(kThreads) k_amb_hits(AmbArgs a) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_amb_final(AmbArgs a) {
+    pdl_enter();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_tracks; k += gridDim.x * blockDim.x) {
         const int t = a.track_tuple[k];
         if (!a.keep[k] || a.n[t] != 3) continue;
@@ -82,14 +85,14 @@ void launch_ambiguities(const int32_t *hits, const int32_t *cells, const uint8_t
               scratch, scratch + n_cells, keep};
     {
         KernelTimer t("k_amb_cells", s);
-        k_amb_cells<<<grid, kThreads, 0, s>>>(a);
+        launch_pdl(k_amb_cells, grid, kThreads, 0, s, a);
     }
     {
         KernelTimer t("k_amb_hits", s);
-        k_amb_hits<<<grid, kThreads, 0, s>>>(a);
+        launch_pdl(k_amb_hits, grid, kThreads, 0, s, a);
     }
     KernelTimer t("k_amb_final", s);
-    k_amb_final<<<grid, kThreads, 0, s>>>(a);
+    launch_pdl(k_amb_final, grid, kThreads, 0, s, a);
 }
 
 }  // namespace ptk

@@ -89,6 +89,7 @@ __device__ __forceinline__ void set_status(const VtxArgs &a, int bit) { atomicOr
 // Tracks of one event are mostly consecutive, so the per-event atomics are
 // aggregated over the lanes of a warp that share an event.
 __global__ void __launch_bounds__(kThreads) k_vtx_count(VtxArgs a) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < a.n_tracks; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + lane;
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_vtx_count(VtxArgs a) {
 }
 
 __global__ void __launch_bounds__(kThreads) k_vtx_fill(VtxArgs a) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < a.n_tracks; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + lane;
@@ -394,6 +396,7 @@ __device__ __forceinline__ double2 weight_and_z(float2 ze) {
 // track, one to each side.
 template <bool kLinks>
 __global__ void __launch_bounds__(kThreads) k_vtx_window(VtxArgs a) {
+    pdl_enter();
     const int total = a.ev_off[a.n_events];
     const float dzc = a.cuts.dz_cut, c2m = a.cuts.chi2_max;
     const int64_t items = (2 * (int64_t)total + 31) & ~31;
@@ -443,6 +446,7 @@ enum VtxPart { kVtxAll, kVtxSort, kVtxRoots };
 
 template <VtxPart kPart>
 __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char vsm[];
     float *sz = reinterpret_cast<float *>(vsm);                   // z0 by sorted position
     int32_t *sid = reinterpret_cast<int32_t *>(sz + kVtxMax);     // track index by sorted position, then rho
@@ -615,6 +619,7 @@ __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
 constexpr int kFitWarps = 8;
 
 __global__ void __launch_bounds__(32 * kFitWarps) k_vtx_fit(VtxArgs a) {
+    pdl_enter();
     const int e = blockIdx.y, c = blockIdx.x * kFitWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= a.nc[e]) return;                                     // uniform over the warp
     const int base = a.ev_off[e], cnt = a.ev_off[e + 1] - base;
@@ -745,6 +750,7 @@ __global__ void __launch_bounds__(32 * kFitWarps) k_vtx_fit(VtxArgs a) {
 constexpr int kOrderThreads = 1024;
 
 __global__ void __launch_bounds__(kOrderThreads) k_vtx_order(VtxArgs a) {
+    pdl_enter();
     __shared__ double s_z[kVtxCap], s_sp[kVtxCap];
     __shared__ int s_vkey[kVtxCap], s_rank[kVtxCap];
     const int e = blockIdx.x, tid = threadIdx.x;
@@ -797,6 +803,7 @@ __global__ void __launch_bounds__(kThreads) k_track_summary(int32_t n_tracks, co
                                                             const int32_t *tuple, const int32_t *ev_off,
                                                             int32_t n_events, float pt_of_kappa, int32_t *ev,
                                                             float *z0, float *ez0, float *pt, uint8_t *nh) {
+    pdl_enter();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_tracks; k += gridDim.x * blockDim.x) {
         const int t = tuple[k];
         const int h = hits[(int64_t)t * PT_NMAX];
@@ -909,38 +916,38 @@ pt_status launch_vertices(const pt_vertex_tracks &in, int32_t n_tracks, int32_t 
         return PT_ERR_CUDA;
     {
         KernelTimer t("k_vtx_count", s);
-        k_vtx_count<<<grid, kThreads, 0, s>>>(a);
+        launch_pdl(k_vtx_count, grid, kThreads, 0, s, a);
     }
     launch_scan(a.ev_off, n_events, part, s);
     {
         KernelTimer t("k_vtx_fill", s);
-        k_vtx_fill<<<grid, kThreads, 0, s>>>(a);
+        launch_pdl(k_vtx_fill, grid, kThreads, 0, s, a);
     }
     if (split) {
         {
             KernelTimer t("k_vtx_sort", s);
-            k_vtx_group<kVtxSort><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+            launch_pdl(k_vtx_group<kVtxSort>, n_events, kVtxThreads, kVtxDynSmem, s, a);
         }
         {
             KernelTimer t("k_vtx_density", s);
-            k_vtx_window<false><<<2 * grid, kThreads, 0, s>>>(a);
+            launch_pdl(k_vtx_window<false>, 2 * grid, kThreads, 0, s, a);
         }
         {
             KernelTimer t("k_vtx_link", s);
-            k_vtx_window<true><<<2 * grid, kThreads, 0, s>>>(a);
+            launch_pdl(k_vtx_window<true>, 2 * grid, kThreads, 0, s, a);
         }
         KernelTimer t("k_vtx_roots", s);
-        k_vtx_group<kVtxRoots><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+        launch_pdl(k_vtx_group<kVtxRoots>, n_events, kVtxThreads, kVtxDynSmem, s, a);
     } else {
         KernelTimer t("k_vtx_group", s);
-        k_vtx_group<kVtxAll><<<n_events, kVtxThreads, kVtxDynSmem, s>>>(a);
+        launch_pdl(k_vtx_group<kVtxAll>, n_events, kVtxThreads, kVtxDynSmem, s, a);
     }
     {
         KernelTimer t("k_vtx_fit", s);
-        k_vtx_fit<<<dim3(kVtxCap / kFitWarps, n_events), 32 * kFitWarps, 0, s>>>(a);
+        launch_pdl(k_vtx_fit, dim3(kVtxCap / kFitWarps, n_events), 32 * kFitWarps, 0, s, a);
     }
     KernelTimer t("k_vtx_order", s);
-    k_vtx_order<<<n_events, kOrderThreads, 0, s>>>(a);
+    launch_pdl(k_vtx_order, n_events, kOrderThreads, 0, s, a);
     return PT_OK;
 }
 
@@ -950,7 +957,7 @@ void launch_track_summary(int32_t n_tracks, const int32_t *hits, const uint8_t *
     // pT [GeV] = 0.299792458 B[T] R[m], R = 1 / (100 |kappa|) with kappa in 1/cm
     const float pt_of_kappa = 0.299792458e-2f * bz;
     KernelTimer t("k_track_summary", s);
-    k_track_summary<<<grid, kThreads, 0, s>>>(n_tracks, hits, tn, params, cov, tuple, ev_off, n_events, pt_of_kappa,
+    launch_pdl(k_track_summary, grid, kThreads, 0, s, n_tracks, hits, tn, params, cov, tuple, ev_off, n_events, pt_of_kappa,
                                              ev, z0, ez0, pt, nhits);
 }
 
