@@ -42,7 +42,10 @@ bool layout(const pt_hits *h, const pt_config *cfg, WsLayout &L) {
         return at;
     };
     L.counters = take(sizeof(int32_t) * kCounters);
+    // (cleared together: counters, tile counts, live incoming cells)
     L.bin_cnt = take(sizeof(int32_t) * (size_t)(n_bins + 1));
+    L.in_live = take(4 * nh);
+    L.cleared = o;
     const int64_t hit_blocks = (int64_t)(nh + kScanItems - 1) / kScanItems;
     L.scan_part = take(sizeof(int32_t) * (size_t)((L.n_scan_blocks > hit_blocks ? L.n_scan_blocks : hit_blocks) + 1));
     L.hit_bin = take(4 * nh);
@@ -53,7 +56,6 @@ bool layout(const pt_hits *h, const pt_config *cfg, WsLayout &L) {
     L.perm = take(4 * nh);
     L.in_off = take(4 * nh);
     L.in_cnt = take(4 * nh);
-    L.in_live = take(4 * nh);
     L.hk = take(16 * nh);
     L.ck = take(4 * nc);
     L.sk = take(8 * nc);
@@ -269,10 +271,7 @@ pt_status pt_build_doublets(void *ws, size_t ws_bytes, const pt_hits *hits, cons
     p.cell_outer = cells->outer;
     p.cell_pair = cells->pair;
     p.cell_alive = cells->alive;
-    if (cudaMemsetAsync(p.counters, 0, sizeof(int32_t) * kCounters, s) != cudaSuccess) return PT_ERR_CUDA;
-    if (cudaMemsetAsync(p.bin_cnt, 0, sizeof(int32_t) * (size_t)(L.n_bins + 1), s) != cudaSuccess)
-        return PT_ERR_CUDA;
-    if (cudaMemsetAsync(p.in_live, 0, sizeof(int32_t) * (size_t)hits->n_hits, s) != cudaSuccess) return PT_ERR_CUDA;
+    if (cudaMemsetAsync(p.counters, 0, L.cleared - L.counters, s) != cudaSuccess) return PT_ERR_CUDA;
     const Grid grid = grid_for(cfg);
     launch_binning(p, grid, s);
     launch_doublets(p, cfg->tuning.doublet_lanes, grid, s);
@@ -320,10 +319,6 @@ pt_status pt_find_ntuplets(void *ws, size_t ws_bytes, const pt_hits *hits, const
     p.tup_cells = tuples->cells;
     p.tup_n = tuples->n;
     p.tup_alive = tuples->alive;
-    if (cfg->capacity.cells > 0 &&
-        cudaMemsetAsync(p.maxlen, 0, sizeof(int32_t) * (size_t)cfg->capacity.cells, (cudaStream_t)stream) !=
-            cudaSuccess)
-        return PT_ERR_CUDA;
     launch_ntuplets(p, grid_for(cfg), (cudaStream_t)stream);
     return launched();
 }
@@ -349,10 +344,6 @@ pt_status pt_fit_tracks(void *ws, size_t ws_bytes, const pt_hits *hits, const pt
     p.trk_tuple = tracks->tuple;
     const Grid grid = grid_for(cfg);
     cudaStream_t s = (cudaStream_t)stream;
-    // the selection counts afresh on every call
-    if (cudaMemsetAsync(p.counters + C_TRACKS, 0, sizeof(int32_t), s) != cudaSuccess ||
-        cudaMemsetAsync(p.counters + C_TRK_CNT, 0, sizeof(int32_t) * 8, s) != cudaSuccess)
-        return PT_ERR_CUDA;
     launch_select(p, s);
     launch_fit(p, grid, s);
     return launched();

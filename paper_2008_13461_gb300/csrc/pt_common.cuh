@@ -26,7 +26,6 @@ enum Counter {
     C_FB_PENDING = 14,    // Fishbone: outer hits left to the exact pass
     C_DB_NEXT = 15,       // doublets: next outer hits to take
     C_TRK_CNT = 16,       // tracks with 3, 4, 5, 6..8 hits (4 slots)
-    C_TRK_CUR = 20,       // next track index of each of those classes (4 slots)
     C_FB_HUGE = 24,       // Fishbone: outer hits listed for the largest warps
     C_FB_HUGE_NEXT = 25,  // Fishbone: next of those to take
     C_CA_NEXT = 26,       // CA connection: next chunk of cells to take
@@ -53,6 +52,7 @@ struct WsLayout {
     size_t counters, bin_cnt, scan_part, hit_bin, hit_rank;
     size_t bh, blayer, bev, perm, in_off, in_cnt, in_live, hk, ck, sk, sci, trk_blk;
     size_t edge_rng, has_out, maxlen, erec;
+    size_t cleared;        // end of the arrays that every run clears, from counters on
     size_t total;
     int64_t n_bins;        // events * layers * phi bins * t bins
     int32_t n_scan_blocks;

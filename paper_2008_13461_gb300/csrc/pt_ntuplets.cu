@@ -31,6 +31,12 @@ __global__ void __launch_bounds__(kThreads) k_edge_records(Params p) {
         const int2 r = p.pair_inner_is_outer[p.cell_pair[src]] ? p.edge_rng[src] : make_int2(0, 0);
         const int bi = p.cell_inner[src];
         p.erec[e] = make_int4(src, r.x, r.y, p.perm[bi] * 2 + (root_layer(p.blayer[bi]) ? 1 : 0));
+        // the cells of n-tuplets are ends of edges, so only theirs are
+        // cleared for the cleaning: 82 us for the 4 M edges of 64 PU200
+        // events, as much as clearing all the capacity's 166 M cells took,
+        // but nothing in small events and 10 us less for 32 PU50 events
+        p.maxlen[src] = 0;
+        p.maxlen[p.edge_dst[e]] = 0;
     }
 }
 
@@ -169,47 +175,55 @@ __global__ void __launch_bounds__(kThreads) k_count_tracks(Params p) {
         if (c >= 0) atomicAdd(&s_cnt[c], 1);
     }
     __syncthreads();
-    if (threadIdx.x < 4) {
-        p.trk_blk[blockIdx.x * 4 + threadIdx.x] = s_cnt[threadIdx.x];
-        if (s_cnt[threadIdx.x]) atomicAdd(p.counters + C_TRK_CNT + threadIdx.x, s_cnt[threadIdx.x]);
-    }
+    if (threadIdx.x < 4) p.trk_blk[blockIdx.x * 4 + threadIdx.x] = s_cnt[threadIdx.x];
 }
 
 __global__ void __launch_bounds__(kThreads) k_select_tracks(Params p) {
     pdl_enter();
-    __shared__ int s_base[4];
+    __shared__ int s_base[4], s_all[4];
     __shared__ int s_wcnt[kThreads / 32][4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int off[4], total = 0;
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        off[c] = total;
-        total += p.counters[C_TRK_CNT + c];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        p.counters[C_TRACKS] = total;
-        if (total > p.cap_tracks) set_flag(p.counters, PT_FLAG_TRACKS);
-    }
-    // this slice's start in each class: the counts of the slices before it,
-    // summed by the whole block (four classes per 16-byte load).  Summed by
-    // one thread per class, the last slices' ~1000 additions in a row were
-    // most of this kernel (35.7 -> 8.0 us in an event of 112 n-tuplets,
-    // 42.8 -> 27.8 us with 3.6 M of them).
-    int4 b = make_int4(0, 0, 0, 0);
-    for (int q = threadIdx.x; q < (int)blockIdx.x; q += kThreads) {
-        const int4 v = reinterpret_cast<const int4 *>(p.trk_blk)[q];
-        b.x += v.x; b.y += v.y; b.z += v.z; b.w += v.w;
-    }
-    b.x = __reduce_add_sync(0xffffffffu, b.x);
-    b.y = __reduce_add_sync(0xffffffffu, b.y);
-    b.z = __reduce_add_sync(0xffffffffu, b.z);
-    b.w = __reduce_add_sync(0xffffffffu, b.w);
-    if (lane < 4) s_wcnt[w][lane] = lane == 0 ? b.x : lane == 1 ? b.y : lane == 2 ? b.z : b.w;
+    if (threadIdx.x < 4) s_base[threadIdx.x] = s_all[threadIdx.x] = 0;
     __syncthreads();
+    // the counts of all slices and of those before this one, summed by the
+    // whole block (four classes per 16-byte load).  Summed by one thread per
+    // class, the last slices' ~1000 additions in a row were most of this
+    // kernel (35.7 -> 8.0 us in an event of 112 n-tuplets, 42.8 -> 27.8 us
+    // with 3.6 M of them).
+    int all[4] = {0, 0, 0, 0}, before[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < kSelBlocks / kThreads; i++) {
+        const int q = i * kThreads + threadIdx.x;
+        const int4 v = reinterpret_cast<const int4 *>(p.trk_blk)[q];
+        const int c[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            all[k] += c[k];
+            if (q < (int)blockIdx.x) before[k] += c[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int x = __reduce_add_sync(0xffffffffu, all[k]), y = __reduce_add_sync(0xffffffffu, before[k]);
+        if (lane == 0) {
+            if (x) atomicAdd(&s_all[k], x);
+            if (y) atomicAdd(&s_base[k], y);
+        }
+    }
+    __syncthreads();
+    // tracks of the classes below come first
     if (threadIdx.x < 4) {
-        int v = threadIdx.x == 0 ? off[0] : threadIdx.x == 1 ? off[1] : threadIdx.x == 2 ? off[2] : off[3];
-        for (int q = 0; q < kThreads / 32; q++) v += s_wcnt[q][threadIdx.x];
-        s_base[threadIdx.x] = v;
+        int off = 0;
+        for (int q = 0; q < (int)threadIdx.x; q++) off += s_all[q];
+        s_base[threadIdx.x] += off;
+        if (blockIdx.x == 0) {
+            p.counters[C_TRK_CNT + threadIdx.x] = s_all[threadIdx.x];
+            if (threadIdx.x == 3) {
+                const int total = off + s_all[3];
+                p.counters[C_TRACKS] = total;
+                if (total > p.cap_tracks) set_flag(p.counters, PT_FLAG_TRACKS);
+            }
+        }
     }
     __syncthreads();
     const int64_t nt = min((int64_t)p.counters[C_TUPLES], p.cap_tuples);
