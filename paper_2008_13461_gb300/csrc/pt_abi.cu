@@ -199,6 +199,16 @@ Params make_params(void *ws, const WsLayout &L, const pt_hits *h, const pt_confi
         // far above float32 rounding of the angles involved
         p.pair_dphi[k] = (float)(atan(sqrt((double)c.pair[k].tan2_dphi)) + 1e-4);
         p.pair_pt_a[k] = c.pair[k].k_pt > 0.f ? (float)(1.0 / sqrt((double)c.pair[k].k_pt)) : 0.f;
+        // bounds used by the doublet filter, whose derivation is there
+        const pt_layer &li = cfg->geometry.layer[c.pair[k].inner], &lu = cfg->geometry.layer[c.pair[k].outer];
+        const double u = 5.9604645e-8, tan = sqrt((double)c.pair[k].tan2_dphi), zm = c.pair[k].zmax;
+        const double zi = fmax(fabs((double)li.zmin), fabs((double)li.zmax));
+        const double zo = fmax(fabs((double)lu.zmin), fabs((double)lu.zmax));
+        const double rr = (fabs((double)li.rmax) + 0.01) * (fabs((double)lu.rmax) + 0.01);
+        p.pair_tan[k] = (float)tan;
+        p.pair_err_zip[k] = (float)(8.0 * u * (zo * li.rmax + zi * lu.rmax + 2.0 * zm * (lu.rmax + li.rmax)) + 1e-27);
+        p.pair_err_phi[k] = (float)(8.0 * u * rr * (1.0 + tan) + 1e-27);
+        p.pair_err_c[k] = (float)(4.0 * u * rr);
         const int lo = c.pair[k].outer;
         p.pairs_by_outer[lo][p.n_pairs_by_outer[lo]++] = (int8_t)k;
         p.layer_is_inner[c.pair[k].inner] = 1;

@@ -12,23 +12,25 @@ namespace ptk {
 
 constexpr int kThreads = 256;            // threads per block of every kernel
 constexpr int kMaxPairsPerLayer = 8;
-constexpr int kCounters = 32 + 2 * PT_MAX_PAIRS;
-
-// workspace counters (int32 slots at the start of ws)
+// workspace counters (int32 slots at the start of ws).  The ones every warp
+// of a kernel adds to have 128 bytes to themselves: an L2 slice takes about
+// one atomic a clock.
+constexpr int kHot = 32 + 2 * PT_MAX_PAIRS;      // first of those, one per 32 slots
+constexpr int kCounters = kHot + 6 * 32;
 enum Counter {
-    C_CELLS = 0, C_EDGES = 1, C_TUPLES = 2, C_TRACKS = 3, C_FLAGS = 4, C_FALLBACK = 5,
+    C_CELLS = kHot, C_EDGES = kHot + 32, C_TUPLES = kHot + 64, C_TRACKS = 3, C_FLAGS = 4, C_FALLBACK = 5,
     C_ALIVE_CELLS = 6, C_ALIVE_TUPLES = 7,
-    C_FB_NEXT = 9,        // Fishbone: next chunk of outer hits to take
+    C_FB_NEXT = kHot + 96,     // Fishbone: next chunk of outer hits to take
     C_FB_BIG = 10,        // Fishbone: outer hits listed for the large warps
     C_FB_BIG_NEXT = 11,   // Fishbone: next listed outer hit to take
     C_CA_PENDING = 12,    // CA connection: cells left to the exact pass
     C_DB_PENDING = 13,    // doublets: outer hits left to the exact pass
     C_FB_PENDING = 14,    // Fishbone: outer hits left to the exact pass
-    C_DB_NEXT = 15,       // doublets: next outer hits to take
+    C_DB_NEXT = kHot + 128,    // doublets: next outer hits to take
     C_TRK_CNT = 16,       // tracks with 3, 4, 5, 6..8 hits (4 slots)
     C_FB_HUGE = 24,       // Fishbone: outer hits listed for the largest warps
     C_FB_HUGE_NEXT = 25,  // Fishbone: next of those to take
-    C_CA_NEXT = 26,       // CA connection: next chunk of cells to take
+    C_CA_NEXT = kHot + 160,    // CA connection: next chunk of cells to take
     C_PAIR_CAND = 32      // doublet candidates per layer pair (64-bit, PT_MAX_PAIRS of them)
 };
 
@@ -105,6 +107,10 @@ struct Params {
     pt_pair_cuts pair[PT_MAX_PAIRS];
     float pair_dphi[PT_MAX_PAIRS];       // azimuthal half window of PhiW (rad)
     float pair_pt_a[PT_MAX_PAIRS];       // 1 / (2 R) of the PT cut's minimum circumradius R (0: no cut)
+    float pair_tan[PT_MAX_PAIRS];        // sqrt(tan2_dphi)
+    float pair_err_zip[PT_MAX_PAIRS];    // rounding bounds of the doublet filter (pt_doublets.cu) over the
+    float pair_err_phi[PT_MAX_PAIRS];    //   pair's envelopes: of ZIP, of PhiW
+    float pair_err_c[PT_MAX_PAIRS];      //   and of the cross product i x o
     int32_t n_pairs;
     int8_t pairs_by_outer[PT_N_LAYERS][kMaxPairsPerLayer];
     int32_t n_pairs_by_outer[PT_N_LAYERS];

@@ -47,6 +47,54 @@ __device__ __forceinline__ void t_window(const Params &p, const pt_pair_cuts &pc
     }
 }
 
+// Fast filter of one candidate (i inner, o outer) for the main pass: 1 all
+// four cuts hold, 0 one of them fails, 2 too close to a cut to say.
+//
+// The sharper filters bring their own error bounds and compensated products,
+// about twice the operations (k_doublets 1721 -> 1652 us for 64 PU200 events),
+// so the cuts are taken in forms with few operations and bounds that are
+// constants of the pair; one candidate in ~10^5 lies within them and goes to
+// the sharper filters.  With u = 2^-24, hits within their layers' envelopes (checked on
+// input) and every rounding at most u relative:
+//  ZIP   F = (zmax ro - zmax ri) - |zi ro - zo ri|, each product and sum
+//        rounded at most twice: off by less than 3u (|zo| ri + |zi| ro +
+//        2 zmax (ro + ri)); taken as 8u with the layers' largest values.  F >
+//        0 implies ro > ri.
+//  PhiW  the condition is tan Dt - |C| >= 0 (Dt > 0 follows): |C| and Dt are
+//        off by 2u ri ro, tan by 2u relative: less than 5u ri ro (1 + tan),
+//        taken as 8u; |x|, |y| <= r + 2^-14.
+//  PT    H = |o-i|^2 |i|^2 - k C^2 with k = k_pt / |o|^2: the first term and k
+//        are off by 7u relative (differences of grid values are exact, sums of
+//        squares 3u, the product and the quotient the rest), C by c = 2u ri ro
+//        (taken as 4u) and so k C^2 by k (2 |C| c + c^2) besides; taken as
+//        16u (P + k C^2) + k (4 |C| c + 2 c^2).
+struct PairFilter {
+    float zlo, zhi, zmax, zr, tan, k, ez, ep, c4, kc2;
+};
+
+__device__ __forceinline__ int pair_filter(const PairFilter &f, const float4 &i, const float4 &o) {
+    const float F = fmaf(-f.zmax, i.w, f.zr) - fabsf(fmaf(i.z, o.w, -(o.z * i.w)));
+    const float C = fabsf(fmaf(i.x, o.y, -(i.y * o.x)));
+    const float G = fmaf(f.tan, fmaf(i.x, o.x, i.y * o.y), -C);
+    const float dx = o.x - i.x, dy = o.y - i.y;
+    const float P = fmaf(dx, dx, dy * dy) * fmaf(i.x, i.x, i.y * i.y);
+    const float q = f.k * C, t = q * C, H = P - t;
+    const float e = fmaf(16.0f * kU, P + t, fmaf(f.c4, q, f.kc2));
+    const bool zw = i.z >= f.zlo && i.z <= f.zhi;
+    if (zw && F > f.ez && G > f.ep && H > e) return 1;
+    return !zw || F < -f.ez || G < -f.ep || H < -e ? 0 : 2;
+}
+
+// One cell of outer hit o at index c.
+__device__ __forceinline__ void write_cell(const Params &p, int64_t c, int i, int o, uint8_t pair) {
+    if (c >= p.cap_cells) return;
+    p.cell_inner[c] = i;
+    p.cell_outer[c] = o;
+    p.cell_pair[c] = pair;
+    p.cell_alive[c] = 1;
+    p.has_out[c] = 0;
+}
+
 // Sweep all candidate inner hits of outer hit o.  kWrite = false: fill the
 // group's shared buffer (up to cap entries) and count; kWrite = true: write
 // cells directly at global index base + slot.  kExact = false: the
@@ -61,6 +109,7 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
     const float xo = ho.x, yo = ho.y, zo = ho.z, ro = ho.w;
     const int Lo = p.blayer[o], ev = p.bev[o];
     const float phio = atan2f(yo, xo);
+    const float io2 = __fdividef(1.0f, fmaf(xo, xo, yo * yo));
     const unsigned lanes = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     const unsigned below = (1u << lane) - 1u;
     int count = 0;
@@ -103,6 +152,17 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
             f0 = 0;
             f1 = p.n_phi - 1;
         }
+        PairFilter pf;
+        pf.zlo = pc.zlo;
+        pf.zhi = pc.zhi;
+        pf.zmax = pc.zmax;
+        pf.zr = pc.zmax * ro;
+        pf.tan = p.pair_tan[pi];
+        pf.k = pc.k_pt * io2;
+        pf.ez = p.pair_err_zip[pi];
+        pf.ep = p.pair_err_phi[pi];
+        pf.c4 = 4.0f * p.pair_err_c[pi];
+        pf.kc2 = 2.0f * pf.k * p.pair_err_c[pi] * p.pair_err_c[pi];
         const int row0 = (ev * PT_N_LAYERS + pc.inner) * p.n_phi;
         const int nrows = f1 - f0 + 1;
         unsigned cand = 0;
@@ -146,7 +206,9 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
                     i = sl + s_row[j];
                     const float4 hi = __ldg(p.bh + i);
                     const float xi = hi.x, yi = hi.y, zi = hi.z, ri = hi.w;
-                    if (zi >= pc.zlo && zi <= pc.zhi) {
+                    v = kExact ? 2 : pair_filter(pf, hi, ho);
+                    if (v == 2) v = zi >= pc.zlo && zi <= pc.zhi ? 2 : 0;
+                    if (v == 2) {
                         v = pred_zip<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, pc.zmax, p.counters);
                         if (v) {
                             const int v2 = pred_phiw<kExact>(xi, yi, xo, yo, pc.tan2_dphi, p.counters, zi, ri, zo, ro);
@@ -164,14 +226,7 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
                 if (acc) {
                     const int slot = count + __popc(m & below);
                     if (kWrite) {
-                        const int64_t c = base + slot;
-                        if (c < p.cap_cells) {
-                            p.cell_inner[c] = i;
-                            p.cell_outer[c] = o;
-                            p.cell_pair[c] = (uint8_t)pi;
-                            p.cell_alive[c] = 1;
-                            p.has_out[c] = 0;
-                        }
+                        write_cell(p, base + slot, i, o, (uint8_t)pi);
                     } else if (slot < cap) {
                         s_inner[slot] = i;
                         s_pair[slot] = (uint8_t)pi;
@@ -185,51 +240,25 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
     return count;
 }
 
-// Cells of outer hit o (one group of G lanes).  kExact = false: returns
-// false without writing anything when a candidate is undecided.
-template <int G, bool kExact>
-__device__ __forceinline__ bool doublets_hit(const Params &p, int o, int lane, unsigned gmask, int gshift,
-                                             int32_t *s_inner, uint8_t *s_pair, int32_t *s_row, int cap,
-                                             unsigned long long *s_cand = nullptr) {
-    bool und = false;
-    const int n = sweep_outer<G, false, kExact>(p, o, lane, gmask, gshift, s_inner, s_pair, s_row, cap, 0, &und,
-                                                 s_cand);
-    if (!kExact && __ballot_sync(gmask, und)) return false;
-    int64_t base = 0;
-    if (lane == 0 && n > 0) base = atomicAdd(p.counters + C_CELLS, n);
-    base = __shfl_sync(gmask, base, gshift);
-    if (n <= cap) {
-        __syncwarp(gmask);
-        for (int k = lane; k < n; k += G) {
-            const int64_t c = base + k;
-            if (c < p.cap_cells) {
-                p.cell_inner[c] = s_inner[k];
-                p.cell_outer[c] = o;
-                p.cell_pair[c] = s_pair[k];
-                p.cell_alive[c] = 1;
-                p.has_out[c] = 0;
-            }
-        }
-    } else {
-        sweep_outer<G, true, kExact>(p, o, lane, gmask, gshift, nullptr, nullptr, s_row, 0, base, &und);
-    }
-    if (lane == 0) {
-        p.in_off[o] = (int32_t)base;
-        p.in_cnt[o] = n;
-        if (base + n > p.cap_cells) set_flag(p.counters, PT_FLAG_CELLS);
-    }
-    __syncwarp(gmask);
-    return true;
+__device__ __forceinline__ void write_range(const Params &p, int o, int64_t base, int n) {
+    p.in_off[o] = (int32_t)base;
+    p.in_cnt[o] = n;
+    if (base + n > p.cap_cells) set_flag(p.counters, PT_FLAG_CELLS);
 }
 
 // Main pass: float32 filters only (no big-integer code, so far fewer
 // registers); an outer hit with an undecided candidate (about one in 10^3)
 // is listed for the exact pass.  It also counts the candidates tested per
 // layer pair (the exact pass repeats a few of them and does not count).
+// The cells of a warp's outer hits are reserved with one atomic and written
+// by all its lanes, hit after hit: with an atomic and a loop for each hit, the
+// one counter's L2 slice was 73% busy (all slices: 23%) and the byte arrays
+// were written eight bytes at a time (164 -> 104 us for 32 PU50 events, 110 ->
+// 100 us for one PU200 event, 1652 -> 1621 us for 64 of them).
 template <int G>
 __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
     pdl_enter();
-    constexpr int kGroups = kThreads / G;
+    constexpr int kGroups = kThreads / G, kPerWarp = 32 / G;
     constexpr int kBuf = 32 * G;   // 40 KB of shared memory per block for every G
     __shared__ int32_t s_inner[kGroups][kBuf];
     __shared__ uint8_t s_pair[kGroups][kBuf];
@@ -237,24 +266,58 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
     __shared__ unsigned long long s_cand[PT_MAX_PAIRS];
     if (threadIdx.x < PT_MAX_PAIRS) s_cand[threadIdx.x] = 0;
     __syncthreads();
-    const int lane = threadIdx.x % G, grp = threadIdx.x / G, wl = threadIdx.x & 31;
+    const int lane = threadIdx.x % G, grp = threadIdx.x / G, wl = threadIdx.x & 31, gw = wl / G;
     const int gshift = wl & ~(G - 1);
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << gshift);
     const int n_binned = p.bin_cnt[p.n_bins];
-    // the warps take the binned outer hits in order, 32 / G at a time: the
-    // cells are laid out nearly in the order of their outer hits
+    // the warps take the binned outer hits in order: the cells are laid out
+    // nearly in the order of their outer hits
     for (;;) {
         int o0 = 0;
-        if (wl == 0) o0 = atomicAdd(p.counters + C_DB_NEXT, 32 / G);
+        if (wl == 0) o0 = atomicAdd(p.counters + C_DB_NEXT, kPerWarp);
         o0 = __shfl_sync(0xffffffffu, o0, 0);
         if (o0 >= n_binned) break;
-        const int o = o0 + wl / G;
-        if (o < n_binned &&
-            !doublets_hit<G, false>(p, o, lane, gmask, gshift, s_inner[grp], s_pair[grp], s_row[grp], kBuf, s_cand) &&
-            lane == 0) {
-            // listed in hit_bin, free once the hits are binned (one slot per hit)
-            p.hit_bin[atomicAdd(p.counters + C_DB_PENDING, 1)] = o;
+        const int o = o0 + gw;
+        int n = 0;
+        bool und = false;
+        if (o < n_binned)
+            n = sweep_outer<G, false, false>(p, o, lane, gmask, gshift, s_inner[grp], s_pair[grp], s_row[grp], kBuf, 0,
+                                             &und, s_cand);
+        const unsigned um = __ballot_sync(0xffffffffu, und);
+        const bool put = o < n_binned && !(um & gmask);
+        // listed in hit_bin, free once the hits are binned (one slot per hit)
+        if (o < n_binned && !put && lane == 0) p.hit_bin[atomicAdd(p.counters + C_DB_PENDING, 1)] = o;
+        if (!put) n = 0;
+        int first[kPerWarp + 1];     // the groups' cells end to end
+        first[0] = 0;
+#pragma unroll
+        for (int q = 0; q < kPerWarp; q++) first[q + 1] = first[q] + __shfl_sync(0xffffffffu, n, q * G);
+        const int total = first[kPerWarp];
+        int64_t base = 0;
+        if (wl == 0 && total > 0) base = atomicAdd(p.counters + C_CELLS, total);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        int mine = 0;
+#pragma unroll
+        for (int q = 0; q < kPerWarp; q++) mine = gw == q ? first[q] : mine;
+        if (put && lane == 0) write_range(p, o, base + mine, n);
+        __syncwarp();
+        if (!__any_sync(0xffffffffu, n > kBuf)) {
+            for (int k = wl; k < total; k += 32) {
+                int q = 0, at = k;
+#pragma unroll
+                for (int t = 1; t < kPerWarp; t++)
+                    if (k >= first[t]) {
+                        q = t;
+                        at = k - first[t];
+                    }
+                write_cell(p, base + k, s_inner[grp - gw + q][at], o0 + q, s_pair[grp - gw + q][at]);
+            }
+        } else if (n <= kBuf) {      // beside a hit with more cells than its buffer holds
+            for (int k = lane; k < n; k += G) write_cell(p, base + mine + k, s_inner[grp][k], o, s_pair[grp][k]);
+        } else {
+            sweep_outer<G, true, false>(p, o, lane, gmask, gshift, nullptr, nullptr, s_row[grp], 0, base + mine, &und);
         }
+        __syncwarp();
     }
     __syncthreads();
     if (threadIdx.x < p.n_pairs && s_cand[threadIdx.x])
@@ -272,8 +335,22 @@ __global__ void __launch_bounds__(kThreads) k_doublets_exact(Params p) {
     __shared__ int32_t s_row[kGroups][2 * G];
     const int lane = threadIdx.x % G, grp = threadIdx.x / G;
     const int n = p.counters[C_DB_PENDING];
-    for (int k = grp * gridDim.x + blockIdx.x; k < n; k += gridDim.x * kGroups)
-        doublets_hit<G, true>(p, p.hit_bin[k], lane, 0xffffffffu, 0, s_inner[grp], s_pair[grp], s_row[grp], kBuf);
+    for (int k = grp * gridDim.x + blockIdx.x; k < n; k += gridDim.x * kGroups) {
+        const int o = p.hit_bin[k];
+        bool und = false;
+        const int nc = sweep_outer<G, false, true>(p, o, lane, 0xffffffffu, 0, s_inner[grp], s_pair[grp], s_row[grp],
+                                                   kBuf, 0, &und);
+        int64_t base = 0;
+        if (lane == 0 && nc > 0) base = atomicAdd(p.counters + C_CELLS, nc);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (lane == 0) write_range(p, o, base, nc);
+        __syncwarp();
+        if (nc <= kBuf)
+            for (int j = lane; j < nc; j += G) write_cell(p, base + j, s_inner[grp][j], o, s_pair[grp][j]);
+        else
+            sweep_outer<G, true, true>(p, o, lane, 0xffffffffu, 0, nullptr, nullptr, s_row[grp], 0, base, &und);
+        __syncwarp();
+    }
 }
 
 void launch_doublets(const Params &p, int lanes, const Grid &g, cudaStream_t s) {

@@ -19,7 +19,7 @@ namespace {
 // plus the counters.
 constexpr int64_t kMaxHits = int64_t(1) << 20;
 constexpr int64_t kMaxTiles = int64_t(1) << 22;
-constexpr size_t kCountersBytes = 256;
+constexpr size_t kCountersBytes = (sizeof(int32_t) * kCounters + 255) / 256 * 256;
 constexpr size_t kPartBytes = 4 * (size_t)(kMaxTiles / kScanItems + 256);
 constexpr size_t kScratchBytes = kCountersBytes + kPartBytes + 13 * (size_t)kMaxHits + 8 * 256;
 
