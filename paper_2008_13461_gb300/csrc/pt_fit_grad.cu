@@ -626,13 +626,16 @@ __device__ void grad_track(const Params &p, int32_t t, const float *gp, float gc
 }
 
 // One kernel per hit count, over the track range of that count.
-// Blocks of two warps, as in the fit (4 warps: 1486 -> 1408 us for 1 M
-// triplets, whose 170 registers let an SM hold 10 warps of these, 8 of
-// those), in four waves of resident blocks (with one, 1710 us).
+// Blocks of two warps, as in the fit (87 k tracks of 32 PU50 events: 107 ->
+// 99, 161 -> 161 and 83 -> 75 us for 3, 4 and 5 hits; 1 M triplets 1486 ->
+// 1464 us), in four waves of resident blocks (with one, 1710 us).  The code is
+// compiled for up to four warps: compiled for two, other multiply-adds are
+// fused, which the gradient of a nearly straight track (a difference of terms
+// in 1 / kappa^2) shows in its third digit.
 constexpr int kGradThreads = 64;
 
 template <int N>
-__global__ void __launch_bounds__(kGradThreads) k_fit_grad(Params p, const float *gpar, const float *gchi, float *gx, float *gy,
+__global__ void __launch_bounds__(128) k_fit_grad(Params p, const float *gpar, const float *gchi, float *gx, float *gy,
                                                   float *gz) {
     pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS | PT_FLAG_TUPLES | PT_FLAG_TRACKS)) return;
