@@ -92,7 +92,7 @@ class DifferentiableFit:
         b = self.bufs
         cfg = self.pipe._cfg(b.capacity)
         h = self._hits(x, y, z)
-        _, _, tuples, _ = b.structs()
+        tuples = b.tuples_struct()
         s = self._stream()
         L.fit_tracks(b.ws.data_ptr(), b.ws.numel(), h, cfg, tuples, self._tracks(), s)
         st, c = L.read_counts(b.ws.data_ptr(), b.ws.numel(), h, cfg, s)
@@ -106,11 +106,11 @@ class DifferentiableFit:
         dev = x.device
         gp = (gparams if gparams is not None else torch.zeros(0, 5, device=dev)).to(torch.float32).contiguous()
         gc = None if gchi2 is None else gchi2.to(torch.float32).contiguous()
-        gx, gy, gz = (torch.zeros_like(x) for _ in range(3))
+        gx, gy, gz = torch.zeros((3,) + x.shape, dtype=x.dtype, device=dev).unbind()
         if gparams is None:
             k = int(gc.numel()) if gc is not None else 0
             gp = torch.zeros(k, 5, device=dev)
-        _, _, tuples, _ = b.structs()
+        tuples = b.tuples_struct()
         L.fit_tracks_grad(b.ws.data_ptr(), b.ws.numel(), self._hits(x, y, z), self.pipe._cfg(b.capacity), tuples,
                           self._tracks(), gp.data_ptr(), None if gc is None else gc.data_ptr(), gx.data_ptr(),
                           gy.data_ptr(), gz.data_ptr(), self._stream())
@@ -137,9 +137,10 @@ class DifferentiableFit:
         gxo, gyo, gzo = ((g if g is not None else torch.zeros_like(x)).contiguous() for g in (gxo, gyo, gzo))
         nm = self.centres.shape[0]
         want_hits = any(needs[:3])
-        gx, gy, gz = ((torch.zeros_like(x) for _ in range(3)) if want_hits else (None, None, None))
-        gs = torch.zeros(nm, 3, device=x.device) if needs[3] else None
-        gr = torch.zeros(nm, 3, device=x.device) if needs[4] else None
+        gx, gy, gz = (torch.zeros((3,) + x.shape, dtype=x.dtype, device=x.device).unbind() if want_hits
+                      else (None, None, None))
+        gsr = torch.zeros(2, nm, 3, device=x.device)
+        gs, gr = (g if need else None for g, need in zip(gsr.unbind(), needs[3:5]))
         ptr = lambda t: None if t is None else t.data_ptr()
         L.align_hits_grad(x.numel(), x.data_ptr(), y.data_ptr(), z.data_ptr(), self.module.data_ptr(), nm,
                           self.centres.data_ptr(), rot.data_ptr(), gxo.data_ptr(), gyo.data_ptr(), gzo.data_ptr(),

@@ -50,10 +50,13 @@ class Buffers:
     trk_ndf: torch.Tensor
     trk_tuple: torch.Tensor
 
+    def tuples_struct(self):
+        return L.Tuples(_ptr(self.tup_hits), _ptr(self.tup_cells), _ptr(self.tup_n), _ptr(self.tup_alive))
+
     def structs(self):
         cells = L.Cells(_ptr(self.cell_inner), _ptr(self.cell_outer), _ptr(self.cell_pair), _ptr(self.cell_alive))
         edges = L.Edges(_ptr(self.edge_src), _ptr(self.edge_dst))
-        tuples = L.Tuples(_ptr(self.tup_hits), _ptr(self.tup_cells), _ptr(self.tup_n), _ptr(self.tup_alive))
+        tuples = self.tuples_struct()
         tracks = L.Tracks(_ptr(self.trk_params), _ptr(self.trk_cov), _ptr(self.trk_chi2), _ptr(self.trk_ndf),
                           _ptr(self.trk_tuple))
         return cells, edges, tuples, tracks
@@ -76,15 +79,12 @@ def find_vertices(ev, z0, ez0, pt, nhits, keep, n_events: int, cuts: dict | None
                              "int32 / float32 x3 / uint8 / uint8")
     s = (stream or torch.cuda.current_stream(dev)).cuda_stream
     E, M = n_events, max_vertices
-    out = dict(n=torch.empty(max(1, E), dtype=torch.int32, device=dev),
-               z=torch.empty(max(1, E * M), dtype=torch.float32, device=dev),
-               ez=torch.empty(max(1, E * M), dtype=torch.float32, device=dev),
-               chi2=torch.empty(max(1, E * M), dtype=torch.float32, device=dev),
-               sumpt2=torch.empty(max(1, E * M), dtype=torch.float32, device=dev),
-               ndf=torch.empty(max(1, E * M), dtype=torch.int32, device=dev),
-               ntracks=torch.empty(max(1, E * M), dtype=torch.int32, device=dev),
-               track_vertex=torch.empty(max(1, k), dtype=torch.int32, device=dev),
-               status=torch.zeros(1, dtype=torch.int32, device=dev))
+    # the call is short, so it allocates twice, not once per output (the
+    # library clears the status itself)
+    res = dict(zip(("n", "track_vertex", "status", "ndf", "ntracks"),
+                   torch.empty(E + k + 1 + 2 * E * M, dtype=torch.int32, device=dev).split((E, k, 1, E * M, E * M))))
+    res.update(zip(("z", "ez", "chi2", "sumpt2"), torch.empty(4, E, M, dtype=torch.float32, device=dev).unbind()))
+    res["ndf"], res["ntracks"] = res["ndf"].view(E, M), res["ntracks"].view(E, M)
     nbytes = L.vertex_scratch_size(k, E)
     scratch = torch.empty(2 * ((nbytes + 15) // 16), dtype=torch.int64, device=dev)     # 16-byte units
     assert scratch.numel() * scratch.element_size() >= nbytes
@@ -92,16 +92,12 @@ def find_vertices(ev, z0, ez0, pt, nhits, keep, n_events: int, cuts: dict | None
                          _ptr(keep))
     vc = L.VertexCuts(c["pt_min"], c["ez0_max"], c["dz_cut"], c["chi2_max"], c["split_chi2"], int(c["min_hits"]),
                       int(c["min_tracks"]))
-    vo = L.Vertices(*(out[n].data_ptr() for n in ("n", "z", "ez", "chi2", "sumpt2", "ndf", "ntracks",
+    vo = L.Vertices(*(res[n].data_ptr() for n in ("n", "z", "ez", "chi2", "sumpt2", "ndf", "ntracks",
                                                     "track_vertex", "status")))
     L.find_vertices(trk, k, E, vc, M, scratch.data_ptr(), scratch.numel() * scratch.element_size(), vo, s)
     if stream is not None:
         scratch.record_stream(stream)
-    out["scratch"] = scratch                                   # kept alive until the stream has used it
-    res = {n: (t[:E * M].view(E, M) if n in ("z", "ez", "chi2", "sumpt2", "ndf", "ntracks") else t)
-           for n, t in out.items()}
-    res["n"] = out["n"][:E]
-    res["track_vertex"] = out["track_vertex"][:k]
+    res["scratch"] = scratch                                   # kept alive until the stream has used it
     return res
 
 
@@ -195,6 +191,11 @@ class Pipeline:
         return L.Hits(x.data_ptr(), y.data_ptr(), z.data_ptr(), r.data_ptr(), module.data_ptr(), ev_off.data_ptr(),
                       x.numel(), ev_off.numel() - 1)
 
+    @staticmethod
+    def _sizes(x, ev_off) -> L.Hits:
+        """What the calls read that only look into the workspace."""
+        return L.Hits(None, None, None, None, None, None, x.numel(), ev_off.numel() - 1)
+
     def _cfg(self, capacity: dict) -> L.Config:
         c = L.Config.from_buffer_copy(self.cfg)
         c.capacity = L.Capacity(capacity["cells"], capacity["edges"], capacity["tuples"], capacity["tracks"])
@@ -236,26 +237,25 @@ class Pipeline:
 
     def counts(self, bufs: Buffers, x, y, z, r, module, ev_off, stream=None) -> tuple[int, L.Counts]:
         s = (stream or torch.cuda.current_stream(self.device)).cuda_stream
-        return L.read_counts(bufs.ws.data_ptr(), bufs.ws.numel(), self._hits(x, y, z, r, module, ev_off),
-                             self._cfg(bufs.capacity), s)
+        return L.read_counts(bufs.ws.data_ptr(), bufs.ws.numel(), self._sizes(x, ev_off), self._cfg(bufs.capacity), s)
 
     def hit_order(self, bufs: Buffers, x, y, z, r, module, ev_off) -> torch.Tensor:
         """Binned position -> input hit index (a view into the workspace)."""
-        h = self._hits(x, y, z, r, module, ev_off)
-        ptr = L.hit_order(bufs.ws.data_ptr(), bufs.ws.numel(), h, self._cfg(bufs.capacity))
-        off = ptr - bufs.ws.data_ptr()
-        return bufs.ws[off:off + 4 * max(1, x.numel())].view(torch.int32)[:x.numel()]
+        base, n = bufs.ws.data_ptr(), x.numel()
+        off = L.hit_order(base, bufs.ws.numel(), self._sizes(x, ev_off), self._cfg(bufs.capacity)) - base
+        return bufs.ws[off:off + 4 * n].view(torch.int32)
 
     def result(self, bufs: Buffers, counts: L.Counts, x, y, z, r, module, ev_off) -> Result:
         nc, ne, nt, nk = counts.n_cells, counts.n_edges, counts.n_tuples, counts.n_tracks
+        rows = lambda t, n, w: t.as_strided((n, w), (w, 1))        # one view each: small events notice
         return Result(
             counts=counts,
             cells=dict(inner=bufs.cell_inner[:nc], outer=bufs.cell_outer[:nc], pair=bufs.cell_pair[:nc],
                        alive=bufs.cell_alive[:nc]),
             edges=dict(src=bufs.edge_src[:ne], dst=bufs.edge_dst[:ne]),
-            tuples=dict(hits=bufs.tup_hits[:nt * L.NMAX].view(-1, L.NMAX), cells=bufs.tup_cells[:nt * L.NMAX]
-                        .view(-1, L.NMAX), n=bufs.tup_n[:nt], alive=bufs.tup_alive[:nt]),
-            tracks=dict(params=bufs.trk_params[:nk * 5].view(-1, 5), cov=bufs.trk_cov[:nk * 15].view(-1, 15),
+            tuples=dict(hits=rows(bufs.tup_hits, nt, L.NMAX), cells=rows(bufs.tup_cells, nt, L.NMAX),
+                        n=bufs.tup_n[:nt], alive=bufs.tup_alive[:nt]),
+            tracks=dict(params=rows(bufs.trk_params, nk, 5), cov=rows(bufs.trk_cov, nk, 15),
                         chi2=bufs.trk_chi2[:nk], ndf=bufs.trk_ndf[:nk], tuple=bufs.trk_tuple[:nk]),
             hit_order=self.hit_order(bufs, x, y, z, r, module, ev_off),
         )
@@ -268,8 +268,7 @@ class Pipeline:
         k, nc = counts.n_tracks, counts.n_cells
         keep = torch.empty(max(1, k), dtype=torch.uint8, device=self.device)
         scratch = torch.empty(max(1, nc + n_hits), dtype=torch.int32, device=self.device)
-        _, _, tuples, _ = bufs.structs()
-        L.resolve_ambiguities(tuples, bufs.trk_tuple.data_ptr(), k, bufs.trk_chi2.data_ptr(),
+        L.resolve_ambiguities(bufs.tuples_struct(), bufs.trk_tuple.data_ptr(), k, bufs.trk_chi2.data_ptr(),
                               bufs.trk_params.data_ptr() + 3 * 4, 5, nc, n_hits, scratch.data_ptr(), keep.data_ptr(), s)
         if stream is not None:
             scratch.record_stream(stream)      # freed here, used by `stream`: keep it until the work is done
@@ -281,10 +280,8 @@ class Pipeline:
         ev, z0, ez0, pt, nhits (device tensors of n_tracks)."""
         s = (stream or torch.cuda.current_stream(self.device)).cuda_stream
         k = counts.n_tracks
-        o = dict(ev=torch.empty(max(1, k), dtype=torch.int32, device=self.device),
-                 z0=torch.empty(max(1, k), dtype=torch.float32, device=self.device),
-                 ez0=torch.empty(max(1, k), dtype=torch.float32, device=self.device),
-                 pt=torch.empty(max(1, k), dtype=torch.float32, device=self.device),
+        o = dict(zip(("z0", "ez0", "pt"), torch.empty(3, max(1, k), dtype=torch.float32, device=self.device).unbind()),
+                 ev=torch.empty(max(1, k), dtype=torch.int32, device=self.device),
                  nhits=torch.empty(max(1, k), dtype=torch.uint8, device=self.device))
         _, _, tuples, tracks = bufs.structs()
         L.track_summary(self._hits(x, y, z, r, module, ev_off), tuples, tracks, k, self.cfg.fit.bz,
