@@ -48,39 +48,84 @@ struct DfsPath {
     int32_t hit[PT_NMAX - 1];
 };
 
+// n-tuplets found by a warp and not yet written.  One atomic on the counter of
+// n-tuplets for the few lanes that found one together is what bounded the
+// search (an L2 slice takes about one a clock); a warp reserves room for 32 or
+// more at a time and writes them as whole rows: 332 -> 155 us for the 3.6 M
+// n-tuplets of 64 PU200 events, 245 -> 144 us for 24 stress events (room for
+// 32, written from 8 on: 270 and 196 us).
+constexpr int kDfsWarps = kThreads / 32;
+constexpr int kDfsHold = 64;
+
+struct DfsHold {
+    int32_t hits[kDfsWarps][kDfsHold][PT_NMAX], cells[kDfsWarps][kDfsHold][PT_NMAX];   // unused places -1
+    uint8_t n[kDfsWarps][kDfsHold];
+    int count[kDfsWarps];
+};
+
 // the path of cells cell[D] (a root) .. cell[0] (the leaf) as an n-tuplet
 template <int D>
-__device__ __forceinline__ void dfs_emit(const Params &p, const DfsPath &pa, int leaf_outer) {
-    // one atomic for the lanes that emit together
-    const unsigned am = __activemask();
-    const int leader = __ffs(am) - 1, lane = threadIdx.x & 31;
-    int t = 0;
-    if (lane == leader) t = atomicAdd(p.counters + C_TUPLES, __popc(am));
-    t = __shfl_sync(am, t, leader) + __popc(am & ((1u << lane) - 1u));
-    if (t >= p.cap_tuples) {
-        set_flag(p.counters, PT_FLAG_TUPLES);
-        return;
+__device__ __forceinline__ void dfs_emit(const Params &p, DfsHold &hold, const DfsPath &pa, int leaf_outer) {
+    const int w = threadIdx.x >> 5;
+    int32_t *hits, *cells;
+    const int at = atomicAdd(&hold.count[w], 1);
+    if (at < kDfsHold) {
+        hits = hold.hits[w][at];
+        cells = hold.cells[w][at];
+        hold.n[w][at] = (uint8_t)(D + 2);
+    } else {          // no room before the warp meets again: straight to its place
+        const int t = atomicAdd(p.counters + C_TUPLES, 1);
+        if (t >= p.cap_tuples) {
+            set_flag(p.counters, PT_FLAG_TUPLES);
+            return;
+        }
+        hits = p.tup_hits + (int64_t)t * PT_NMAX;
+        cells = p.tup_cells + (int64_t)t * PT_NMAX;
+        p.tup_n[t] = (uint8_t)(D + 2);
+        p.tup_alive[t] = 1;
     }
-    int32_t *hits = p.tup_hits + (int64_t)t * PT_NMAX;
-    int32_t *cells = p.tup_cells + (int64_t)t * PT_NMAX;
     hits[0] = pa.hit[D] >> 1;
 #pragma unroll
-    for (int q = 0; q <= D; q++) {
+    for (int q = 0; q < PT_NMAX; q++) {
         // the outer hit of a cell is the inner hit of the next one
-        cells[q] = pa.cell[D - q];
-        hits[q + 1] = D - q >= 1 ? pa.hit[D - q - 1] >> 1 : leaf_outer;
+        cells[q] = q <= D ? pa.cell[q <= D ? D - q : 0] : -1;
+        if (q + 1 < PT_NMAX)
+            hits[q + 1] = q < D ? pa.hit[q < D ? D - q - 1 : 0] >> 1 : q == D ? leaf_outer : -1;
     }
-    p.tup_n[t] = (uint8_t)(D + 2);
-    p.tup_alive[t] = 1;
+}
+
+// writes the warp's held n-tuplets (whole warp)
+__device__ __forceinline__ void dfs_flush(const Params &p, DfsHold &hold) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __syncwarp();
+    const int n = min(hold.count[w], kDfsHold);
+    int t0 = 0;
+    if (lane == 0 && n > 0) t0 = atomicAdd(p.counters + C_TUPLES, n);
+    t0 = __shfl_sync(0xffffffffu, t0, 0);
+    const int fit = (int)max((int64_t)0, min((int64_t)n, p.cap_tuples - t0));
+    if (fit < n && lane == 0) set_flag(p.counters, PT_FLAG_TUPLES);
+    int32_t *hits = p.tup_hits + (int64_t)t0 * PT_NMAX, *cells = p.tup_cells + (int64_t)t0 * PT_NMAX;
+    for (int k = lane; k < fit * PT_NMAX; k += 32) {
+        hits[k] = (&hold.hits[w][0][0])[k];
+        cells[k] = (&hold.cells[w][0][0])[k];
+    }
+    for (int k = lane; k < fit; k += 32) {
+        p.tup_n[t0 + k] = hold.n[w][k];
+        p.tup_alive[t0 + k] = 1;
+    }
+    __syncwarp();
+    if (lane == 0) hold.count[w] = 0;
+    __syncwarp();
 }
 
 // Depth D of the search: cell[D] has cnt incoming edges from position first.
 // No incoming edge: a path starts here, emitted if cell[D] is a root and the
 // path has at least three hits.  Paths longer than PT_NMAX hits are cut.
 template <int D>
-__device__ __forceinline__ void dfs_level(const Params &p, DfsPath &pa, int first, int cnt, int leaf_outer) {
+__device__ __forceinline__ void dfs_level(const Params &p, DfsHold &hold, DfsPath &pa, int first, int cnt,
+                                          int leaf_outer) {
     if (cnt == 0) {
-        if (D >= 1 && (pa.hit[D] & 1)) dfs_emit<D>(p, pa, leaf_outer);
+        if (D >= 1 && (pa.hit[D] & 1)) dfs_emit<D>(p, hold, pa, leaf_outer);
         return;
     }
     if constexpr (D + 1 < PT_NMAX - 1) {
@@ -90,7 +135,7 @@ __device__ __forceinline__ void dfs_level(const Params &p, DfsPath &pa, int firs
             const int4 r = p.erec[e];
             pa.cell[D + 1] = r.x;
             pa.hit[D + 1] = r.w;
-            dfs_level<D + 1>(p, pa, r.y, r.z, leaf_outer);
+            dfs_level<D + 1>(p, hold, pa, r.y, r.z, leaf_outer);
         }
     }
 }
@@ -102,18 +147,27 @@ __global__ void __launch_bounds__(kThreads) k_dfs(Params p) {
     pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int64_t ne = min((int64_t)p.counters[C_EDGES], p.cap_edges);
+    __shared__ DfsHold hold;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) hold.count[w] = 0;
+    __syncwarp();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += stride) {
-        const int c = p.edge_dst[e];
-        if (p.has_out[c]) continue;
-        const int4 r = p.erec[e];
-        DfsPath pa;
-        pa.cell[0] = c;
-        pa.hit[0] = p.perm[p.cell_inner[c]] * 2;
-        pa.cell[1] = r.x;
-        pa.hit[1] = r.w;
-        dfs_level<1>(p, pa, r.y, r.z, p.perm[p.cell_outer[c]]);
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; e0 < ne; e0 += stride) {
+        const int64_t e = e0 + lane;
+        const int c = e < ne ? p.edge_dst[e] : -1;
+        if (c >= 0 && !p.has_out[c]) {
+            const int4 r = p.erec[e];
+            DfsPath pa;
+            pa.cell[0] = c;
+            pa.hit[0] = p.perm[p.cell_inner[c]] * 2;
+            pa.cell[1] = r.x;
+            pa.hit[1] = r.w;
+            dfs_level<1>(p, hold, pa, r.y, r.z, p.perm[p.cell_outer[c]]);
+        }
+        __syncwarp();
+        if (hold.count[w] >= kDfsHold / 2) dfs_flush(p, hold);
     }
+    dfs_flush(p, hold);
 }
 
 // L(c) = longest n-tuplet containing cell c
