@@ -34,7 +34,7 @@ enum Counter {
     C_PAIR_CAND = 32      // doublet candidates per layer pair (64-bit, PT_MAX_PAIRS of them)
 };
 
-// Slope-key bucket of a live incoming cell of a hit with n of them (lowest
+// Slope-key bucket of an incoming cell of a hit with n of them (lowest
 // key k0, inverse bucket width iw): the Fishbone orders the cells by it and
 // the connection searches by it, so both evaluate these same roundings.
 // For an integer b in [1, nb - 1], sk_bucket(key) < b exactly when
@@ -80,10 +80,10 @@ struct Params {
                                          //   incoming edges, input index of its inner hit * 2 + root
     float *ck;                           // R-z slope key of each cell w.r.t. its outer hit (scratch)
     float4 *hk;                          // per hit: max sqrt(1+key^2) and min gap of its incoming
-                                         //   cells; lowest key and inverse bucket width of the live ones
-    int32_t *in_live;                    // per hit: live incoming cells
-    float2 *sk;                          // live incoming cells of each hit by slope-key bucket:
-    int32_t *sci;                        //   (key, inner hit as int bits) and the cell index
+                                         //   cells; lowest key and inverse bucket width
+    int32_t *in_live;                    // per hit: incoming cells listed in sk, sci (0: none)
+    float2 *sk;                          // incoming cells of each hit by slope-key bucket: (key, inner hit
+    int32_t *sci;                        //   as int bits, -1 for a dead cell) and the cell index
     uint8_t *has_out;
     int32_t *maxlen;
     int32_t *trk_blk;                    // track selection: per block and class, counts then offsets

@@ -4,9 +4,9 @@
 //
 // Cells (b,c) are taken in cell order (cells are grouped by their outer hit
 // c, so neighbouring threads work on neighbouring middle hits).
-// The live cells ending on b were written by the Fishbone kernel ordered by
+// The cells ending on b were written by the Fishbone kernel ordered by
 // a bucket of their R-z slope key relative to b (monotone in the key, about
-// one cell per bucket), with their inner hits, so the candidates (a,b) of a
+// one cell per bucket), with their inner hits (-1 for the dead ones), so the candidates (a,b) of a
 // cell lie in a contiguous run of that array (the buckets of its key
 // window), found by binary search over the buckets.
 //
@@ -152,7 +152,7 @@ __device__ __forceinline__ int scan_cell(const Params &p, int x, Emit &&emit) {
     for (int r = lower_bucket(S, ns, sk_bucket(lo, hk.z, hk.w, nb), hk.z, hk.w); r < ns; r++) {
         const float2 e = __ldg(S + r);
         if (sk_coord(e.x, hk.z, hk.w) >= fend) break;     // a bucket above hi's
-        if (!(fabsf(e.x - key_c) <= wdt)) continue;
+        if (!(fabsf(e.x - key_c) <= wdt) || __float_as_int(e.y) < 0) continue;      // (-1: a dead cell)
         const int v = connects<kExact>(p, __ldg(p.bh + __float_as_int(e.y)), B, C, rg);
         if (v == 2) return -2;
         if (v) emit(n++, b0 + r);

@@ -12,16 +12,34 @@
 // memory traffic.  Alignment within eps implies that the unit directions of
 // two siblings differ by at most du = eps pi/2 (plus float32 slack), hence
 // so does any 1-Lipschitz key of them (u^_z for a barrel o, the radial
-// component for a disk o).  The siblings are counting-sorted into about
-// one key bucket each, and each cell is compared only with the later cells
+// component for a disk o).  The siblings are counting-sorted into one or two
+// key buckets each, and each cell is compared only with the later cells
 // of its own bucket and of the next K buckets, K covering a key difference
 // of du: a superset of its aligned siblings, so the result is exact at
 // ~O(k) work per outer hit.
 //
+// The same pass prepares the CA connection: it writes the cells of o ordered
+// by a bucket of their R-z slope key relative to o (with the inner hit, -1
+// for a dead cell, and the cell index; the bucket is monotone in the key,
+// about one cell per bucket, free order inside), the bucket parameters, and
+// per hit the bounds the slope window needs (over all cells of o).  Both sorts
+// are done at once: their counters share 32-bit words, so one clearing, one
+// scan and one loop over the cells each for counting and placing serve both.
+//
+// What bounds it is the work in shared memory and the instructions around
+// it.  For 64 PU200 events (small and medium warps) 2.84 + 0.75 ms; with the
+// scan's 16-byte accesses (its entries met in a few banks: half of the
+// kernel's shared-memory cycles) 2.69 + 0.70 ms; with both sorts at once and
+// up to two direction buckets per cell 2.19 + 0.78 ms; 24 events with pT > 0.3
+// GeV 0.84 + 1.17 + 0.52 ms (small, medium, large) to 0.67 + 0.92 + 0.36 ms; 32
+// PU50 events 193 to 151 us.  A dead cell is marked with a byte store: the same
+// with an atomicOr of a bit, in a branch that single lanes take, costs
+// 0.77 ms; so does a list of the close pairs for later, 0.2 ms.
+//
 // Shared memory per warp bounds the siblings it can hold, and the warps an
 // SM can keep resident bound how well the gathers of the inner hits are
-// hidden.  Most outer hits have fewer than ~200 cells, so three launches
-// share the work: many small warps take chunks of 32 outer hits from a queue
+// hidden.  Most outer hits have fewer than ~180 cells, so three launches
+// share the work: many small warps take chunks of outer hits from a queue
 // and list the outer hits with more cells, which medium (up to 320 cells)
 // and large warps (up to 512) then take one at a time; an exact pass takes
 // the rest (undecided tests, more cells), sorted in shared memory like the
@@ -29,37 +47,32 @@
 // hits), with a pairwise loop over global memory beyond: that loop from 512
 // cells on took 2.15 of the 8.8 ms of a batch of 24 such events, against
 // 0.07 ms now.
-//
-// The same pass prepares the CA connection: it writes the live cells of o
-// ordered by a bucket of their R-z slope key relative to o (with the inner
-// hit and the cell index; the bucket is monotone in the key, about one cell
-// per bucket, free order inside), the bucket parameters, and per hit the
-// bounds the slope window needs (taken over all cells of o, a superset of
-// the live ones, so the window only widens).
 #include "pt_common.cuh"
 #include "pt_kernels.cuh"
 
 namespace ptk {
 
-constexpr int kFbDirect = 12;        // up to this many siblings: compare all pairs
-
-// Per warp and cell: u = h_inner - h_o (exact) and 1/|u| in w; the cell's
-// position (bits 0-9), its inner layer (10-14) and key bucket (16-25).
-// C: the cell's R-z slope key and inner hit are kept for the second pass
-// (else written to and read back from global memory).
-template <int W, int M, int NB, bool C>
-struct FbSmem {
-    float4 rec[W][M];
-    int meta[W][M];
-    int16_t idx[W][M];               // cell positions sorted by bucket
-    uint8_t dead[W][M];
-    int pos[W][NB];
-    float ck[W][C ? M : 1];
-    int32_t inner[W][C ? M : 1];
+// Per warp: the cells of one outer hit (up to M) and NB bucket counters, whose
+// low halves count the cells by direction key and whose high halves by
+// R-z slope key, so that one scan serves both sorts.
+// C: the slope keys are kept here (else written to and read back from global
+// memory, for warps whose cells would not fit otherwise).
+template <int M, int NB, bool C>
+struct __align__(16) FbWarp {
+    float4 rec[M];                   // u = h_inner - h_o (exact), 1/|u| in w
+    uint32_t pos[NB];                // counts, then starts, then ends
+    float ck[C ? M : 1];             // R-z slope key
+    uint32_t meta[M];                // slot; then direction bucket and, in the high half, slope bucket and then place
+    uint16_t idx[M];                 // cells sorted by direction bucket
+    uint8_t dead[M];
 };
 
-__device__ __forceinline__ int rec_cell(int m) { return m & 1023; }
-constexpr int kRecLayerMask = 31 << 10;
+// pair_slot in shared memory: a lane-wise index into the kernel's parameters
+// would serialise
+__device__ __forceinline__ void load_slots(const Params &p, uint8_t *slot) {
+    if (threadIdx.x < PT_MAX_PAIRS) slot[threadIdx.x] = (uint8_t)p.pair_slot[threadIdx.x];
+    __syncthreads();
+}
 
 // Bucket key of a record: u^_z (barrel o) or the radial component of u^
 // (disk o; (rx, ry) is o's radial direction).  Explicit roundings, so every
@@ -77,24 +90,6 @@ __device__ __forceinline__ long long len2u(float ux, float uy, float uz) {
 
 __device__ __forceinline__ int cell_layer(const Params &p, int64_t c) { return p.pair[p.cell_pair[c]].inner; }
 
-// Does sibling d (record r2, meta m2) kill cell j (record r1, unit vector
-// v1, meta m1)?  Same inner layer, unit directions close (a necessary
-// condition of alignment), aligned, and strictly shorter or as long with a
-// smaller input index of the inner hit.  kExact = false: an undecided
-// alignment sets und.
-template <bool kExact>
-__device__ __forceinline__ bool fb_kills(const Params &p, int64_t b, int j, const float4 &r1, const float3 &v1,
-                                         int m1, int d, int m2, const float4 &r2, float unit_thr, bool &und) {
-    if (d == j || ((m1 ^ m2) & kRecLayerMask)) return false;
-    const float dx = v1.x - r2.x * r2.w, dy = v1.y - r2.y * r2.w, dz = v1.z - r2.z * r2.w;
-    if (dx * dx + dy * dy + dz * dz > unit_thr) return false;
-    const int v = pred_fb_d<kExact>(r1.x, r1.y, r1.z, r2.x, r2.y, r2.z, p.fishbone_eps2, p.counters);
-    if (v == 2) und = true;
-    if (v != 1) return false;
-    const long long l1 = len2u(r1.x, r1.y, r1.z), l2 = len2u(r2.x, r2.y, r2.z);
-    return l2 < l1 || (l2 == l1 && p.perm[p.cell_inner[b + d]] < p.perm[p.cell_inner[b + j]]);
-}
-
 // Warp-wide minimum, maximum and sum with one redux instruction each.  The
 // float map keeps their order (non-negative floats keep their bits,
 // negative ones have the magnitude bits flipped; no NaN reaches it), and a
@@ -108,52 +103,53 @@ __device__ __forceinline__ float warp_min(float f) { return fval(__reduce_min_sy
 __device__ __forceinline__ float warp_max(float f) { return fval(__reduce_max_sync(0xffffffffu, ford(f))); }
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xffffffffu, v); }
 
-// exclusive prefix sum of a[0, nb) in place (nb a power of two >= 32;
-// one warp, nb / 32 entries per lane)
-__device__ __forceinline__ void warp_exclusive_scan(int *a, int nb, int lane) {
-    const int per = nb >> 5;
-    int sum = 0;
-    for (int q = 0; q < per; q++) sum += a[lane * per + q];
-    int incl = sum;
+// exclusive prefix sums of both halves of a[0, nb) in place (nb a power of two >= 32; one
+// warp): 128 entries at a time, four per lane in one 16-byte access.  (Entries
+// lane * nb / 32 + q, one after the other, met in 2 to 4 banks: half of the
+// kernel's shared-memory cycles were those conflicts.)
+__device__ __forceinline__ void warp_exclusive_scan(uint32_t *a, int nb, int lane) {
+    uint32_t carry = 0;
+    for (int q = 4 * lane; q - 4 * lane < nb; q += 128) {
+        uint4 v = q < nb ? *reinterpret_cast<const uint4 *>(a + q) : make_uint4(0, 0, 0, 0);
+        const uint32_t sum = (v.x + v.y) + (v.z + v.w);
+        uint32_t incl = sum;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += t;
-    }
-    int run = incl - sum;
-    for (int q = 0; q < per; q++) {
-        const int v = a[lane * per + q];
-        a[lane * per + q] = run;
-        run += v;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += t;
+        }
+        const uint32_t e = carry + incl - sum;
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+        v = make_uint4(e, e + v.x, e + v.x + v.y, e + v.x + v.y + v.z);
+        if (q < nb) *reinterpret_cast<uint4 *>(a + q) = v;
     }
 }
 
-// Verdicts of the n cells of outer hit o (one warp); returns the lane's
-// count of live cells.  kGlobal: n may exceed M (pairwise loop compiled in).
-// kExact = false (float32 filters only): returns -1, having written no
-// verdict, when n > M or an alignment test is undecided.
-template <int W, int M, int NB, bool kGlobal, bool kExact, bool C>
-__device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64_t b, int lane, int w,
-                                            float unit_thr, float du, FbSmem<W, M, NB, C> &sm) {
-    // NB: at least the buckets of M cells (sk_buckets), and of the direction sort
+// Verdicts of the n <= M cells of outer hit o (one warp); returns the lane's
+// count of live cells.  kExact = false (float32 filters only): returns -1,
+// having written no verdict, when an alignment test is undecided.
+template <int M, int NB, bool C, bool kExact>
+__device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64_t b, int lane, float unit_thr,
+                                            float du, FbWarp<M, NB, C> &sm, const uint8_t *slot) {
+    // NB: at least the buckets of M cells (sk_buckets)
     static_assert(NB >= 32 && NB >= M && (NB & (NB - 1)) == 0, "bucket array too small");
-    if (!kExact && n > M) return -1;
     const float4 ho = __ldg(p.bh + o);
-    const bool disk = p.layer[p.blayer[o]].kind == PT_LAYER_DISK;
-    const bool in_smem = !kGlobal || n <= M;
+    const int Lo = p.blayer[o];
+    const bool disk = p.layer[Lo].kind == PT_LAYER_DISK;
     const float irr = rsqrtf(ho.x * ho.x + ho.y * ho.y);
     const float rx = ho.x * irr, ry = ho.y * irr;
     // a hit on a layer that is the inner layer of no pair starts no cell:
     // the connection never reads the slope keys of the cells ending on it
-    const bool starts = p.layer_is_inner[p.blayer[o]] != 0;
-    // pass 1: R-z slope keys (barrel o: (z_o - z_a)/(r_o - r_a); disk o:
-    // (r_o - r_a)/(z_o - z_a)) with the per-hit bounds; records and the
-    // range of the bucket keys
+    const bool starts = p.layer_is_inner[Lo] != 0;
+    // pass 1: records, direction keys' range, and the R-z slope keys (barrel
+    // o: (z_o - z_a)/(r_o - r_a); disk o: (r_o - r_a)/(z_o - z_a)) with the
+    // per-hit bounds and their range
     float k2max = 0.f, gmin = 3.0e38f, bmin = 3.0f, bmax = -3.0f;
+    float smin = __int_as_float(0x7f800000), smax = -smin;
     for (int j = lane; j < n; j += 32) {
-        const int i = p.cell_inner[b + j];
-        const int L = cell_layer(p, b + j);
-        const float4 a = __ldg(p.bh + i);
+        const float4 a = __ldg(p.bh + p.cell_inner[b + j]);
+        sm.meta[j] = slot[p.cell_pair[b + j]];
+        sm.dead[j] = 0;
         if (starts) {
             const float dr = ho.w - a.w, dz = ho.z - a.z;
             const float num = disk ? dr : dz, den = disk ? dz : dr;
@@ -162,215 +158,181 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
             const float ck = den != 0.f ? __fdividef(num, den) : __int_as_float(0x7f800000);
             k2max = fmaxf(k2max, ck * ck);
             gmin = fminf(gmin, fabsf(den));
-            if (C && in_smem) {
-                sm.ck[w][j] = ck;
-                sm.inner[w][j] = i;
-            } else {
-                p.ck[b + j] = ck;
+            if (C) sm.ck[j] = ck;
+            else p.ck[b + j] = ck;
+            if (fabsf(ck) <= 3.4e38f) {
+                smin = fminf(smin, ck);
+                smax = fmaxf(smax, ck);
             }
         }
-        if (in_smem) {
-            const float ux = a.x - ho.x, uy = a.y - ho.y, uz = a.z - ho.z;
-            const float4 r = make_float4(ux, uy, uz, rsqrtf(ux * ux + uy * uy + uz * uz));
-            sm.rec[w][j] = r;
-            sm.meta[w][j] = j | (L << 10) | (p.pair_slot[p.cell_pair[b + j]] << 26);
-            sm.dead[w][j] = 0;
-            const float key = fb_key(r, disk, rx, ry);
-            bmin = fminf(bmin, key);
-            bmax = fmaxf(bmax, key);
-        }
+        const float ux = a.x - ho.x, uy = a.y - ho.y, uz = a.z - ho.z;
+        const float4 r = make_float4(ux, uy, uz, rsqrtf(ux * ux + uy * uy + uz * uz));
+        sm.rec[j] = r;
+        const float key = fb_key(r, disk, rx, ry);
+        bmin = fminf(bmin, key);
+        bmax = fmaxf(bmax, key);
     }
-    k2max = warp_max(k2max);
-    gmin = warp_min(gmin);
-    const float kmax = sqrtf(1.0f + k2max);        // max of sqrt(1 + key^2)
-    if (lane == 0 && starts) reinterpret_cast<float2 *>(p.hk + o)[0] = make_float2(kmax, gmin);
+    bmin = warp_min(bmin);
+    bmax = warp_max(bmax);
+    // Direction buckets: each inner layer of o has its own aligned range of
+    // nbr buckets (one or two buckets per cell), so a cell meets only siblings
+    // on its own layer.  Two keys within du lie at most K buckets apart (K
+    // bounds du / width plus the rounding of the bucket coordinates, below
+    // 6e-4 for up to 2048 buckets).  Slope buckets: about one per cell.
+    const int nbs = sk_buckets(n), nb = min(NB, 2 * nbs);
+    const int nbr = nb >> p.fb_slot_shift[Lo];
+    const float span = fmaxf(bmax - bmin, fmaxf(fabsf(bmin), fabsf(bmax)) * 1e-6f);
+    const float iw = span > 0.f ? (float)nbr / span : 0.f;
+    const int K = (int)fminf(du * iw + 6e-4f, (float)nbr) + 1;
+    float siw = 0.f;
+    if (starts) {
+        k2max = warp_max(k2max);
+        gmin = warp_min(gmin);
+        smin = warp_min(smin);
+        smax = warp_max(smax);
+        const float sspan = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
+        siw = sspan > 0.f && sspan <= 3.4e38f ? (float)nbs / sspan : 0.f;
+        // bound of sqrt(1 + key^2), smallest gap, lowest key, inverse width
+        if (lane == 0) p.hk[o] = make_float4(sqrtf(1.0f + k2max), gmin, smin, siw);
+    }
+    for (int q = lane; q < nb; q += 32) sm.pos[q] = 0;
     __syncwarp();
-
+    for (int j = lane; j < n; j += 32) {
+        const float key = fb_key(sm.rec[j], disk, rx, ry);
+        uint32_t m = sm.meta[j] * nbr + min(max((int)((key - bmin) * iw), 0), nbr - 1);
+        atomicAdd(&sm.pos[m], 1u);
+        if (starts) {
+            const uint32_t bs = sk_bucket(C ? sm.ck[j] : p.ck[b + j], smin, siw, nbs);
+            atomicAdd(&sm.pos[bs], 1u << 16);
+            m |= bs << 16;
+        }
+        sm.meta[j] = m;
+    }
+    __syncwarp();
+    warp_exclusive_scan(sm.pos, nb, lane);
+    __syncwarp();
+    for (int j = lane; j < n; j += 32) {
+        const uint32_t m = sm.meta[j];
+        sm.idx[atomicAdd(&sm.pos[m & 0xffffu], 1u) & 0xffffu] = (uint16_t)j;
+        if (starts)
+            sm.meta[j] = (m & 0xffffu) | (atomicAdd(&sm.pos[m >> 16], 1u << 16) & 0xffff0000u);
+    }
+    __syncwarp();
+    // sm.pos[bk] now holds the ends of bucket bk.  Each pair once: every cell
+    // against the cells after it in its own bucket and the next K buckets of
+    // its layer (a superset of its siblings within du of its key); of an
+    // aligned pair the longer cell dies (equal lengths: the larger input
+    // index of the inner hit).
     bool und = false;
-    if (kGlobal && !in_smem) {
-        // more siblings than the warp holds: plain pairwise loop
-        const GHit gh = ghit(ho.x, ho.y, ho.z, ho.w);
-        const FHit h = {ho.x, ho.y, ho.z, ho.w};
-        for (int j = lane; j < n; j += 32) {
-            const int i1 = p.cell_inner[b + j];
-            const int L1 = cell_layer(p, b + j);
-            const FHit h1 = load_hit(p.bh, i1);
-            const GHit g1 = ghit(h1.x, h1.y, h1.z, h1.r);
-            const long long l1 = (g1.x - gh.x) * (g1.x - gh.x) + (g1.y - gh.y) * (g1.y - gh.y) +
-                                 (g1.z - gh.z) * (g1.z - gh.z);
-            bool dead = false;
-            for (int d = 0; d < n && !dead; d++) {
-                if (d == j || cell_layer(p, b + d) != L1) continue;
-                const int i2 = p.cell_inner[b + d];
-                const FHit h2 = load_hit(p.bh, i2);
-                if (!pred_fb(h1, h2, h, p.fishbone_eps2, p.counters)) continue;
-                const GHit g2 = ghit(h2.x, h2.y, h2.z, h2.r);
-                const long long l2 = (g2.x - gh.x) * (g2.x - gh.x) + (g2.y - gh.y) * (g2.y - gh.y) +
-                                     (g2.z - gh.z) * (g2.z - gh.z);
-                dead = l2 < l1 || (l2 == l1 && p.perm[i2] < p.perm[i1]);
-            }
-            if (dead) p.cell_alive[b + j] = 0;
-        }
-    } else if (n <= kFbDirect) {
-        for (int j = lane; j < n; j += 32) {
-            const float4 r1 = sm.rec[w][j];
-            const float3 v1 = make_float3(r1.x * r1.w, r1.y * r1.w, r1.z * r1.w);
-            const int m1 = sm.meta[w][j];
-            bool dead = false;
-            for (int d = 0; d < n && !dead; d++)
-                dead = fb_kills<kExact>(p, b, j, r1, v1, m1, d, sm.meta[w][d], sm.rec[w][d], unit_thr, und);
-            if (dead) sm.dead[w][j] = 1;
-        }
-    } else {
-        bmin = warp_min(bmin);
-        bmax = warp_max(bmax);
-        // counting sort of the cells into buckets of (inner layer, direction
-        // key): each inner layer of o has its own aligned range of nbr
-        // buckets (about one bucket per cell), so a cell meets only siblings
-        // on its own layer.  Two keys within du lie at most K buckets apart
-        // (K bounds du / width plus the rounding of the bucket coordinates,
-        // below 3e-4 for up to 1024 buckets).
-        const int nb = min(NB, max(32, 1 << (32 - __clz(n - 1))));
-        const int ssh = p.fb_slot_shift[p.blayer[o]];
-        const int nbr = nb >> ssh;
-        const float span = fmaxf(bmax - bmin, fmaxf(fabsf(bmin), fabsf(bmax)) * 1e-6f);
-        const float iw = span > 0.f ? (float)nbr / span : 0.f;
-        const int K = (int)fminf(du * iw + 3e-4f, (float)nbr) + 1;
-        for (int q = lane; q < nb; q += 32) sm.pos[w][q] = 0;
-        __syncwarp();
-        for (int j = lane; j < n; j += 32) {
-            const float key = fb_key(sm.rec[w][j], disk, rx, ry);
-            const int m = sm.meta[w][j];
-            const int bk = (m >> 26) * nbr + min(max((int)((key - bmin) * iw), 0), nbr - 1);
-            sm.meta[w][j] = (m & 0xffff) | (bk << 16);
-            atomicAdd(&sm.pos[w][bk], 1);
-        }
-        __syncwarp();
-        warp_exclusive_scan(sm.pos[w], nb, lane);
-        __syncwarp();
-        for (int j = lane; j < n; j += 32) sm.idx[w][atomicAdd(&sm.pos[w][sm.meta[w][j] >> 16], 1)] = (int16_t)j;
-        __syncwarp();
-        // sm.pos[bk] is now the end of bucket bk.  Each pair once: every cell
-        // against the cells after it in its own bucket and the next K
-        // buckets of its layer (a superset of its siblings within du of its
-        // key); of an aligned pair the longer cell dies (equal lengths: the
-        // larger input index of the inner hit).
-        for (int q0 = lane; q0 < n; q0 += 32) {
-            const int j = sm.idx[w][q0];
-            const float4 r1 = sm.rec[w][j];
-            const float3 v1 = make_float3(r1.x * r1.w, r1.y * r1.w, r1.z * r1.w);
-            const int bk1 = sm.meta[w][j] >> 16;
-            const int qend = sm.pos[w][min(bk1 + K, bk1 | (nbr - 1))];
-            for (int q = q0 + 1; q < qend; q++) {
-                const int d = sm.idx[w][q];
-                const float4 r2 = sm.rec[w][d];
-                const float dx = v1.x - r2.x * r2.w, dy = v1.y - r2.y * r2.w, dz = v1.z - r2.z * r2.w;
-                if (dx * dx + dy * dy + dz * dz > unit_thr) continue;
-                const int v = pred_fb_d<kExact>(r1.x, r1.y, r1.z, r2.x, r2.y, r2.z, p.fishbone_eps2, p.counters);
-                if (v == 2) und = true;
-                if (v != 1) continue;
-                const long long l1 = len2u(r1.x, r1.y, r1.z), l2 = len2u(r2.x, r2.y, r2.z);
-                const bool j_wins = l1 < l2 || (l1 == l2 && p.perm[p.cell_inner[b + j]] < p.perm[p.cell_inner[b + d]]);
-                sm.dead[w][j_wins ? d : j] = 1;
-            }
+    for (int q0 = lane; q0 < n; q0 += 32) {
+        const int j = sm.idx[q0];
+        const float4 r1 = sm.rec[j];
+        const float3 v1 = make_float3(r1.x * r1.w, r1.y * r1.w, r1.z * r1.w);
+        const int bk1 = sm.meta[j] & 0xffffu;
+        const int qend = sm.pos[min(bk1 + K, bk1 | (nbr - 1))] & 0xffffu;
+        for (int q = q0 + 1; q < qend; q++) {
+            const int d = sm.idx[q];
+            const float4 r2 = sm.rec[d];
+            const float dx = v1.x - r2.x * r2.w, dy = v1.y - r2.y * r2.w, dz = v1.z - r2.z * r2.w;
+            if (dx * dx + dy * dy + dz * dz > unit_thr) continue;
+            const int v = pred_fb_d<kExact>(r1.x, r1.y, r1.z, r2.x, r2.y, r2.z, p.fishbone_eps2, p.counters);
+            if (v == 2) und = true;
+            if (v != 1) continue;
+            const long long l1 = len2u(r1.x, r1.y, r1.z), l2 = len2u(r2.x, r2.y, r2.z);
+            const bool j_wins = l1 < l2 || (l1 == l2 && p.perm[p.cell_inner[b + j]] < p.perm[p.cell_inner[b + d]]);
+            sm.dead[j_wins ? d : j] = 1;
         }
     }
     __syncwarp();
     if (!kExact && __any_sync(0xffffffffu, und)) return -1;
 
-    // pass 2: the live cells, grouped by slope-key bucket for the CA
-    // connection.  A hit on a layer that is the inner layer of no pair
-    // starts no cell, so the connection never searches the cells ending on
-    // it: only their Fishbone verdicts are written.
+    // pass 2: the verdicts, and the cells grouped by slope-key bucket for the
+    // CA connection, a dead one with the inner hit -1 (any order inside a
+    // bucket: the connection searches by bucket)
     int alive = 0;
-    if (!starts) {
-        int nl = 0;
-        for (int j = lane; j < n; j += 32) {
-            const bool dead = in_smem ? sm.dead[w][j] != 0 : p.cell_alive[b + j] == 0;
-            if (dead && in_smem) p.cell_alive[b + j] = 0;
-            alive += !dead;
-        }
-        nl = warp_sum(alive);
-        if (lane == 0) p.in_live[o] = nl;
-    } else if (in_smem) {
-        // slope key and inner hit of each live cell (the records are free)
-        float smin = __int_as_float(0x7f800000), smax = -smin;
-        for (int j = lane; j < n; j += 32) {
-            if (sm.dead[w][j]) {
-                p.cell_alive[b + j] = 0;
-                continue;
-            }
-            const float key = C ? sm.ck[w][j] : p.ck[b + j];
-            const int ii = C ? sm.inner[w][j] : p.cell_inner[b + j];
-            sm.rec[w][j] = make_float4(key, __int_as_float(ii), 0.f, 0.f);
-            if (fabsf(key) <= 3.4e38f) {
-                smin = fminf(smin, key);
-                smax = fmaxf(smax, key);
-            }
-            alive++;
-        }
-        const int nl = warp_sum(alive);
-        smin = warp_min(smin);
-        smax = warp_max(smax);
-        // counting sort into about one bucket per cell; the connection
-        // searches by bucket, so the order inside a bucket is free
-        const int nb = sk_buckets(nl);
-        const float span = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
-        const float iw = span > 0.f && span <= 3.4e38f ? (float)nb / span : 0.f;
-        for (int q = lane; q < nb; q += 32) sm.pos[w][q] = 0;
-        __syncwarp();
-        for (int j = lane; j < n; j += 32) {
-            if (sm.dead[w][j]) continue;
-            const int bk = sk_bucket(sm.rec[w][j].x, smin, iw, nb);
-            sm.meta[w][j] = bk;
-            atomicAdd(&sm.pos[w][bk], 1);
-        }
-        __syncwarp();
-        warp_exclusive_scan(sm.pos[w], nb, lane);
-        __syncwarp();
-        for (int j = lane; j < n; j += 32) {
-            if (sm.dead[w][j]) continue;
-            const float4 r = sm.rec[w][j];
-            const int q = atomicAdd(&sm.pos[w][sm.meta[w][j]], 1);
-            p.sk[b + q] = make_float2(r.x, r.y);
-            p.sci[b + q] = (int32_t)(b + j);
-        }
-        if (lane == 0) {
-            p.in_live[o] = nl;
-            reinterpret_cast<float2 *>(p.hk + o)[1] = make_float2(smin, iw);
-        }
-    } else {
-        // (only outer hits with very many cells) rank by direct comparison:
-        // sorted keys, so sorted buckets too
-        float smin = __int_as_float(0x7f800000), smax = -smin;
-        for (int j = lane; j < n; j += 32) {
-            if (!p.cell_alive[b + j]) continue;
-            const float key = p.ck[b + j];
-            const int ii = p.cell_inner[b + j];
-            int rank = 0;
-            for (int i = 0; i < n; i++) {
-                if (!p.cell_alive[b + i]) continue;
-                const float ki = p.ck[b + i];
-                rank += ki < key || (ki == key && i < j);
-            }
-            p.sk[b + rank] = make_float2(key, __int_as_float(ii));
-            p.sci[b + rank] = (int32_t)(b + j);
-            if (fabsf(key) <= 3.4e38f) {
-                smin = fminf(smin, key);
-                smax = fmaxf(smax, key);
-            }
-            alive++;
-        }
-        const int nl = warp_sum(alive);
-        smin = warp_min(smin);
-        smax = warp_max(smax);
-        const float span = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
-        const float iw = span > 0.f && span <= 3.4e38f ? (float)sk_buckets(nl) / span : 0.f;
-        if (lane == 0) {
-            p.in_live[o] = nl;
-            reinterpret_cast<float2 *>(p.hk + o)[1] = make_float2(smin, iw);
+    for (int j = lane; j < n; j += 32) {
+        const bool dead = sm.dead[j];
+        if (dead) p.cell_alive[b + j] = 0;
+        else alive++;
+        if (starts) {
+            const int64_t q = b + (sm.meta[j] >> 16);
+            p.sk[q] = make_float2(C ? sm.ck[j] : p.ck[b + j], __int_as_float(dead ? -1 : p.cell_inner[b + j]));
+            p.sci[q] = (int32_t)(b + j);
         }
     }
+    if (lane == 0) p.in_live[o] = n;       // (never all dead: the shortest of them lives)
+    __syncwarp();
+    return alive;
+}
+
+// The same for any n with a pairwise loop over global memory and ranks by
+// direct comparison (outer hits with more cells than a warp holds: sorted
+// keys, so sorted buckets too).
+__device__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int lane) {
+    const float4 ho = __ldg(p.bh + o);
+    const bool disk = p.layer[p.blayer[o]].kind == PT_LAYER_DISK;
+    const bool starts = p.layer_is_inner[p.blayer[o]] != 0;
+    const GHit gh = ghit(ho.x, ho.y, ho.z, ho.w);
+    const FHit h = {ho.x, ho.y, ho.z, ho.w};
+    float k2max = 0.f, gmin = 3.0e38f;
+    float smin = __int_as_float(0x7f800000), smax = -smin;
+    for (int j = lane; j < n; j += 32) {
+        const int i1 = p.cell_inner[b + j];
+        const int L1 = cell_layer(p, b + j);
+        const FHit h1 = load_hit(p.bh, i1);
+        if (starts) {
+            const float dr = ho.w - h1.r, dz = ho.z - h1.z;
+            const float num = disk ? dr : dz, den = disk ? dz : dr;
+            const float ck = den != 0.f ? __fdividef(num, den) : __int_as_float(0x7f800000);
+            k2max = fmaxf(k2max, ck * ck);
+            gmin = fminf(gmin, fabsf(den));
+            p.ck[b + j] = ck;
+            if (fabsf(ck) <= 3.4e38f) {
+                smin = fminf(smin, ck);
+                smax = fmaxf(smax, ck);
+            }
+        }
+        const GHit g1 = ghit(h1.x, h1.y, h1.z, h1.r);
+        const long long l1 = (g1.x - gh.x) * (g1.x - gh.x) + (g1.y - gh.y) * (g1.y - gh.y) +
+                             (g1.z - gh.z) * (g1.z - gh.z);
+        bool dead = false;
+        for (int d = 0; d < n && !dead; d++) {
+            if (d == j || cell_layer(p, b + d) != L1) continue;
+            const int i2 = p.cell_inner[b + d];
+            const FHit h2 = load_hit(p.bh, i2);
+            if (!pred_fb(h1, h2, h, p.fishbone_eps2, p.counters)) continue;
+            const GHit g2 = ghit(h2.x, h2.y, h2.z, h2.r);
+            const long long l2 = (g2.x - gh.x) * (g2.x - gh.x) + (g2.y - gh.y) * (g2.y - gh.y) +
+                                 (g2.z - gh.z) * (g2.z - gh.z);
+            dead = l2 < l1 || (l2 == l1 && p.perm[i2] < p.perm[i1]);
+        }
+        if (dead) p.cell_alive[b + j] = 0;
+    }
+    if (starts) {
+        k2max = warp_max(k2max);
+        gmin = warp_min(gmin);
+        smin = warp_min(smin);
+        smax = warp_max(smax);
+        const float span = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
+        const float iw = span > 0.f && span <= 3.4e38f ? (float)sk_buckets(n) / span : 0.f;
+        if (lane == 0) p.hk[o] = make_float4(sqrtf(1.0f + k2max), gmin, smin, iw);
+    }
+    __syncwarp();
+    int alive = 0;
+    for (int j = lane; j < n; j += 32) {
+        const bool dead = p.cell_alive[b + j] == 0;
+        alive += !dead;
+        if (!starts) continue;
+        const float key = p.ck[b + j];
+        int rank = 0;
+        for (int i = 0; i < n; i++) {
+            const float ki = p.ck[b + i];
+            rank += ki < key || (ki == key && i < j);
+        }
+        p.sk[b + rank] = make_float2(key, __int_as_float(dead ? -1 : p.cell_inner[b + j]));
+        p.sci[b + rank] = (int32_t)(b + j);
+    }
+    if (lane == 0) p.in_live[o] = n;
     __syncwarp();
     return alive;
 }
@@ -394,15 +356,17 @@ __device__ __forceinline__ void add_alive(const Params &p, int v) {
 // with 32 whatever the size, one PU200 event (30.8 k hits) kept 962 of 4864
 // warps busy (454 -> 75 us with chunks by size; a PU50 event 158 -> 19 us, a
 // batch of 32 of them 279 -> 194 us).
-constexpr int kFbSmallMax = 192;
+constexpr int kFbSmallMax = 184;
 constexpr int kFbMidMax = 320;
 
-template <int W, int M, int NB, int kMinBlocks>
+template <int W, int M, int NB, int kMinBlocks, bool C = true>
 __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p, float unit_thr, float du,
                                                                     int chunk_log2) {
     pdl_enter();
-    __shared__ FbSmem<W, M, NB, true> sm;
+    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ uint8_t s_slot[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
+    load_slots(p, s_slot);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     int my_alive = 0;
@@ -439,7 +403,7 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
             todo &= todo - 1;
             const int n = __shfl_sync(0xffffffffu, nl, t);
             const int b = __shfl_sync(0xffffffffu, bl, t);
-            const int a = fishbone_hit<W, M, NB, false, false, true>(p, o0 + t, n, b, lane, w, unit_thr, du, sm);
+            const int a = fishbone_hit<M, NB, C, false>(p, o0 + t, n, b, lane, unit_thr, du, sm[w], s_slot);
             if (a >= 0) my_alive += a;
             else list_pending(p, o0 + t, lane);
         }
@@ -452,8 +416,10 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
 template <int W, int M, int NB, bool kFromBack, bool C>
 __global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_thr, float du) {
     pdl_enter();
-    __shared__ FbSmem<W, M, NB, C> sm;
+    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ uint8_t s_slot[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
+    load_slots(p, s_slot);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int my_alive = 0;
     const int n_list = p.counters[kFromBack ? C_FB_HUGE : C_FB_BIG];
@@ -463,8 +429,8 @@ __global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_
         k = __shfl_sync(0xffffffffu, k, 0);
         if (k >= n_list) break;
         const int o = p.fb_big[kFromBack ? p.n_hits - 1 - k : k];
-        const int a = fishbone_hit<W, M, NB, false, false, C>(p, o, p.in_cnt[o], p.in_off[o], lane, w, unit_thr, du,
-                                                              sm);
+        const int n = p.in_cnt[o];
+        const int a = n <= M ? fishbone_hit<M, NB, C, false>(p, o, n, p.in_off[o], lane, unit_thr, du, sm[w], s_slot) : -1;
         if (a >= 0) my_alive += a;
         else list_pending(p, o, lane);
     }
@@ -474,17 +440,21 @@ __global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_
 // Exact pass: the outer hits listed by the kernels above (an undecided
 // alignment test, or more cells than a large warp holds), with the exact
 // predicate and the pairwise loop for any number of cells.
-template <int W, int M, int NB>
+template <int W, int M, int NB, bool C = true>
 __global__ void __launch_bounds__(32 * W) k_fishbone_exact(Params p, float unit_thr, float du) {
     pdl_enter();
-    __shared__ FbSmem<W, M, NB, true> sm;
+    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ uint8_t s_slot[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
+    load_slots(p, s_slot);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int my_alive = 0;
     const int n_list = p.counters[C_FB_PENDING];
     for (int k = blockIdx.x * W + w; k < n_list; k += gridDim.x * W) {
         const int o = p.hit_bin[k];
-        my_alive += fishbone_hit<W, M, NB, true, true, true>(p, o, p.in_cnt[o], p.in_off[o], lane, w, unit_thr, du, sm);
+        const int n = p.in_cnt[o], b = p.in_off[o];
+        my_alive += n <= M ? fishbone_hit<M, NB, C, true>(p, o, n, b, lane, unit_thr, du, sm[w], s_slot)
+                           : fishbone_pairwise(p, o, n, b, lane);
     }
     add_alive(p, my_alive);
 }
@@ -495,7 +465,7 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
         int chunk_log2 = 0;
         while (chunk_log2 < 5 && (p.n_hits >> (chunk_log2 + 1)) >= 4 * 8 * g.blocks(4)) chunk_log2++;
         KernelTimer t("k_fishbone_small", s);
-        launch_pdl(k_fishbone_small<8, kFbSmallMax, 256, 4>, g.blocks(4), 256, 0, s, p, unit_thr, du, chunk_log2);
+        launch_pdl(k_fishbone_small<8, kFbSmallMax, 512, 4>, g.blocks(4), 256, 0, s, p, unit_thr, du, chunk_log2);
     }
     {
         KernelTimer t("k_fishbone_medium", s);
@@ -503,7 +473,7 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
     }
     {
         KernelTimer t("k_fishbone_large", s);
-        launch_pdl(k_fishbone_large<2, 512, 1024, true, true>, g.blocks(5), 64, 0, s, p, unit_thr, du);
+        launch_pdl(k_fishbone_large<2, 512, 1024, true, true>, g.blocks(6), 64, 0, s, p, unit_thr, du);
     }
     KernelTimer t("k_fishbone_exact", s);
     launch_pdl(k_fishbone_exact<1, 1024, 1024>, g.blocks(6), 32, 0, s, p, unit_thr, du);
