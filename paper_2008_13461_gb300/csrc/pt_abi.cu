@@ -60,6 +60,7 @@ bool layout(const pt_hits *h, const pt_config *cfg, WsLayout &L) {
     L.ck = take(4 * nc);
     L.sk = take(8 * nc);
     L.sci = take(4 * nc);
+    L.sk_end = take(2 * nc);
     L.edge_rng = take(8 * nc);
     L.has_out = take(nc);
     L.maxlen = take(4 * nc);
@@ -176,6 +177,7 @@ Params make_params(void *ws, const WsLayout &L, const pt_hits *h, const pt_confi
     p.ck = (float *)(w + L.ck);
     p.sk = (float2 *)(w + L.sk);
     p.sci = (int32_t *)(w + L.sci);
+    p.sk_end = (uint16_t *)(w + L.sk_end);
     p.in_live = (int32_t *)(w + L.in_live);
     p.edge_rng = (int2 *)(w + L.edge_rng);
     p.has_out = (uint8_t *)(w + L.has_out);

@@ -46,13 +46,20 @@ __device__ __forceinline__ int sk_bucket(float key, float k0, float iw, int nb) 
     return min(max(__float2int_rz(sk_coord(key, k0, iw)), 0), nb - 1);
 }
 
+// The ends of those buckets, for the connection to start at: one per 1 << sk_end_shift
+// buckets, as many as leave no more of them than cells (a power of
+// two), for hits of up to kSkEnds cells (what a warp of the Fishbone sorts).
+constexpr int kSkEnds = 1024;
+__device__ __forceinline__ int sk_ends(int n) { return 1 << (31 - __clz(n)); }
+__device__ __forceinline__ int sk_end_shift(int n) { return max(5, 32 - __clz(n - 1)) - (31 - __clz(n)); }
+
 // class of a track by its hit count: 3, 4, 5, 6..8 -> 0..3
 __device__ __forceinline__ int track_class(int n) { return min(n, 6) - 3; }
 
 // Byte offsets of every workspace array (all 256-byte aligned).
 struct WsLayout {
     size_t counters, bin_cnt, scan_part, hit_bin, hit_rank;
-    size_t bh, blayer, bev, perm, in_off, in_cnt, in_live, hk, ck, sk, sci, trk_blk;
+    size_t bh, blayer, bev, perm, in_off, in_cnt, in_live, hk, ck, sk, sci, sk_end, trk_blk;
     size_t edge_rng, has_out, maxlen, erec;
     size_t cleared;        // end of the arrays that every run clears, from counters on
     size_t total;
@@ -84,6 +91,7 @@ struct Params {
     int32_t *in_live;                    // per hit: incoming cells listed in sk, sci (0: none)
     float2 *sk;                          // incoming cells of each hit by slope-key bucket: (key, inner hit
     int32_t *sci;                        //   as int bits, -1 for a dead cell) and the cell index
+    uint16_t *sk_end;                    // per hit, from its first cell on: ends of its slope-key buckets (sk_ends)
     uint8_t *has_out;
     int32_t *maxlen;
     int32_t *trk_blk;                    // track selection: per block and class, counts then offsets

@@ -6,9 +6,12 @@
 // c, so neighbouring threads work on neighbouring middle hits).
 // The cells ending on b were written by the Fishbone kernel ordered by
 // a bucket of their R-z slope key relative to b (monotone in the key, about
-// one cell per bucket), with their inner hits (-1 for the dead ones), so the candidates (a,b) of a
-// cell lie in a contiguous run of that array (the buckets of its key
-// window), found by binary search over the buckets.
+// one cell per bucket), with their inner hits (-1 for a dead one), so the candidates (a,b) of a
+// cell lie in a contiguous run of that array, the buckets of its key
+// window; the Fishbone also leaves the ends of the buckets, so the run is
+// found with two loads (a binary search took about seven one after the
+// other: 2167 -> 1970 us for 64 PU200 events, and the ends cost the Fishbone 55).
+// Longer lists than a warp of the Fishbone sorts are searched.
 //
 // The R-z cut is very tight, so it is first used as a window on the slope
 // key.  For a barrel b, with key = dz/dr of a segment,
@@ -22,19 +25,28 @@
 // window test itself, a float32 R-z test with an error bound and then the
 // exact predicate chain decide.
 //
-// The kernel waits on dependent L2 loads, so it is compiled for 10
-// resident blocks of 4 warps per SM (48 registers), which hides more of that
-// latency than 8 blocks did, and spills less than 12.
+// A warp takes 128 consecutive cells at a time, in order from a queue, and
+// lists those that can have candidates (their inner hit's layer is the outer
+// layer of a pair: about a quarter).  Each lane then finds the run of one of
+// them, but what comes after is done on the runs laid end to end, an entry per
+// lane, and the entries that pass the window are collected until 32 are
+// there for the predicates: a run has 0 to ~10 entries, two on average, of
+// which one in three passes, so with a cell per lane from start to end 12 of 32
+// lanes were at work on average, and the loads of a run came one after the
+// other.  What passes comes in the order of the cells, so the edges of a
+// cell are contiguous in the order found (the depth-first search walks them
+// backwards from the cell's edge range), and the warp writes the edges of its
+// 128 cells with one reservation.
 //
-// A warp takes 128 consecutive cells at a time, in order from a queue.
-// Only cells whose inner hit has live cells ending on it have candidates at
-// all (about a quarter), so the warp first lists those and then runs their
-// searches on full lanes.
-// The incoming edges of a cell are written contiguously (the depth-first
-// search walks them backwards from the cell's edge range); the warp
-// reserves the edges of its 128 cells with one atomic, each cell remembers
-// its first few accepted candidates in shared memory, and a cell with more
-// (rare) scans again to write them all.
+// The kernel waits on dependent L2 loads, so it is compiled for as many
+// resident warps as its shared memory leaves (12 blocks of 4 per SM, 40
+// registers; 10 blocks: 10% slower).  64 PU200 events 1970 -> 1410 us, 24
+// events with pT > 0.3 GeV 1420 -> 940, 32 PU50 events 95 -> 70, one PU200
+// event 78 -> 51.  Chunks of 64 or 96 cells take 14% and 6% longer (rounds of
+// searches that are not full), of 192 or 256 no less, and leave an end of few
+// warps in one event (63, 75 us); a claim of the next chunk ahead of time
+// does the same (70 us).  One 64-byte record of what is read of a middle
+// hit, and a search with four probes at a time, measured the same or worse.
 //
 // The predicates run as float32 filters only; a cell with a candidate they
 // cannot decide (about one in 10^5) is left to a second pass that has the
@@ -46,8 +58,9 @@
 namespace ptk {
 
 constexpr int kCaWarps = 4;
-constexpr int kCaQueue = 4;         // accepted candidates remembered per cell
 constexpr int kCaChunk = 4;         // rounds of 32 cells per edge reservation
+constexpr int kCaPer = 32 * kCaChunk;
+constexpr int kCaAcc = 160;         // edges a warp remembers
 
 // The predicate chain: 1 connects, 0 does not; with kExact = false, 2 when
 // a float32 filter cannot decide and none fails.
@@ -101,7 +114,8 @@ __device__ __forceinline__ int warp_excl(int v, int lane, int &total) {
     return incl - v;
 }
 
-// first position of s[0, n) whose key's bucket is >= bk (buckets ascending)
+// first position of s[0, n) whose key's bucket is >= bk (buckets ascending);
+// for the lists without ends of buckets
 __device__ __forceinline__ int lower_bucket(const float2 *s, int n, int bk, float k0, float iw) {
     const float fb = (float)bk;
     int l = 0, h = bk > 0 ? n : 0;
@@ -113,65 +127,201 @@ __device__ __forceinline__ int lower_bucket(const float2 *s, int n, int bk, floa
     return l;
 }
 
-// Every inner cell (a,b) connecting to the live cell x = (b,c), in the
-// order of b's bucket-ordered arrays: emit(t, i) for the t-th one, i its
-// index there.
-// Returns their number, or -2 (kExact = false) when a candidate is
-// undecided.
-template <bool kExact, class Emit>
-__device__ __forceinline__ int scan_cell(const Params &p, int x, Emit &&emit) {
-    const int b = p.cell_inner[x], c = p.cell_outer[x];
+// The candidates (a,b) of a cell x = (b,c): entries [r, end) of b's
+// bucket-ordered arrays, of which those with |key - key_c| <= wdt pass the
+// window.
+struct Search {
+    FHit B, C;
+    float key_c, wdt;
+    int32_t r, end;
+    bool disk;
+};
+
+__device__ __forceinline__ Search search_of(const Params &p, int b, int c) {
+    Search s;
+    s.r = s.end = 0;
     const int64_t b0 = p.in_off[b];
     int ns = p.in_live[b];
     if (b0 + ns > p.cap_cells) ns = 0;
-    if (ns == 0) return 0;
-    const FHit B = load_hit(p.bh, b), C = load_hit(p.bh, c);
-    const bool disk = p.layer[p.blayer[b]].kind == PT_LAYER_DISK;
-    const pt_ca_cuts rg = p.region[disk ? 1 : 0];
-    const float tol = p.region_tol[disk ? 1 : 0];
+    if (ns == 0) return s;
+    s.B = load_hit(p.bh, b);
+    s.C = load_hit(p.bh, c);
+    s.disk = p.layer[p.blayer[b]].kind == PT_LAYER_DISK;
+    const float tol = s.disk ? p.region_tol[1] : p.region_tol[0];
     const float4 hk = p.hk[b];
-    const float dr = C.r - B.r, dz = C.z - B.z;
-    const float num = disk ? dr : dz, den = disk ? dz : dr;
-    const float key_c = den != 0.f ? num / den : __int_as_float(0x7f800000);
+    const float dr = s.C.r - s.B.r, dz = s.C.z - s.B.z;
+    const float num = s.disk ? dr : dz, den = s.disk ? dz : dr;
+    s.key_c = den != 0.f ? num / den : __int_as_float(0x7f800000);
     // window half-width, widened for float32 rounding of the keys
-    float wdt = tol * (hk.x / fabsf(den) + sqrtf(1.0f + key_c * key_c) / hk.y);
-    wdt = wdt * (1.0f + 1e-5f) + 1e-5f * (1.0f + fabsf(key_c) + hk.x);
+    float wdt = tol * (hk.x / fabsf(den) + sqrtf(1.0f + s.key_c * s.key_c) / hk.y);
+    wdt = wdt * (1.0f + 1e-5f) + 1e-5f * (1.0f + fabsf(s.key_c) + hk.x);
     if (!(wdt == wdt) || den == 0.f) wdt = __int_as_float(0x7f800000);
+    s.wdt = wdt;
     // keys passing the window test lie in [lo, hi]
-    const float sl = (fabsf(key_c) + wdt) * 9.5367431640625e-7f;
-    const float lo = key_c - wdt - sl;
-    float hi = key_c + wdt + sl;
+    const float sl = (fabsf(s.key_c) + wdt) * 9.5367431640625e-7f;
+    const float lo = s.key_c - wdt - sl;
+    float hi = s.key_c + wdt + sl;
     if (!(hi == hi)) hi = __int_as_float(0x7f800000);
     // the cells are ordered by a bucket of their key, monotone in the key:
     // the run searched is that of the buckets of [lo, hi]
-    const float2 *S = p.sk + b0;
     const int nb = sk_buckets(ns);
-    const int bhi = sk_bucket(hi, hk.z, hk.w, nb);
-    const float fend = bhi < nb - 1 ? (float)(bhi + 1) : __int_as_float(0x7f800000);
+    const int blo = sk_bucket(lo, hk.z, hk.w, nb), bhi = sk_bucket(hi, hk.z, hk.w, nb);
+    if (ns <= kSkEnds) {
+        const uint16_t *E = p.sk_end + b0;
+        const int sh = sk_end_shift(ns), e0 = blo >> sh;
+        s.r = e0 > 0 ? __ldg(E + e0 - 1) : 0;
+        s.end = __ldg(E + (bhi >> sh));
+    } else {
+        const float2 *S = p.sk + b0;
+        s.r = lower_bucket(S, ns, blo, hk.z, hk.w);
+        s.end = bhi < nb - 1 ? lower_bucket(S, ns, bhi + 1, hk.z, hk.w) : ns;
+    }
+    s.r += (int32_t)b0;
+    s.end += (int32_t)b0;
+    return s;
+}
+
+// an entry passes the window (inner hit -1: a dead cell)
+__device__ __forceinline__ bool in_window(const float2 &e, float key_c, float wdt) {
+    return fabsf(e.x - key_c) <= wdt && __float_as_int(e.y) >= 0;
+}
+
+// Every inner cell (a,b) connecting to the live cell x = (b,c), one after the
+// other in the order of b's bucket-ordered arrays: emit(t, i) for the t-th
+// one, i its index there.  Returns their number.
+template <bool kExact, class Emit>
+__device__ __forceinline__ int scan_cell(const Params &p, int x, Emit &&emit) {
+    const Search s = search_of(p, p.cell_inner[x], p.cell_outer[x]);
     int n = 0;
-    for (int r = lower_bucket(S, ns, sk_bucket(lo, hk.z, hk.w, nb), hk.z, hk.w); r < ns; r++) {
-        const float2 e = __ldg(S + r);
-        if (sk_coord(e.x, hk.z, hk.w) >= fend) break;     // a bucket above hi's
-        if (!(fabsf(e.x - key_c) <= wdt) || __float_as_int(e.y) < 0) continue;      // (-1: a dead cell)
-        const int v = connects<kExact>(p, __ldg(p.bh + __float_as_int(e.y)), B, C, rg);
-        if (v == 2) return -2;
-        if (v) emit(n++, b0 + r);
+    for (int k = s.r; k < s.end; k++) {
+        const float2 e = __ldg(p.sk + k);
+        if (!in_window(e, s.key_c, s.wdt)) continue;
+        if (connects<kExact>(p, __ldg(p.bh + __float_as_int(e.y)), s.B, s.C, p.region[s.disk ? 1 : 0]) == 1)
+            emit(n++, k);
     }
     return n;
 }
 
-__global__ void __launch_bounds__(32 * kCaWarps, 10) k_connect(Params p) {
+// Per warp: the cells of a chunk to search, the searches of up to 32 of them,
+// and the edges found.
+struct __align__(16) CaWarp {
+    FHit B[32], C[32];
+    float4 own[32];                  // key, half-width; as ints, entry minus flat index, and position | disk << 8
+    int32_t cand[3][64];             // candidates that passed the window: entry, inner hit, search
+    int32_t b[kCaPer], c[kCaPer];    // cells to search: inner and outer hit,
+    uint8_t pos[kCaPer];             //   position in the chunk
+    uint8_t acc_pos[kCaAcc];         // edges found, by position: position of the cell,
+    int32_t acc[kCaAcc];             //   entry of the inner cell
+    uint32_t und[kCaChunk];          // positions left to the exact pass
+};
+
+// Writes the na edges found, and the edge ranges of their cells: one
+// reservation.  With last = false the cell of the last edge may have more to
+// come, so its edges stay; if there are none but those, the cell is left to
+// the exact pass (which takes any number).  Returns how many stay.
+__device__ __noinline__ int write_edges(const Params &p, CaWarp &sm, int64_t x0, int na, bool last, int lane) {
+    const unsigned below = (1u << lane) - 1u;
+    // drop the edges of cells left to the exact pass (rare)
+    if (__any_sync(0xffffffffu, lane < kCaChunk && sm.und[lane] != 0)) {
+        int n = 0;
+        for (int i0 = 0; i0 < na; i0 += 32) {
+            const int i = i0 + lane;
+            const int pos = i < na ? sm.acc_pos[i] : 0, k = i < na ? sm.acc[i] : 0;
+            const bool keep = i < na && !((sm.und[pos >> 5] >> (pos & 31)) & 1);
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) {
+                sm.acc_pos[n + __popc(m & below)] = (uint8_t)pos;
+                sm.acc[n + __popc(m & below)] = k;
+            }
+            n += __popc(m);
+            __syncwarp();
+        }
+        na = n;
+        if (na == 0) return 0;
+    }
+    int stay = 0;
+    if (!last) {
+        const int pos = sm.acc_pos[na - 1];
+        for (int i = lane; i < na; i += 32) stay += sm.acc_pos[i] == pos;
+        stay = __reduce_add_sync(0xffffffffu, stay);
+        if (stay == na) {
+            if (na + 32 <= kCaAcc) return na;
+            __syncwarp();
+            if (lane == 0) sm.und[pos >> 5] |= 1u << (pos & 31);
+            __syncwarp();
+            return 0;
+        }
+    }
+    const int n = na - stay;
+    int64_t base = 0;
+    if (lane == 0) {
+        base = atomicAdd(p.counters + C_EDGES, n);
+        if (base + n > p.cap_edges) set_flag(p.counters, PT_FLAG_EDGES);
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int i = lane; i < n; i += 32) {
+        const int pos = sm.acc_pos[i];
+        const int ci = __ldg(p.sci + sm.acc[i]);
+        if (base + i < p.cap_edges) {
+            p.edge_src[base + i] = ci;
+            p.edge_dst[base + i] = (int32_t)(x0 + pos);
+        }
+        p.has_out[ci] = 1;
+        if (i == 0 || sm.acc_pos[i - 1] != pos) {
+            int e = i + 1;
+            while (e < n && sm.acc_pos[e] == pos) e++;
+            p.edge_rng[x0 + pos] = make_int2((int32_t)(base + i), e - i);
+        }
+    }
+    for (int i0 = 0; i0 < stay; i0 += 32) {
+        const int i = i0 + lane;
+        const int pos = i < stay ? sm.acc_pos[n + i] : 0, k = i < stay ? sm.acc[n + i] : 0;
+        __syncwarp();
+        if (i < stay) {
+            sm.acc_pos[i] = (uint8_t)pos;
+            sm.acc[i] = k;
+        }
+        __syncwarp();
+    }
+    return stay;
+}
+
+// the predicates on candidates 0..n-1 <= 32, a lane each; those that connect
+// join the edges found
+__device__ __forceinline__ int test_candidates(const Params &p, CaWarp &sm, int64_t x0, int n, int na, int lane) {
+    while (na + 32 > kCaAcc) na = write_edges(p, sm, x0, na, false, lane);
+    int v = 0, k = 0, pos = 0;
+    if (lane < n) {
+        const int i = sm.cand[2][lane];
+        const float4 a = __ldg(p.bh + sm.cand[1][lane]);
+        k = sm.cand[0][lane];
+        const int at = __float_as_int(sm.own[i].w);
+        pos = at & 255;
+        v = connects<false>(p, a, sm.B[i], sm.C[i], p.region[at >> 8]);
+        if (v == 2) atomicOr(&sm.und[pos >> 5], 1u << (pos & 31));
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, v == 1);
+    if (v == 1) {
+        const int t = na + __popc(m & ((1u << lane) - 1u));
+        sm.acc[t] = k;
+        sm.acc_pos[t] = (uint8_t)pos;
+    }
+    __syncwarp();
+    return na + __popc(m);
+}
+
+__global__ void __launch_bounds__(32 * kCaWarps, 12) k_connect(Params p) {
     pdl_enter();
-    constexpr int kPer = 32 * kCaChunk;
-    __shared__ int32_t s_q[kCaWarps][kCaQueue][kPer];   // accepted inner cells per chunk position
-    __shared__ int32_t s_m[kCaWarps][kPer];             // edges per chunk position (-1: no live cell,
-                                                        //   -2: a cell that can have no incoming edge)
-    __shared__ int16_t s_list[kCaWarps][kPer];          // positions whose inner hit has live cells
+    __shared__ CaWarp s_warp[kCaWarps];
+    __shared__ uint8_t s_inner_is_outer[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
+    if (threadIdx.x < PT_MAX_PAIRS) s_inner_is_outer[threadIdx.x] = p.pair_inner_is_outer[threadIdx.x];
+    __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    CaWarp &sm = s_warp[w];
     const unsigned below = (1u << lane) - 1u;
     const int64_t n_cells = min((int64_t)p.counters[C_CELLS], p.cap_cells);
-    const int n_chunks = (int)((n_cells + kPer - 1) / kPer);
+    const int n_chunks = (int)((n_cells + kCaPer - 1) / kCaPer);
     // the warps take the chunks in order from a queue: the chunks in flight
     // are neighbours, and so are the middle hits whose sorted cells they read
     for (;;) {
@@ -179,97 +329,103 @@ __global__ void __launch_bounds__(32 * kCaWarps, 10) k_connect(Params p) {
         if (lane == 0) ch = atomicAdd(p.counters + C_CA_NEXT, 1);
         ch = __shfl_sync(0xffffffffu, ch, 0);
         if (ch >= n_chunks) break;
-        const int64_t x0 = (int64_t)ch * kPer;
-        // 1) live cells, and a list of those with candidates at all (the
-        //    inner hit has live cells ending on it), so that the searches
-        //    run on full warps
+        const int64_t x0 = (int64_t)ch * kCaPer;
+        // 1) the live cells whose inner hit can have cells ending on it (no
+        //    cell ends on a layer that is the outer layer of no pair; most
+        //    cells start on BPix1: no edge range is written for them, and the
+        //    search records read none), so that the searches run on full warps
         int nlist = 0;
-        unsigned ranged = 0;     // lanes with a cell whose edge range is written
+        if (lane < kCaChunk) sm.und[lane] = 0;
 #pragma unroll
         for (int it = 0; it < kCaChunk; it++) {
             const int pos = it * 32 + lane;
             const int64_t x = x0 + pos;
-            int st = -1;
-            bool need = false;
-            if (x < n_cells && p.cell_alive[x]) {
-                // no cell ends on an inner hit on a layer that is the outer
-                // layer of no pair (most cells start on BPix1): such a cell
-                // has no incoming edges, and no edge range is written for
-                // it (-2; the search records read none)
-                st = -2;
-                if (p.pair_inner_is_outer[p.cell_pair[x]]) {
-                    st = 0;
-                    need = p.in_live[p.cell_inner[x]] > 0;
-                }
-            }
-            s_m[w][pos] = st;
-            ranged |= __ballot_sync(0xffffffffu, st >= 0);
+            const bool need = x < n_cells && p.cell_alive[x] && s_inner_is_outer[p.cell_pair[x]];
             const unsigned m = __ballot_sync(0xffffffffu, need);
-            if (need) s_list[w][nlist + __popc(m & below)] = (int16_t)pos;
+            if (need) {
+                const int i = nlist + __popc(m & below);
+                sm.b[i] = p.cell_inner[x];
+                sm.c[i] = p.cell_outer[x];
+                sm.pos[i] = (uint8_t)pos;
+                p.edge_rng[x] = make_int2(0, 0);
+            }
             nlist += __popc(m);
         }
-        // a chunk of cells that can have no incoming edge (the cells of
-        // outer hits on BPix2 all start on BPix1) has nothing more to do
-        if (!ranged) continue;
+        if (nlist == 0) continue;
         __syncwarp();
         // 2) the searches
-        for (int i = lane; i < nlist; i += 32) {
-            const int pos = s_list[w][i];
-            int m = scan_cell<false>(p, (int)(x0 + pos), [&](int t, int64_t k) {
-                if (t < kCaQueue) s_q[w][t][pos] = p.sci[k];
-            });
-            if (m == -2) {   // undecided: left to the exact pass
-                const int k = atomicAdd(p.counters + C_CA_PENDING, 1);
-                if (k < p.cap_cells) reinterpret_cast<int32_t *>(p.ck)[k] = (int32_t)(x0 + pos);
-                else set_flag(p.counters, PT_FLAG_CELLS);
-                m = -1;
+        int na = 0;
+        for (int i0 = 0; i0 < nlist; i0 += 32) {
+            Search se;
+            int cnt = 0, pos = 0;
+            if (i0 + lane < nlist) {
+                pos = sm.pos[i0 + lane];
+                se = search_of(p, sm.b[i0 + lane], sm.c[i0 + lane]);
+                cnt = se.end - se.r;
             }
-            s_m[w][pos] = m;
-        }
-        __syncwarp();
-        // 3) edges of the chunk: one reservation, then each cell's edges
-        //    contiguously and its edge range
-        int tot = 0;
-#pragma unroll
-        for (int it = 0; it < kCaChunk; it++) tot += max(s_m[w][it * 32 + lane], 0);
-        int total;
-        const int excl = warp_excl(tot, lane, total);
-        int64_t base = 0;
-        if (lane == 0 && total > 0) base = atomicAdd(p.counters + C_EDGES, total);
-        base = __shfl_sync(0xffffffffu, base, 0) + excl;
-#pragma unroll 1
-        for (int it = 0; it < kCaChunk; it++) {
-            const int pos = it * 32 + lane;
-            const int64_t x = x0 + pos;
-            const int m = s_m[w][pos];
-            if (m < 0) continue;
-            if (m > 0) {
-                if (m <= kCaQueue) {
-                    for (int t = 0; t < m; t++) {
-                        const int ci = s_q[w][t][pos];
-                        if (base + t < p.cap_edges) {
-                            p.edge_src[base + t] = ci;
-                            p.edge_dst[base + t] = (int32_t)x;
-                        }
-                        p.has_out[ci] = 1;
-                    }
-                } else {   // rare: scan again to write them all
-                    const int64_t e0 = base;
-                    scan_cell<false>(p, (int)x, [&](int t, int64_t k) {
-                        const int ci = p.sci[k];
-                        if (e0 + t < p.cap_edges) {
-                            p.edge_src[e0 + t] = ci;
-                            p.edge_dst[e0 + t] = (int32_t)x;
-                        }
-                        p.has_out[ci] = 1;
-                    });
+            int total;
+            const int excl = warp_excl(cnt, lane, total);
+            const unsigned some = __ballot_sync(0xffffffffu, cnt > 0);
+            if (cnt > 0) {
+                const int i = __popc(some & below);
+                sm.B[i] = se.B;
+                sm.C[i] = se.C;
+                sm.own[i] = make_float4(se.key_c, se.wdt, __int_as_float(se.r - excl),
+                                        __int_as_float(pos | (se.disk ? 256 : 0)));
+            }
+            __syncwarp();
+            int nq = 0, before = -1;
+            for (int f = 0; f < total; f += 32) {
+                // the search that flat entry f + lane belongs to: the last one starting at or before it
+                const unsigned at = (unsigned)(excl - f);
+                const unsigned starts = __reduce_or_sync(0xffffffffu, cnt > 0 && at < 32u ? 1u << at : 0u);
+                const int i = before + __popc(starts & (below | (1u << lane)));
+                before += __popc(starts);
+                bool pass = false;
+                int k = 0, inner = 0;
+                if (f + lane < total) {
+                    const float4 o = sm.own[i];
+                    k = __float_as_int(o.z) + f + lane;
+                    const float2 e = __ldg(p.sk + k);
+                    inner = __float_as_int(e.y);
+                    pass = in_window(e, o.x, o.y);
                 }
-                if (base + m > p.cap_edges) set_flag(p.counters, PT_FLAG_EDGES);
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                if (pass) {
+                    const int c = nq + __popc(m & below);
+                    sm.cand[0][c] = k;
+                    sm.cand[1][c] = inner;
+                    sm.cand[2][c] = i;
+                }
+                nq += __popc(m);
+                __syncwarp();
+                const bool end = f + 32 >= total;
+                while (nq >= 32 || (end && nq > 0)) {
+                    na = test_candidates(p, sm, x0, min(nq, 32), na, lane);
+                    nq = max(nq - 32, 0);
+                    if (lane < nq) {
+#pragma unroll
+                        for (int c = 0; c < 3; c++) sm.cand[c][lane] = sm.cand[c][32 + lane];
+                    }
+                    __syncwarp();
+                }
             }
-            p.edge_rng[x] = make_int2((int32_t)base, m);
-            base += m;
         }
+        // 3) their edges
+        if (na > 0) write_edges(p, sm, x0, na, true, lane);
         __syncwarp();
+        // cells with an undecided candidate: left to the exact pass
+        if (__any_sync(0xffffffffu, lane < kCaChunk && sm.und[lane] != 0)) {
+#pragma unroll 1
+            for (int it = 0; it < kCaChunk; it++) {
+                if ((sm.und[it] >> lane) & 1) {
+                    const int k = atomicAdd(p.counters + C_CA_PENDING, 1);
+                    if (k < p.cap_cells) reinterpret_cast<int32_t *>(p.ck)[k] = (int32_t)(x0 + it * 32 + lane);
+                    else set_flag(p.counters, PT_FLAG_CELLS);
+                }
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -284,9 +440,9 @@ __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
     // warp seldom holds two cells whose exact fallbacks would run in turn
     for (int k = threadIdx.x * gridDim.x + blockIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int x = list[k];
-        const int m = scan_cell<true>(p, x, [](int, int64_t) {});
+        const int m = scan_cell<true>(p, x, [](int, int) {});
         const int64_t base = m > 0 ? atomicAdd(p.counters + C_EDGES, m) : 0;
-        scan_cell<true>(p, x, [&](int t, int64_t i) {
+        scan_cell<true>(p, x, [&](int t, int i) {
             const int ci = p.sci[i];
             if (base + t < p.cap_edges) {
                 p.edge_src[base + t] = ci;
@@ -302,7 +458,7 @@ __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
 void launch_connect(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_connect", s);
-        launch_pdl(k_connect, g.blocks(10), 32 * kCaWarps, 0, s, p);
+        launch_pdl(k_connect, g.blocks(12), 32 * kCaWarps, 0, s, p);
     }
     KernelTimer t("k_connect_exact", s);
     launch_pdl(k_connect_exact, g.blocks(4), 128, 0, s, p);

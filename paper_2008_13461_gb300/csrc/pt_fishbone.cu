@@ -21,7 +21,7 @@
 // The same pass prepares the CA connection: it writes the cells of o ordered
 // by a bucket of their R-z slope key relative to o (with the inner hit, -1
 // for a dead cell, and the cell index; the bucket is monotone in the key,
-// about one cell per bucket, free order inside), the bucket parameters, and
+// about one cell per bucket, free order inside), the ends of those buckets, the bucket parameters, and
 // per hit the bounds the slope window needs (over all cells of o).  Both sorts
 // are done at once: their counters share 32-bit words, so one clearing, one
 // scan and one loop over the cells each for counting and placing serve both.
@@ -132,6 +132,7 @@ template <int M, int NB, bool C, bool kExact>
 __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64_t b, int lane, float unit_thr,
                                             float du, FbWarp<M, NB, C> &sm, const uint8_t *slot) {
     // NB: at least the buckets of M cells (sk_buckets)
+    static_assert(M <= kSkEnds, "the connection expects the ends of the buckets");
     static_assert(NB >= 32 && NB >= M && (NB & (NB - 1)) == 0, "bucket array too small");
     const float4 ho = __ldg(p.bh + o);
     const int Lo = p.blayer[o];
@@ -259,6 +260,11 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
             p.sk[q] = make_float2(C ? sm.ck[j] : p.ck[b + j], __int_as_float(dead ? -1 : p.cell_inner[b + j]));
             p.sci[q] = (int32_t)(b + j);
         }
+    }
+    // where the connection starts and ends its searches
+    if (starts) {
+        const int sh = sk_end_shift(n);
+        for (int e = lane; e < sk_ends(n); e += 32) p.sk_end[b + e] = sm.pos[((e + 1) << sh) - 1] >> 16;
     }
     if (lane == 0) p.in_live[o] = n;       // (never all dead: the shortest of them lives)
     __syncwarp();
