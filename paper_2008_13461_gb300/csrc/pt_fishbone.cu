@@ -5,7 +5,7 @@
 // aligned as seen from o form a fishbone; every cell of it dies except the
 // shortest (equal lengths: the smaller input index of the inner hit wins).
 //
-// One warp per outer hit.  The warp keeps, per cell, the difference vector
+// A team of one or more warps per outer hit.  It keeps, per cell, the difference vector
 // u = h_inner - h_o in shared memory; hits are multiples of 2^-14 below 64 in
 // magnitude, so u is exact in float32 and the alignment test and the squared
 // length (an integer in grid units) are evaluated from it with no further
@@ -27,41 +27,46 @@
 // scan and one loop over the cells each for counting and placing serve both.
 //
 // What bounds it is the work in shared memory and the instructions around
-// it.  For 64 PU200 events (small and medium warps) 2.84 + 0.75 ms; with the
+// it.  For 64 PU200 events the hits of up to 184 cells took 2.84 ms; with the
 // scan's 16-byte accesses (its entries met in a few banks: half of the
-// kernel's shared-memory cycles) 2.69 + 0.70 ms; with both sorts at once and
-// up to two direction buckets per cell 2.19 + 0.78 ms; 24 events with pT > 0.3
-// GeV 0.84 + 1.17 + 0.52 ms (small, medium, large) to 0.67 + 0.92 + 0.36 ms; 32
-// PU50 events 193 to 151 us.  A dead cell is marked with a byte store: the same
-// with an atomicOr of a bit, in a branch that single lanes take, costs
-// 0.77 ms; so does a list of the close pairs for later, 0.2 ms.
+// kernel's shared-memory cycles) 2.69; with both sorts at once and
+// up to two direction buckets per cell 2.19.  A dead cell is marked with a byte
+// store: the same with an atomicOr of a bit, in a branch that single lanes
+// take, costs 0.77 ms; so does a list of the close pairs for later, 0.2 ms; so do
+// the pairs laid end to end with full warps of them (0.2 to 0.3 ms: a pair per
+// lane has to find its two cells, which costs what the idle lanes cost).
 //
-// Shared memory per warp bounds the siblings it can hold, and the warps an
-// SM can keep resident bound how well the gathers of the inner hits are
-// hidden.  Most outer hits have fewer than ~180 cells, so three launches
-// share the work: many small warps take chunks of outer hits from a queue
-// and list the outer hits with more cells, which medium (up to 320 cells)
-// and large warps (up to 512) then take one at a time; an exact pass takes
-// the rest (undecided tests, more cells), sorted in shared memory like the
-// others up to 1024 cells, which pT > 0.3 GeV events reach (0.2% of their
-// hits), with a pairwise loop over global memory beyond: that loop from 512
-// cells on took 2.15 of the 8.8 ms of a batch of 24 such events, against
-// 0.07 ms now.
+// The cells of an outer hit sit in shared memory while its team works on them,
+// so the shared memory per hit bounds how many hits an SM holds, and
+// the warps per hit how many warps hide the gathers' latency and how long a
+// hit takes.  Most outer hits have few cells, so three launches share the
+// work: one warp per hit up to 128 cells (256 buckets, 40 warps per SM),
+// taking chunks of outer hits from a queue and listing the others for two
+// warps (up to 288 cells, 40 warps per SM) and four warps per hit (up to 512,
+// 36); an exact pass of eight takes the rest (undecided tests, more
+// cells), sorted in shared memory like the others up to 1024 cells, which
+// pT > 0.3 GeV events reach (0.2% of their hits), with a pairwise loop over
+// global memory beyond.  With one warp per hit throughout (up to 184, 320 and
+// 512 cells; 32, 24 and 12 warps per SM) the four kernels took 2.25 + 0.79 +
+// 0.05 + 0.04 ms for 64 PU200 events, now 1.21 + 1.41 + 0.05 + 0.02; 0.68 + 0.93
+// + 0.36 + 0.07 for 24 events with pT > 0.3 GeV, now 0.42 + 0.76 + 0.37 + 0.02;
+// 62 + 57 + 42 + 17 us for one PU200 event, whose few large hits are a wait for
+// the slowest team, now 47 + 48 + 19 + 13; 158 us for 32 PU50 events, now 146.
+// Limits of 64 or 96 cells for one warp take 8% and 3% longer in all; 256 or 320
+// cells for two warps 2% (more hits of 257 or more for four; fewer hits per SM).
 #include "pt_common.cuh"
 #include "pt_kernels.cuh"
 
 namespace ptk {
 
-// Per warp: the cells of one outer hit (up to M) and NB bucket counters, whose
+// Per team: the cells of one outer hit (up to M) and NB bucket counters, whose
 // low halves count the cells by direction key and whose high halves by
 // R-z slope key, so that one scan serves both sorts.
-// C: the slope keys are kept here (else written to and read back from global
-// memory, for warps whose cells would not fit otherwise).
-template <int M, int NB, bool C>
-struct __align__(16) FbWarp {
+template <int M, int NB>
+struct __align__(16) FbCells {
     float4 rec[M];                   // u = h_inner - h_o (exact), 1/|u| in w
     uint32_t pos[NB];                // counts, then starts, then ends
-    float ck[C ? M : 1];             // R-z slope key
+    float ck[M];                     // R-z slope key
     uint32_t meta[M];                // slot; then direction bucket and, in the high half, slope bucket and then place
     uint16_t idx[M];                 // cells sorted by direction bucket
     uint8_t dead[M];
@@ -103,14 +108,69 @@ __device__ __forceinline__ float warp_min(float f) { return fval(__reduce_min_sy
 __device__ __forceinline__ float warp_max(float f) { return fval(__reduce_max_sync(0xffffffffu, ford(f))); }
 __device__ __forceinline__ int warp_sum(int v) { return __reduce_add_sync(0xffffffffu, v); }
 
+// The T warps that work on one outer hit: a warp of a block of several, or
+// (T > 1) a block.
+template <int T>
+__device__ __forceinline__ void team_sync() {
+    if (T == 1) __syncwarp();
+    else __syncthreads();
+}
+
+// The direction key's and the slope key's ranges and bounds, reduced over a
+// team (part: shared, for T > 1).
+struct FbRange {
+    float bmin, bmax, smin, smax, k2max, gmin;
+};
+
+template <int T>
+__device__ __forceinline__ FbRange team_range(FbRange v, bool starts, FbRange *part) {
+    v.bmin = warp_min(v.bmin);
+    v.bmax = warp_max(v.bmax);
+    if (starts) {
+        v.k2max = warp_max(v.k2max);
+        v.gmin = warp_min(v.gmin);
+        v.smin = warp_min(v.smin);
+        v.smax = warp_max(v.smax);
+    }
+    if (T > 1) {
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < T; w++) {
+            const FbRange q = part[w];
+            v.bmin = fminf(v.bmin, q.bmin);
+            v.bmax = fmaxf(v.bmax, q.bmax);
+            v.smin = fminf(v.smin, q.smin);
+            v.smax = fmaxf(v.smax, q.smax);
+            v.k2max = fmaxf(v.k2max, q.k2max);
+            v.gmin = fminf(v.gmin, q.gmin);
+        }
+    }
+    return v;
+}
+
 // exclusive prefix sums of both halves of a[0, nb) in place (nb a power of two >= 32; one
-// warp): 128 entries at a time, four per lane in one 16-byte access.  (Entries
+// team): 128 entries at a time, four per lane in one 16-byte access.  (Entries
 // lane * nb / 32 + q, one after the other, met in 2 to 4 banks: half of the
-// kernel's shared-memory cycles were those conflicts.)
-__device__ __forceinline__ void warp_exclusive_scan(uint32_t *a, int nb, int lane) {
+// kernel's shared-memory cycles were those conflicts.)  Each warp of a team
+// adds up the entries before its share first.
+template <int T>
+__device__ __forceinline__ void team_exclusive_scan(uint32_t *a, int nb, int lane) {
+    int q0 = 0, q1 = nb;
     uint32_t carry = 0;
-    for (int q = 4 * lane; q - 4 * lane < nb; q += 128) {
-        uint4 v = q < nb ? *reinterpret_cast<const uint4 *>(a + q) : make_uint4(0, 0, 0, 0);
+    if (T > 1) {
+        const int w = threadIdx.x >> 5, share = max(128, nb / T);
+        q0 = min(w * share, nb);
+        q1 = min(q0 + share, nb);
+        for (int q = 4 * lane; q < q0; q += 128) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(a + q);
+            carry += (v.x + v.y) + (v.z + v.w);
+        }
+        carry = __reduce_add_sync(0xffffffffu, carry);     // (halves below 2^16: no more than the cells)
+        __syncthreads();
+    }
+    for (int q = q0 + 4 * lane; q - 4 * lane < q1; q += 128) {
+        uint4 v = q < q1 ? *reinterpret_cast<const uint4 *>(a + q) : make_uint4(0, 0, 0, 0);
         const uint32_t sum = (v.x + v.y) + (v.z + v.w);
         uint32_t incl = sum;
 #pragma unroll
@@ -121,16 +181,16 @@ __device__ __forceinline__ void warp_exclusive_scan(uint32_t *a, int nb, int lan
         const uint32_t e = carry + incl - sum;
         carry += __shfl_sync(0xffffffffu, incl, 31);
         v = make_uint4(e, e + v.x, e + v.x + v.y, e + v.x + v.y + v.z);
-        if (q < nb) *reinterpret_cast<uint4 *>(a + q) = v;
+        if (q < q1) *reinterpret_cast<uint4 *>(a + q) = v;
     }
 }
 
-// Verdicts of the n <= M cells of outer hit o (one warp); returns the lane's
-// count of live cells.  kExact = false (float32 filters only): returns -1,
+// Verdicts of the n <= M cells of outer hit o (one team; t: thread of it); returns the
+// thread's count of live cells.  kExact = false (float32 filters only): returns -1,
 // having written no verdict, when an alignment test is undecided.
-template <int M, int NB, bool C, bool kExact>
-__device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64_t b, int lane, float unit_thr,
-                                            float du, FbWarp<M, NB, C> &sm, const uint8_t *slot) {
+template <int T, int M, int NB, bool kExact>
+__device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64_t b, int t, float unit_thr,
+                                            float du, FbCells<M, NB> &sm, FbRange *part, const uint8_t *slot) {
     // NB: at least the buckets of M cells (sk_buckets)
     static_assert(M <= kSkEnds, "the connection expects the ends of the buckets");
     static_assert(NB >= 32 && NB >= M && (NB & (NB - 1)) == 0, "bucket array too small");
@@ -145,9 +205,9 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
     // pass 1: records, direction keys' range, and the R-z slope keys (barrel
     // o: (z_o - z_a)/(r_o - r_a); disk o: (r_o - r_a)/(z_o - z_a)) with the
     // per-hit bounds and their range
-    float k2max = 0.f, gmin = 3.0e38f, bmin = 3.0f, bmax = -3.0f;
-    float smin = __int_as_float(0x7f800000), smax = -smin;
-    for (int j = lane; j < n; j += 32) {
+    const float inf = __int_as_float(0x7f800000);
+    FbRange rg = {3.0f, -3.0f, inf, -inf, 0.f, 3.0e38f};
+    for (int j = t; j < n; j += 32 * T) {
         const float4 a = __ldg(p.bh + p.cell_inner[b + j]);
         sm.meta[j] = slot[p.cell_pair[b + j]];
         sm.dead[j] = 0;
@@ -157,24 +217,23 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
             // the key only places the cell in the connection's search window,
             // whose margins (1e-5 relative) are far above the 2 ulp of this quotient
             const float ck = den != 0.f ? __fdividef(num, den) : __int_as_float(0x7f800000);
-            k2max = fmaxf(k2max, ck * ck);
-            gmin = fminf(gmin, fabsf(den));
-            if (C) sm.ck[j] = ck;
-            else p.ck[b + j] = ck;
+            rg.k2max = fmaxf(rg.k2max, ck * ck);
+            rg.gmin = fminf(rg.gmin, fabsf(den));
+            sm.ck[j] = ck;
             if (fabsf(ck) <= 3.4e38f) {
-                smin = fminf(smin, ck);
-                smax = fmaxf(smax, ck);
+                rg.smin = fminf(rg.smin, ck);
+                rg.smax = fmaxf(rg.smax, ck);
             }
         }
         const float ux = a.x - ho.x, uy = a.y - ho.y, uz = a.z - ho.z;
         const float4 r = make_float4(ux, uy, uz, rsqrtf(ux * ux + uy * uy + uz * uz));
         sm.rec[j] = r;
         const float key = fb_key(r, disk, rx, ry);
-        bmin = fminf(bmin, key);
-        bmax = fmaxf(bmax, key);
+        rg.bmin = fminf(rg.bmin, key);
+        rg.bmax = fmaxf(rg.bmax, key);
     }
-    bmin = warp_min(bmin);
-    bmax = warp_max(bmax);
+    rg = team_range<T>(rg, starts, part);
+    const float bmin = rg.bmin, bmax = rg.bmax, smin = rg.smin, smax = rg.smax;
     // Direction buckets: each inner layer of o has its own aligned range of
     // nbr buckets (one or two buckets per cell), so a cell meets only siblings
     // on its own layer.  Two keys within du lie at most K buckets apart (K
@@ -187,45 +246,41 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
     const int K = (int)fminf(du * iw + 6e-4f, (float)nbr) + 1;
     float siw = 0.f;
     if (starts) {
-        k2max = warp_max(k2max);
-        gmin = warp_min(gmin);
-        smin = warp_min(smin);
-        smax = warp_max(smax);
         const float sspan = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
         siw = sspan > 0.f && sspan <= 3.4e38f ? (float)nbs / sspan : 0.f;
         // bound of sqrt(1 + key^2), smallest gap, lowest key, inverse width
-        if (lane == 0) p.hk[o] = make_float4(sqrtf(1.0f + k2max), gmin, smin, siw);
+        if (t == 0) p.hk[o] = make_float4(sqrtf(1.0f + rg.k2max), rg.gmin, smin, siw);
     }
-    for (int q = lane; q < nb; q += 32) sm.pos[q] = 0;
-    __syncwarp();
-    for (int j = lane; j < n; j += 32) {
+    for (int q = t; q < nb; q += 32 * T) sm.pos[q] = 0;
+    team_sync<T>();
+    for (int j = t; j < n; j += 32 * T) {
         const float key = fb_key(sm.rec[j], disk, rx, ry);
         uint32_t m = sm.meta[j] * nbr + min(max((int)((key - bmin) * iw), 0), nbr - 1);
         atomicAdd(&sm.pos[m], 1u);
         if (starts) {
-            const uint32_t bs = sk_bucket(C ? sm.ck[j] : p.ck[b + j], smin, siw, nbs);
+            const uint32_t bs = sk_bucket(sm.ck[j], smin, siw, nbs);
             atomicAdd(&sm.pos[bs], 1u << 16);
             m |= bs << 16;
         }
         sm.meta[j] = m;
     }
-    __syncwarp();
-    warp_exclusive_scan(sm.pos, nb, lane);
-    __syncwarp();
-    for (int j = lane; j < n; j += 32) {
+    team_sync<T>();
+    team_exclusive_scan<T>(sm.pos, nb, t & 31);
+    team_sync<T>();
+    for (int j = t; j < n; j += 32 * T) {
         const uint32_t m = sm.meta[j];
         sm.idx[atomicAdd(&sm.pos[m & 0xffffu], 1u) & 0xffffu] = (uint16_t)j;
         if (starts)
             sm.meta[j] = (m & 0xffffu) | (atomicAdd(&sm.pos[m >> 16], 1u << 16) & 0xffff0000u);
     }
-    __syncwarp();
+    team_sync<T>();
     // sm.pos[bk] now holds the ends of bucket bk.  Each pair once: every cell
     // against the cells after it in its own bucket and the next K buckets of
     // its layer (a superset of its siblings within du of its key); of an
     // aligned pair the longer cell dies (equal lengths: the larger input
     // index of the inner hit).
     bool und = false;
-    for (int q0 = lane; q0 < n; q0 += 32) {
+    for (int q0 = t; q0 < n; q0 += 32 * T) {
         const int j = sm.idx[q0];
         const float4 r1 = sm.rec[j];
         const float3 v1 = make_float3(r1.x * r1.w, r1.y * r1.w, r1.z * r1.w);
@@ -244,45 +299,51 @@ __device__ __forceinline__ int fishbone_hit(const Params &p, int o, int n, int64
             sm.dead[j_wins ? d : j] = 1;
         }
     }
-    __syncwarp();
-    if (!kExact && __any_sync(0xffffffffu, und)) return -1;
+    if (T == 1) {
+        __syncwarp();
+        und = __any_sync(0xffffffffu, und);
+    } else {
+        und = __syncthreads_or(und);
+    }
+    if (!kExact && und) return -1;
 
     // pass 2: the verdicts, and the cells grouped by slope-key bucket for the
     // CA connection, a dead one with the inner hit -1 (any order inside a
     // bucket: the connection searches by bucket)
     int alive = 0;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = t; j < n; j += 32 * T) {
         const bool dead = sm.dead[j];
         if (dead) p.cell_alive[b + j] = 0;
         else alive++;
         if (starts) {
             const int64_t q = b + (sm.meta[j] >> 16);
-            p.sk[q] = make_float2(C ? sm.ck[j] : p.ck[b + j], __int_as_float(dead ? -1 : p.cell_inner[b + j]));
+            p.sk[q] = make_float2(sm.ck[j], __int_as_float(dead ? -1 : p.cell_inner[b + j]));
             p.sci[q] = (int32_t)(b + j);
         }
     }
     // where the connection starts and ends its searches
     if (starts) {
         const int sh = sk_end_shift(n);
-        for (int e = lane; e < sk_ends(n); e += 32) p.sk_end[b + e] = sm.pos[((e + 1) << sh) - 1] >> 16;
+        for (int e = t; e < sk_ends(n); e += 32 * T) p.sk_end[b + e] = sm.pos[((e + 1) << sh) - 1] >> 16;
     }
-    if (lane == 0) p.in_live[o] = n;       // (never all dead: the shortest of them lives)
-    __syncwarp();
+    if (t == 0) p.in_live[o] = n;       // (never all dead: the shortest of them lives)
+    team_sync<T>();
     return alive;
 }
 
 // The same for any n with a pairwise loop over global memory and ranks by
-// direct comparison (outer hits with more cells than a warp holds: sorted
+// direct comparison (outer hits with more cells than a team holds: sorted
 // keys, so sorted buckets too).
-__device__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int lane) {
+template <int T>
+__device__ __noinline__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int t, FbRange *part) {
     const float4 ho = __ldg(p.bh + o);
     const bool disk = p.layer[p.blayer[o]].kind == PT_LAYER_DISK;
     const bool starts = p.layer_is_inner[p.blayer[o]] != 0;
     const GHit gh = ghit(ho.x, ho.y, ho.z, ho.w);
     const FHit h = {ho.x, ho.y, ho.z, ho.w};
-    float k2max = 0.f, gmin = 3.0e38f;
-    float smin = __int_as_float(0x7f800000), smax = -smin;
-    for (int j = lane; j < n; j += 32) {
+    const float inf = __int_as_float(0x7f800000);
+    FbRange rg = {3.0f, -3.0f, inf, -inf, 0.f, 3.0e38f};
+    for (int j = t; j < n; j += 32 * T) {
         const int i1 = p.cell_inner[b + j];
         const int L1 = cell_layer(p, b + j);
         const FHit h1 = load_hit(p.bh, i1);
@@ -290,12 +351,12 @@ __device__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int l
             const float dr = ho.w - h1.r, dz = ho.z - h1.z;
             const float num = disk ? dr : dz, den = disk ? dz : dr;
             const float ck = den != 0.f ? __fdividef(num, den) : __int_as_float(0x7f800000);
-            k2max = fmaxf(k2max, ck * ck);
-            gmin = fminf(gmin, fabsf(den));
+            rg.k2max = fmaxf(rg.k2max, ck * ck);
+            rg.gmin = fminf(rg.gmin, fabsf(den));
             p.ck[b + j] = ck;
             if (fabsf(ck) <= 3.4e38f) {
-                smin = fminf(smin, ck);
-                smax = fmaxf(smax, ck);
+                rg.smin = fminf(rg.smin, ck);
+                rg.smax = fmaxf(rg.smax, ck);
             }
         }
         const GHit g1 = ghit(h1.x, h1.y, h1.z, h1.r);
@@ -315,17 +376,14 @@ __device__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int l
         if (dead) p.cell_alive[b + j] = 0;
     }
     if (starts) {
-        k2max = warp_max(k2max);
-        gmin = warp_min(gmin);
-        smin = warp_min(smin);
-        smax = warp_max(smax);
-        const float span = fmaxf(smax - smin, fmaxf(fabsf(smin), fabsf(smax)) * 1e-6f);
+        rg = team_range<T>(rg, true, part);
+        const float span = fmaxf(rg.smax - rg.smin, fmaxf(fabsf(rg.smin), fabsf(rg.smax)) * 1e-6f);
         const float iw = span > 0.f && span <= 3.4e38f ? (float)sk_buckets(n) / span : 0.f;
-        if (lane == 0) p.hk[o] = make_float4(sqrtf(1.0f + k2max), gmin, smin, iw);
+        if (t == 0) p.hk[o] = make_float4(sqrtf(1.0f + rg.k2max), rg.gmin, rg.smin, iw);
     }
-    __syncwarp();
+    team_sync<T>();
     int alive = 0;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = t; j < n; j += 32 * T) {
         const bool dead = p.cell_alive[b + j] == 0;
         alive += !dead;
         if (!starts) continue;
@@ -338,8 +396,8 @@ __device__ int fishbone_pairwise(const Params &p, int o, int n, int64_t b, int l
         p.sk[b + rank] = make_float2(key, __int_as_float(dead ? -1 : p.cell_inner[b + j]));
         p.sci[b + rank] = (int32_t)(b + j);
     }
-    if (lane == 0) p.in_live[o] = n;
-    __syncwarp();
+    if (t == 0) p.in_live[o] = n;
+    team_sync<T>();
     return alive;
 }
 
@@ -362,14 +420,16 @@ __device__ __forceinline__ void add_alive(const Params &p, int v) {
 // with 32 whatever the size, one PU200 event (30.8 k hits) kept 962 of 4864
 // warps busy (454 -> 75 us with chunks by size; a PU50 event 158 -> 19 us, a
 // batch of 32 of them 279 -> 194 us).
-constexpr int kFbSmallMax = 184;
-constexpr int kFbMidMax = 320;
+constexpr int kFbSmallMax = 128, kFbSmallBlocks = 5;
+constexpr int kFbMidMax = 288, kFbMidWarps = 2, kFbMidBlocks = 20;
+constexpr int kFbMaxWarps = 4, kFbMaxBlocks = 9;
+constexpr int kFbExactWarps = 8;
 
-template <int W, int M, int NB, int kMinBlocks, bool C = true>
+template <int W, int M, int NB, int kMinBlocks>
 __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p, float unit_thr, float du,
                                                                     int chunk_log2) {
     pdl_enter();
-    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ FbCells<M, NB> sm[W];
     __shared__ uint8_t s_slot[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     load_slots(p, s_slot);
@@ -409,7 +469,7 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
             todo &= todo - 1;
             const int n = __shfl_sync(0xffffffffu, nl, t);
             const int b = __shfl_sync(0xffffffffu, bl, t);
-            const int a = fishbone_hit<M, NB, C, false>(p, o0 + t, n, b, lane, unit_thr, du, sm[w], s_slot);
+            const int a = fishbone_hit<1, M, NB, false>(p, o0 + t, n, b, lane, unit_thr, du, sm[w], nullptr, s_slot);
             if (a >= 0) my_alive += a;
             else list_pending(p, o0 + t, lane);
         }
@@ -417,50 +477,54 @@ __global__ void __launch_bounds__(32 * W, kMinBlocks) k_fishbone_small(Params p,
     add_alive(p, my_alive);
 }
 
-// Larger warps: the listed outer hits, one at a time from a queue (kFromBack:
+// The listed outer hits, a block at a time from a queue (kFromBack:
 // the list at the back of the array).
-template <int W, int M, int NB, bool kFromBack, bool C>
-__global__ void __launch_bounds__(32 * W) k_fishbone_large(Params p, float unit_thr, float du) {
+template <int T, int M, int NB, bool kFromBack, int kMinBlocks>
+__global__ void __launch_bounds__(32 * T, kMinBlocks) k_fishbone_large(Params p, float unit_thr, float du) {
     pdl_enter();
-    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ FbCells<M, NB> sm;
+    __shared__ FbRange s_part[T];
     __shared__ uint8_t s_slot[PT_MAX_PAIRS];
+    __shared__ int s_next;
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     load_slots(p, s_slot);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int my_alive = 0;
     const int n_list = p.counters[kFromBack ? C_FB_HUGE : C_FB_BIG];
     for (;;) {
-        int k = 0;
-        if (lane == 0) k = atomicAdd(p.counters + (kFromBack ? C_FB_HUGE_NEXT : C_FB_BIG_NEXT), 1);
-        k = __shfl_sync(0xffffffffu, k, 0);
+        if (threadIdx.x == 0) s_next = atomicAdd(p.counters + (kFromBack ? C_FB_HUGE_NEXT : C_FB_BIG_NEXT), 1);
+        __syncthreads();
+        const int k = s_next;
         if (k >= n_list) break;
         const int o = p.fb_big[kFromBack ? p.n_hits - 1 - k : k];
         const int n = p.in_cnt[o];
-        const int a = n <= M ? fishbone_hit<M, NB, C, false>(p, o, n, p.in_off[o], lane, unit_thr, du, sm[w], s_slot) : -1;
+        int a = -1;
+        if (n <= M)
+            a = fishbone_hit<T, M, NB, false>(p, o, n, p.in_off[o], threadIdx.x, unit_thr, du, sm, s_part, s_slot);
         if (a >= 0) my_alive += a;
-        else list_pending(p, o, lane);
+        else list_pending(p, o, threadIdx.x);
+        __syncthreads();
     }
     add_alive(p, my_alive);
 }
 
 // Exact pass: the outer hits listed by the kernels above (an undecided
-// alignment test, or more cells than a large warp holds), with the exact
+// alignment test, or more cells than those hold), with the exact
 // predicate and the pairwise loop for any number of cells.
-template <int W, int M, int NB, bool C = true>
-__global__ void __launch_bounds__(32 * W) k_fishbone_exact(Params p, float unit_thr, float du) {
+template <int T, int M, int NB>
+__global__ void __launch_bounds__(32 * T) k_fishbone_exact(Params p, float unit_thr, float du) {
     pdl_enter();
-    __shared__ FbWarp<M, NB, C> sm[W];
+    __shared__ FbCells<M, NB> sm;
+    __shared__ FbRange s_part[T];
     __shared__ uint8_t s_slot[PT_MAX_PAIRS];
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     load_slots(p, s_slot);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int my_alive = 0;
     const int n_list = p.counters[C_FB_PENDING];
-    for (int k = blockIdx.x * W + w; k < n_list; k += gridDim.x * W) {
+    for (int k = blockIdx.x; k < n_list; k += gridDim.x) {
         const int o = p.hit_bin[k];
         const int n = p.in_cnt[o], b = p.in_off[o];
-        my_alive += n <= M ? fishbone_hit<M, NB, C, true>(p, o, n, b, lane, unit_thr, du, sm[w], s_slot)
-                           : fishbone_pairwise(p, o, n, b, lane);
+        my_alive += n <= M ? fishbone_hit<T, M, NB, true>(p, o, n, b, threadIdx.x, unit_thr, du, sm, s_part, s_slot)
+                           : fishbone_pairwise<T>(p, o, n, b, threadIdx.x, s_part);
     }
     add_alive(p, my_alive);
 }
@@ -469,20 +533,22 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
     {
         // at least four chunks for each resident warp
         int chunk_log2 = 0;
-        while (chunk_log2 < 5 && (p.n_hits >> (chunk_log2 + 1)) >= 4 * 8 * g.blocks(4)) chunk_log2++;
+        while (chunk_log2 < 5 && (p.n_hits >> (chunk_log2 + 1)) >= 4 * 8 * g.blocks(kFbSmallBlocks)) chunk_log2++;
         KernelTimer t("k_fishbone_small", s);
-        launch_pdl(k_fishbone_small<8, kFbSmallMax, 512, 4>, g.blocks(4), 256, 0, s, p, unit_thr, du, chunk_log2);
+        launch_pdl(k_fishbone_small<8, kFbSmallMax, 256, kFbSmallBlocks>, g.blocks(kFbSmallBlocks), 256, 0, s, p, unit_thr, du, chunk_log2);
     }
     {
         KernelTimer t("k_fishbone_medium", s);
-        launch_pdl(k_fishbone_large<4, kFbMidMax, 512, false, false>, g.blocks(6), 128, 0, s, p, unit_thr, du);
+        launch_pdl(k_fishbone_large<kFbMidWarps, kFbMidMax, 512, false, kFbMidBlocks>, g.blocks(kFbMidBlocks),
+                   32 * kFbMidWarps, 0, s, p, unit_thr, du);
     }
     {
         KernelTimer t("k_fishbone_large", s);
-        launch_pdl(k_fishbone_large<2, 512, 1024, true, true>, g.blocks(6), 64, 0, s, p, unit_thr, du);
+        launch_pdl(k_fishbone_large<kFbMaxWarps, 512, 1024, true, kFbMaxBlocks>, g.blocks(kFbMaxBlocks),
+                   32 * kFbMaxWarps, 0, s, p, unit_thr, du);
     }
     KernelTimer t("k_fishbone_exact", s);
-    launch_pdl(k_fishbone_exact<1, 1024, 1024>, g.blocks(6), 32, 0, s, p, unit_thr, du);
+    launch_pdl(k_fishbone_exact<kFbExactWarps, 1024, 1024>, g.blocks(4), 32 * kFbExactWarps, 0, s, p, unit_thr, du);
 }
 
 }  // namespace ptk

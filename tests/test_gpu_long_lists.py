@@ -35,7 +35,7 @@ def crowded_event(n: int, seed: int) -> dict:
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n", [1, 12, 13, 31, 33, 63, 65, 128, 129, 192, 193, 224, 225, 256, 257, 320, 321, 512, 513, 1024, 1025])
+@pytest.mark.parametrize("n", [1, 12, 13, 31, 33, 63, 65, 128, 129, 192, 193, 224, 225, 256, 257, 288, 289, 320, 321, 512, 513, 1024, 1025])
 def test_lists_of_any_length(n):
     batch, cuts = crowded_event(n, n), CU.make_cuts(pt_min=0.3)
     want = oracle_run(batch, cuts, stage=3)
