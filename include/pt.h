@@ -158,7 +158,7 @@ typedef struct {
 typedef struct {
     int32_t n_phi_bins;     /* azimuthal tiles per layer, 16..1024 */
     int32_t n_t_bins;       /* tiles along z (barrel) or r (disks), 1..64 */
-    int32_t doublet_lanes;  /* lanes per outer hit: 4, 8, 16 or 32 */
+    int32_t doublet_lanes;  /* lanes per outer hit: 4, 8, 16 or 32 (for few hits more are used) */
     int32_t connect_lanes;  /* reserved (4, 8, 16 or 32 accepted); the CA
                                connection runs one warp per middle hit */
     int32_t blocks_per_sm;  /* persistent grid size factor, 1..32 */

@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_count(Params p) {
                     if (__ldg(p.ev_off + mid) <= h) lo = mid; else hi = mid - 1;
                 }
                 int pb = phi_tile(atan2f(y, x), p.n_phi);
-                int tb = t_tile(t, tmin, tmax, p.n_t);
+                int tb = t_tile(t, tmin, t_scale(tmin, tmax, p.n_t), p.n_t);
                 bin = ((lo * PT_N_LAYERS + L) * p.n_phi + pb) * p.n_t + tb;
             }
             p.hit_bin[h] = bin;

@@ -163,8 +163,9 @@ __device__ __forceinline__ int phi_tile(float phi, int n_phi) {
     return min(max(b, 0), n_phi - 1);
 }
 
-__device__ __forceinline__ int t_tile(float t, float tmin, float tmax, int n_t) {
-    int b = __float2int_rd((t - tmin) * (n_t / (tmax - tmin)));
+__device__ __forceinline__ float t_scale(float tmin, float tmax, int n_t) { return n_t / (tmax - tmin); }
+__device__ __forceinline__ int t_tile(float t, float tmin, float scale, int n_t) {
+    int b = __float2int_rd((t - tmin) * scale);
     return min(max(b, 0), n_t - 1);
 }
 

@@ -10,6 +10,9 @@
 // shared-memory buffer.  The cells of one outer hit are written
 // contiguously, so the cells sharing an outer hit (needed by the Fishbone
 // and the CA connection) form one range.
+//
+// What bounds it is instruction issue (70% of the slots taken; a candidate
+// costs about 80 instructions per warp, a window about 500).
 #include "pt_common.cuh"
 #include "pt_kernels.cuh"
 
@@ -18,31 +21,90 @@ namespace ptk {
 constexpr float kTwoPiInv = 0.159154943f;
 constexpr float kPi = 3.14159265f;
 
+// Angles for the windows, whose margins are 1e-4: arctangent and arcsine by the
+// polynomials 4.4.49 (below 1e-5 rad) and 4.4.46 (2e-8) of Abramowitz and Stegun,
+// Handbook of Mathematical Functions.
+__device__ __forceinline__ float window_atan2(float y, float x) {
+    const float ax = fabsf(x), ay = fabsf(y), hi = fmaxf(ax, ay);
+    const float q = hi > 0.f ? __fdividef(fminf(ax, ay), hi) : 0.f, q2 = q * q;
+    float a = q * fmaf(q2, fmaf(q2, fmaf(q2, fmaf(q2, 0.0208351f, -0.0851330f), 0.1801410f), -0.3302995f), 0.9998660f);
+    a = ay > ax ? 0.5f * kPi - a : a;
+    a = x < 0.f ? kPi - a : a;
+    return copysignf(a, y);
+}
+__device__ __forceinline__ float window_asin(float x) {   // 0 <= x < 1
+    float c = fmaf(x, -0.0012624911f, 0.0066700901f);
+    c = fmaf(x, c, -0.0170881256f);
+    c = fmaf(x, c, 0.0308918810f);
+    c = fmaf(x, c, -0.0501743046f);
+    c = fmaf(x, c, 0.0889789874f);
+    c = fmaf(x, c, -0.2145988016f);
+    c = fmaf(x, c, 1.5707963050f);
+    const float d = 1.0f - x;
+    return 0.5f * kPi - d * rsqrtf(d) * c;
+}
+
+// What a sweep needs of a layer pair, in shared memory (a lane-wise index
+// into the kernel's parameters serialises, and what does not depend on the
+// outer hit is worked out once: 1623 -> 1544 us for 64 PU200 events, 105 -> 97
+// for 32 PU50 events; the polynomials above 1535 -> 1494 and 99 -> 95).
+struct PairWin {
+    float zlo, zhi, zmax, tan, k_pt, ez, ep, ec;     // cuts, and the filter's bounds
+    float dphi;                                      // azimuthal half window of PhiW
+    float pa, si, sx;                                // PT: 1 / (2 R) (0: no use), asin(rmin / 2R), asin(rmax / 2R) of the inner layer
+    float rmin, rmax, za, zb;                        // inner layer; barrel: its z range, disk: the z range within the cuts
+    float tscale;                                    // tiles per cm of its z (barrel) or r (disk)
+    int32_t inner;                                   // inner layer, -1 - layer for a disk
+};
+
+__device__ __forceinline__ void load_windows(const Params &p, PairWin *win) {
+    const int k = threadIdx.x;
+    if (k < p.n_pairs) {
+        const pt_pair_cuts pc = p.pair[k];
+        const pt_layer li = p.layer[pc.inner];
+        const bool barrel = li.kind == PT_LAYER_BARREL;
+        PairWin w;
+        w.zlo = pc.zlo, w.zhi = pc.zhi, w.zmax = pc.zmax, w.k_pt = pc.k_pt;
+        w.tan = p.pair_tan[k], w.ez = p.pair_err_zip[k], w.ep = p.pair_err_phi[k], w.ec = p.pair_err_c[k];
+        w.dphi = p.pair_dphi[k];
+        const float pa = p.pair_pt_a[k];
+        w.pa = pa > 0.f && li.rmax * pa < 1.f ? pa : 0.f;
+        w.si = asinf(li.rmin * w.pa), w.sx = asinf(li.rmax * w.pa);
+        w.rmin = li.rmin, w.rmax = li.rmax;
+        w.za = barrel ? li.zmin : fmaxf(li.zmin, pc.zlo);
+        w.zb = barrel ? li.zmax : fminf(li.zmax, pc.zhi);
+        w.tscale = barrel ? t_scale(li.zmin, li.zmax, p.n_t) : t_scale(li.rmin, li.rmax, p.n_t);
+        w.inner = barrel ? pc.inner : -1 - pc.inner;
+        win[k] = w;
+    }
+    __syncthreads();
+}
+
 // Conservative window of the inner hit's t coordinate for a pair, from ZIP
-// (z-intercept within +-zmax) and ZW, over the inner layer's envelope.
-__device__ __forceinline__ void t_window(const Params &p, const pt_pair_cuts &pc, float ro, float zo,
-                                         float &tlo, float &thi) {
-    const pt_layer li = p.layer[pc.inner];
-    const float zm = pc.zmax;
-    if (li.kind == PT_LAYER_BARREL) {
-        float f0 = li.rmin / ro, f1 = li.rmax / ro;
+// (z-intercept within +-zmax) and ZW, over the inner layer's envelope; iro =
+// 1 / ro.  The quotients are good to a few ulp: below 3e-5 cm at the largest
+// z, inside the sweep's margin.
+__device__ __forceinline__ void t_window(const PairWin &w, float ro, float iro, float zo, float &tlo, float &thi) {
+    const float zm = w.zmax;
+    if (w.inner >= 0) {
+        float f0 = w.rmin * iro, f1 = w.rmax * iro;
         float c0 = -zm + (zo + zm) * f0, c1 = -zm + (zo + zm) * f1;
         float c2 = zm + (zo - zm) * f0, c3 = zm + (zo - zm) * f1;
-        tlo = fmaxf(fminf(fminf(c0, c1), fminf(c2, c3)), pc.zlo);
-        thi = fminf(fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)), pc.zhi);
+        tlo = fmaxf(fminf(fminf(c0, c1), fminf(c2, c3)), w.zlo);
+        thi = fminf(fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)), w.zhi);
         if (tlo > thi) tlo = thi = 0.5f * (tlo + thi);
     } else {
-        float za = fmaxf(li.zmin, pc.zlo), zb = fminf(li.zmax, pc.zhi);
+        const float za = w.za, zb = w.zb;
         if (fabsf(zo) > zm * 1.001f + 0.01f && za <= zb) {
-            float d0 = zo + zm, d1 = zo - zm;   // same sign
-            float c0 = ro * (za + zm) / d0, c1 = ro * (zb + zm) / d0;
-            float c2 = ro * (za - zm) / d1, c3 = ro * (zb - zm) / d1;
+            const float q0 = __fdividef(ro, zo + zm), q1 = __fdividef(ro, zo - zm);   // same sign
+            float c0 = q0 * (za + zm), c1 = q0 * (zb + zm);
+            float c2 = q1 * (za - zm), c3 = q1 * (zb - zm);
             tlo = fminf(fminf(c0, c1), fminf(c2, c3));
             thi = fminf(fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)), ro);
             if (tlo > thi) tlo = thi = 0.5f * (tlo + thi);
         } else {
-            tlo = li.rmin;
-            thi = li.rmax;
+            tlo = w.rmin;
+            thi = w.rmax;
         }
     }
 }
@@ -95,33 +157,40 @@ __device__ __forceinline__ void write_cell(const Params &p, int64_t c, int i, in
     p.has_out[c] = 0;
 }
 
+// A cell in shared memory: the inner hit, and the pair above kIndexBits.  With
+// more hits than that nothing is kept there: the outer hits are swept again.
+constexpr int kIndexBits = 27;
+static_assert(PT_MAX_PAIRS <= 1 << (32 - kIndexBits), "pair bits");
+
+__device__ __forceinline__ void write_cell(const Params &p, int64_t c, uint32_t e, int o) {
+    write_cell(p, c, (int)(e & ((1u << kIndexBits) - 1u)), o, (uint8_t)(e >> kIndexBits));
+}
+
 // Sweep all candidate inner hits of outer hit o.  kWrite = false: fill the
-// group's shared buffer (up to cap entries) and count; kWrite = true: write
+// shared buffer (up to cap entries, step apart) and count; kWrite = true: write
 // cells directly at global index base + slot.  kExact = false: the
 // predicates are float32 filters only, and *undecided is set on the lanes
 // that met a candidate they cannot decide.  s_cand (or null): per-pair
 // counts of the candidate inner hits tested, summed in shared memory.
 template <int G, bool kWrite, bool kExact>
-__device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int gshift, int32_t *s_inner,
-                           uint8_t *s_pair, int32_t *s_row, int cap, int64_t base, bool *undecided,
+__device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane, unsigned gmask, int gshift, uint32_t *buf,
+                           int step, int cap, int32_t *s_row, int64_t base, bool *undecided,
                            unsigned long long *s_cand = nullptr) {
     const float4 ho = __ldg(p.bh + o);
     const float xo = ho.x, yo = ho.y, zo = ho.z, ro = ho.w;
     const int Lo = p.blayer[o], ev = p.bev[o];
-    const float phio = atan2f(yo, xo);
-    const float io2 = __fdividef(1.0f, fmaf(xo, xo, yo * yo));
+    const float phio = window_atan2(yo, xo);
+    const float io2 = __fdividef(1.0f, fmaf(xo, xo, yo * yo)), iro = __fdividef(1.0f, ro);
     const unsigned lanes = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     const unsigned below = (1u << lane) - 1u;
     int count = 0;
     const int npo = p.n_pairs_by_outer[Lo];
     for (int k = 0; k < npo; k++) {
         const int pi = p.pairs_by_outer[Lo][k];
-        const pt_pair_cuts pc = p.pair[pi];
+        const PairWin &w = win[pi];
         float tlo, thi;
-        t_window(p, pc, ro, zo, tlo, thi);
-        const pt_layer li = p.layer[pc.inner];
-        const float tmin = li.kind == PT_LAYER_BARREL ? li.zmin : li.rmin;
-        const float tmax = li.kind == PT_LAYER_BARREL ? li.zmax : li.rmax;
+        t_window(w, ro, iro, zo, tlo, thi);
+        const float tmin = w.inner >= 0 ? w.za : w.rmin;
         // Tile ranges: the t window's float32 bounds are within ~1e-5 cm of
         // the exact ones, so a margin of 1e-4 cm keeps every accepted hit
         // inside; the half-width in phi already carries a 1e-4 rad margin
@@ -130,8 +199,8 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
         // same functions), so the tiles cover a superset of the accepted
         // hits whatever the tile counts.
         const float mt = 1e-4f + 1e-6f * fmaxf(fabsf(tlo), fabsf(thi));
-        const int tb0 = t_tile(tlo - mt, tmin, tmax, p.n_t);
-        const int tb1 = t_tile(thi + mt, tmin, tmax, p.n_t);
+        const int tb0 = t_tile(tlo - mt, tmin, w.tscale, p.n_t);
+        const int tb1 = t_tile(thi + mt, tmin, w.tscale, p.n_t);
         // The PT cut (circumradius of beam line, inner and outer hit >= R)
         // accepts an azimuth difference up to |asin(r_o / 2R) - asin(r_i / 2R)|
         // or from pi - asin(r_o / 2R) - asin(r_i / 2R) on (both radii below
@@ -140,11 +209,10 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
         // range lies beyond the pair's PhiW window, the first, taken over the
         // inner layer's radii with a margin far above the rounding of the
         // float32 arcsines, narrows the window to this outer hit.
-        float dphi = p.pair_dphi[pi];
-        const float pa = p.pair_pt_a[pi];
-        if (pa > 0.f && ro * pa < 1.f && li.rmax * pa < 1.f) {
-            const float so = asinf(ro * pa), si = asinf(li.rmin * pa), sx = asinf(li.rmax * pa);
-            if (kPi - so - sx > dphi + 1e-3f) dphi = fminf(dphi, fmaxf(so - si, sx - so) + 1e-4f);
+        float dphi = w.dphi;
+        if (w.pa > 0.f && ro * w.pa < 1.f) {
+            const float so = window_asin(ro * w.pa);
+            if (kPi - so - w.sx > dphi + 1e-3f) dphi = fminf(dphi, fmaxf(so - w.si, w.sx - so) + 1e-4f);
         }
         int f0 = __float2int_rd((phio - dphi + kPi) * (p.n_phi * kTwoPiInv));
         int f1 = __float2int_rd((phio + dphi + kPi) * (p.n_phi * kTwoPiInv));
@@ -153,17 +221,17 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
             f1 = p.n_phi - 1;
         }
         PairFilter pf;
-        pf.zlo = pc.zlo;
-        pf.zhi = pc.zhi;
-        pf.zmax = pc.zmax;
-        pf.zr = pc.zmax * ro;
-        pf.tan = p.pair_tan[pi];
-        pf.k = pc.k_pt * io2;
-        pf.ez = p.pair_err_zip[pi];
-        pf.ep = p.pair_err_phi[pi];
-        pf.c4 = 4.0f * p.pair_err_c[pi];
-        pf.kc2 = 2.0f * pf.k * p.pair_err_c[pi] * p.pair_err_c[pi];
-        const int row0 = (ev * PT_N_LAYERS + pc.inner) * p.n_phi;
+        pf.zlo = w.zlo;
+        pf.zhi = w.zhi;
+        pf.zmax = w.zmax;
+        pf.zr = w.zmax * ro;
+        pf.tan = w.tan;
+        pf.k = w.k_pt * io2;
+        pf.ez = w.ez;
+        pf.ep = w.ep;
+        pf.c4 = 4.0f * w.ec;
+        pf.kc2 = 2.0f * pf.k * w.ec * w.ec;
+        const int row0 = (ev * PT_N_LAYERS + (w.inner >= 0 ? w.inner : -1 - w.inner)) * p.n_phi;
         const int nrows = f1 - f0 + 1;
         unsigned cand = 0;
         // The rows of the window are separate ranges of the binned hits,
@@ -175,7 +243,8 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
             int beg = 0, len = 0;
             if (r0 + lane < nrows) {
                 const int f = f0 + r0 + lane;
-                const int fb = ((f % p.n_phi) + p.n_phi) % p.n_phi;
+                // (|phi| <= pi and dphi < 1.6: f lies within a turn of [0, n_phi))
+                const int fb = f < 0 ? f + p.n_phi : f >= p.n_phi ? f - p.n_phi : f;
                 const int tile = (row0 + fb) * p.n_t;
                 beg = p.bin_cnt[tile + tb0];
                 len = p.bin_cnt[tile + tb1 + 1] - beg;
@@ -207,15 +276,15 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
                     const float4 hi = __ldg(p.bh + i);
                     const float xi = hi.x, yi = hi.y, zi = hi.z, ri = hi.w;
                     v = kExact ? 2 : pair_filter(pf, hi, ho);
-                    if (v == 2) v = zi >= pc.zlo && zi <= pc.zhi ? 2 : 0;
+                    if (v == 2) v = zi >= pf.zlo && zi <= pf.zhi ? 2 : 0;
                     if (v == 2) {
-                        v = pred_zip<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, pc.zmax, p.counters);
+                        v = pred_zip<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, pf.zmax, p.counters);
                         if (v) {
-                            const int v2 = pred_phiw<kExact>(xi, yi, xo, yo, pc.tan2_dphi, p.counters, zi, ri, zo, ro);
+                            const int v2 = pred_phiw<kExact>(xi, yi, xo, yo, p.pair[pi].tan2_dphi, p.counters, zi, ri, zo, ro);
                             v = v2 ? (v | v2) : 0;
                         }
                         if (v) {
-                            const int v3 = pred_pt<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, pc.k_pt, p.counters);
+                            const int v3 = pred_pt<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, p.pair[pi].k_pt, p.counters);
                             v = v3 ? (v | v3) : 0;
                         }
                     }
@@ -228,8 +297,7 @@ __device__ int sweep_outer(const Params &p, int o, int lane, unsigned gmask, int
                     if (kWrite) {
                         write_cell(p, base + slot, i, o, (uint8_t)pi);
                     } else if (slot < cap) {
-                        s_inner[slot] = i;
-                        s_pair[slot] = (uint8_t)pi;
+                        buf[step * slot] = (uint32_t)i | (uint32_t)pi << kIndexBits;
                     }
                 }
                 count += __popc(m);
@@ -255,20 +323,28 @@ __device__ __forceinline__ void write_range(const Params &p, int o, int64_t base
 // one counter's L2 slice was 73% busy (all slices: 23%) and the byte arrays
 // were written eight bytes at a time (164 -> 104 us for 32 PU50 events, 110 ->
 // 100 us for one PU200 event, 1652 -> 1621 us for 64 of them).
+// Two groups share a buffer and fill it from its ends; only if their cells
+// don't fit together are both hits swept again, by all lanes of the warp.  With
+// a buffer of 256 cells for each, and its own lanes sweeping a hit again while
+// the others waited, 24 events with pT > 0.3 GeV, where every tenth hit has
+// more cells, took 940 us against 799, and 64 PU200 events 1544 against 1535.
 template <int G>
 __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
     pdl_enter();
     constexpr int kGroups = kThreads / G, kPerWarp = 32 / G;
-    constexpr int kBuf = 32 * G;   // 40 KB of shared memory per block for every G
-    __shared__ int32_t s_inner[kGroups][kBuf];
-    __shared__ uint8_t s_pair[kGroups][kBuf];
+    constexpr int kBuf = 40 * G;   // 40 KB of shared memory per block for every G
+    constexpr int kPair = kPerWarp > 1 ? 2 : 1, kCap = kPair * kBuf;   // groups that share a buffer, from its ends
+    __shared__ uint32_t s_buf[kGroups / kPair][kCap];
     __shared__ int32_t s_row[kGroups][2 * G];
     __shared__ unsigned long long s_cand[PT_MAX_PAIRS];
+    __shared__ PairWin s_win[PT_MAX_PAIRS];
     if (threadIdx.x < PT_MAX_PAIRS) s_cand[threadIdx.x] = 0;
-    __syncthreads();
+    load_windows(p, s_win);
     const int lane = threadIdx.x % G, grp = threadIdx.x / G, wl = threadIdx.x & 31, gw = wl / G;
     const int gshift = wl & ~(G - 1);
     const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << gshift);
+    const int cap = p.n_hits >> kIndexBits ? 0 : kCap;
+    const bool odd = kPair > 1 && (gw & 1);
     const int n_binned = p.bin_cnt[p.n_bins];
     // the warps take the binned outer hits in order: the cells are laid out
     // nearly in the order of their outer hits
@@ -281,8 +357,10 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
         int n = 0;
         bool und = false;
         if (o < n_binned)
-            n = sweep_outer<G, false, false>(p, o, lane, gmask, gshift, s_inner[grp], s_pair[grp], s_row[grp], kBuf, 0,
-                                             &und, s_cand);
+            n = sweep_outer<G, false, false>(p, s_win, o, lane, gmask, gshift, s_buf[grp / kPair] + (odd ? kCap - 1 : 0),
+                                             odd ? -1 : 1, cap, s_row[grp], 0, &und, s_cand);
+        // what two hits leave in their buffer is whole if both fit
+        const int both = kPair > 1 ? n + __shfl_xor_sync(0xffffffffu, n, G) : n;
         const unsigned um = __ballot_sync(0xffffffffu, und);
         const bool put = o < n_binned && !(um & gmask);
         // listed in hit_bin, free once the hits are binned (one slot per hit)
@@ -301,7 +379,8 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
         for (int q = 0; q < kPerWarp; q++) mine = gw == q ? first[q] : mine;
         if (put && lane == 0) write_range(p, o, base + mine, n);
         __syncwarp();
-        if (!__any_sync(0xffffffffu, n > kBuf)) {
+        const unsigned over = __ballot_sync(0xffffffffu, lane == 0 && n > 0 && both > cap);
+        if (!over) {
             for (int k = wl; k < total; k += 32) {
                 int q = 0, at = k;
 #pragma unroll
@@ -310,12 +389,20 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
                         q = t;
                         at = k - first[t];
                     }
-                write_cell(p, base + k, s_inner[grp - gw + q][at], o0 + q, s_pair[grp - gw + q][at]);
+                write_cell(p, base + k, s_buf[(grp - gw + q) / kPair][kPair > 1 && (q & 1) ? kCap - 1 - at : at], o0 + q);
             }
-        } else if (n <= kBuf) {      // beside a hit with more cells than its buffer holds
-            for (int k = lane; k < n; k += G) write_cell(p, base + mine + k, s_inner[grp][k], o, s_pair[grp][k]);
         } else {
-            sweep_outer<G, true, false>(p, o, lane, gmask, gshift, nullptr, nullptr, s_row[grp], 0, base + mine, &und);
+            // beside hits with more cells than their buffer holds; those are swept again by all lanes
+            if (both <= cap)
+                for (int k = lane; k < n; k += G)
+                    write_cell(p, base + mine + k, s_buf[grp / kPair][odd ? kCap - 1 - k : k], o);
+            for (unsigned m = over; m; m &= m - 1) {
+                const int from = __ffs(m) - 1;
+                const int64_t at = base + __shfl_sync(0xffffffffu, mine, from);
+                __syncwarp();
+                sweep_outer<32, true, false>(p, s_win, o0 + from / G, wl, 0xffffffffu, 0, nullptr, 0, 0,
+                                             s_row[grp - gw], at, &und);
+            }
         }
         __syncwarp();
     }
@@ -329,26 +416,28 @@ __global__ void __launch_bounds__(kThreads, 5) k_doublets(Params p) {
 // and no warp runs two hits' exact fallbacks one after the other.
 __global__ void __launch_bounds__(kThreads) k_doublets_exact(Params p) {
     pdl_enter();
-    constexpr int G = 32, kGroups = kThreads / G, kBuf = 32 * G;
-    __shared__ int32_t s_inner[kGroups][kBuf];
-    __shared__ uint8_t s_pair[kGroups][kBuf];
+    constexpr int G = 32, kGroups = kThreads / G, kBuf = 40 * G;
+    __shared__ uint32_t s_buf[kGroups][kBuf];
     __shared__ int32_t s_row[kGroups][2 * G];
+    __shared__ PairWin s_win[PT_MAX_PAIRS];
+    load_windows(p, s_win);
     const int lane = threadIdx.x % G, grp = threadIdx.x / G;
+    const int cap = p.n_hits >> kIndexBits ? 0 : kBuf;
     const int n = p.counters[C_DB_PENDING];
     for (int k = grp * gridDim.x + blockIdx.x; k < n; k += gridDim.x * kGroups) {
         const int o = p.hit_bin[k];
         bool und = false;
-        const int nc = sweep_outer<G, false, true>(p, o, lane, 0xffffffffu, 0, s_inner[grp], s_pair[grp], s_row[grp],
-                                                   kBuf, 0, &und);
+        const int nc = sweep_outer<G, false, true>(p, s_win, o, lane, 0xffffffffu, 0, s_buf[grp], 1, cap, s_row[grp], 0,
+                                                   &und);
         int64_t base = 0;
         if (lane == 0 && nc > 0) base = atomicAdd(p.counters + C_CELLS, nc);
         base = __shfl_sync(0xffffffffu, base, 0);
         if (lane == 0) write_range(p, o, base, nc);
         __syncwarp();
-        if (nc <= kBuf)
-            for (int j = lane; j < nc; j += G) write_cell(p, base + j, s_inner[grp][j], o, s_pair[grp][j]);
+        if (nc <= cap)
+            for (int j = lane; j < nc; j += G) write_cell(p, base + j, s_buf[grp][j], o);
         else
-            sweep_outer<G, true, true>(p, o, lane, 0xffffffffu, 0, nullptr, nullptr, s_row[grp], 0, base, &und);
+            sweep_outer<G, true, true>(p, s_win, o, lane, 0xffffffffu, 0, nullptr, 0, 0, s_row[grp], base, &und);
         __syncwarp();
     }
 }
@@ -357,6 +446,11 @@ void launch_doublets(const Params &p, int lanes, const Grid &g, cudaStream_t s) 
     {
         KernelTimer t("k_doublets", s);
         const int grid = g.blocks(5);
+        // Few hits: more lanes for each, so that every resident warp gets at
+        // least four claims (one PU200 event: 1.3 claims with 8 lanes, 83 ->
+        // 57 us with 32; one PU50 event 20 -> 17; from ~100 k hits on 8 lanes are
+        // as good or better, 32 PU50 events 99 against 143 us with 16)
+        while (lanes < 32 && (int64_t)p.n_hits * lanes < (int64_t)4 * kThreads * grid) lanes *= 2;
         switch (lanes) {
         case 4: launch_pdl(k_doublets<4>, grid, kThreads, 0, s, p); break;
         case 8: launch_pdl(k_doublets<8>, grid, kThreads, 0, s, p); break;
