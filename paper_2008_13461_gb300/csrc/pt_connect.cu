@@ -186,22 +186,6 @@ __device__ __forceinline__ bool in_window(const float2 &e, float key_c, float wd
     return fabsf(e.x - key_c) <= wdt && __float_as_int(e.y) >= 0;
 }
 
-// Every inner cell (a,b) connecting to the live cell x = (b,c), one after the
-// other in the order of b's bucket-ordered arrays: emit(t, i) for the t-th
-// one, i its index there.  Returns their number.
-template <bool kExact, class Emit>
-__device__ __forceinline__ int scan_cell(const Params &p, int x, Emit &&emit) {
-    const Search s = search_of(p, p.cell_inner[x], p.cell_outer[x]);
-    int n = 0;
-    for (int k = s.r; k < s.end; k++) {
-        const float2 e = __ldg(p.sk + k);
-        if (!in_window(e, s.key_c, s.wdt)) continue;
-        if (connects<kExact>(p, __ldg(p.bh + __float_as_int(e.y)), s.B, s.C, p.region[s.disk ? 1 : 0]) == 1)
-            emit(n++, k);
-    }
-    return n;
-}
-
 // Per warp: the cells of a chunk to search, the searches of up to 32 of them,
 // and the edges found.
 struct __align__(16) CaWarp {
@@ -429,29 +413,57 @@ __global__ void __launch_bounds__(32 * kCaWarps, 12) k_connect(Params p) {
     }
 }
 
-// The cells with an undecided candidate (a few hundred), one thread each,
-// with the exact predicates; each reserves its own edges.
+// The cells with an undecided candidate (a few hundred), a warp each, with the
+// exact predicates: an entry per lane, so that a cell waits for one exact
+// evaluation and not for those of its run one after the other, twice (a
+// thread per cell: 63 -> 20 us for 24 events with pT > 0.3 GeV, 25 -> 11 for one
+// PU200 event).  A run of more than 32 entries is gone through twice, to count
+// and to write.
 __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
     pdl_enter();
     if (upstream_overflow(p, PT_FLAG_CELLS)) return;
     const int n = (int)min((int64_t)p.counters[C_CA_PENDING], p.cap_cells);
     const int32_t *list = reinterpret_cast<const int32_t *>(p.ck);
-    // cells dealt round the blocks first: they spread over the SMs, and a
-    // warp seldom holds two cells whose exact fallbacks would run in turn
-    for (int k = threadIdx.x * gridDim.x + blockIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    // cells dealt round the blocks first: they spread over the SMs
+    for (int k = w * gridDim.x + blockIdx.x; k < n; k += gridDim.x * (blockDim.x >> 5)) {
         const int x = list[k];
-        const int m = scan_cell<true>(p, x, [](int, int) {});
-        const int64_t base = m > 0 ? atomicAdd(p.counters + C_EDGES, m) : 0;
-        scan_cell<true>(p, x, [&](int t, int i) {
-            const int ci = p.sci[i];
-            if (base + t < p.cap_edges) {
-                p.edge_src[base + t] = ci;
-                p.edge_dst[base + t] = x;
+        const Search s = search_of(p, p.cell_inner[x], p.cell_outer[x]);
+        const auto hit = [&](int e0) {
+            const int e = e0 + lane;
+            bool v = false;
+            if (e < s.end) {
+                const float2 q = __ldg(p.sk + e);
+                if (in_window(q, s.key_c, s.wdt))
+                    v = connects<true>(p, __ldg(p.bh + __float_as_int(q.y)), s.B, s.C, p.region[s.disk ? 1 : 0]);
             }
-            p.has_out[ci] = 1;
-        });
-        if (base + m > p.cap_edges) set_flag(p.counters, PT_FLAG_EDGES);
-        p.edge_rng[x] = make_int2((int32_t)base, m);
+            return __ballot_sync(0xffffffffu, v);
+        };
+        unsigned found = hit(s.r);
+        int m = __popc(found);
+        for (int e0 = s.r + 32; e0 < s.end; e0 += 32) m += __popc(hit(e0));
+        int64_t base = 0;
+        if (lane == 0 && m > 0) base = atomicAdd(p.counters + C_EDGES, m);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        int64_t at = base;
+        for (int e0 = s.r; e0 < s.end && m > 0; e0 += 32) {
+            if (e0 > s.r) found = hit(e0);
+            if ((found >> lane) & 1) {
+                const int ci = p.sci[e0 + lane];
+                const int64_t t = at + __popc(found & below);
+                if (t < p.cap_edges) {
+                    p.edge_src[t] = ci;
+                    p.edge_dst[t] = x;
+                }
+                p.has_out[ci] = 1;
+            }
+            at += __popc(found);
+        }
+        if (lane == 0) {
+            if (base + m > p.cap_edges) set_flag(p.counters, PT_FLAG_EDGES);
+            p.edge_rng[x] = make_int2((int32_t)base, m);
+        }
     }
 }
 

@@ -275,7 +275,7 @@ __device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane,
                     i = sl + s_row[j];
                     const float4 hi = __ldg(p.bh + i);
                     const float xi = hi.x, yi = hi.y, zi = hi.z, ri = hi.w;
-                    v = kExact ? 2 : pair_filter(pf, hi, ho);
+                    v = pair_filter(pf, hi, ho);
                     if (v == 2) v = zi >= pf.zlo && zi <= pf.zhi ? 2 : 0;
                     if (v == 2) {
                         v = pred_zip<kExact>(xi, yi, zi, ri, xo, yo, zo, ro, pf.zmax, p.counters);
