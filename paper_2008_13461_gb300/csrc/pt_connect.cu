@@ -305,7 +305,12 @@ __global__ void __launch_bounds__(32 * kCaWarps, 12) k_connect(Params p) {
     CaWarp &sm = s_warp[w];
     const unsigned below = (1u << lane) - 1u;
     const int64_t n_cells = min((int64_t)p.counters[C_CELLS], p.cap_cells);
-    const int n_chunks = (int)((n_cells + kCaPer - 1) / kCaPer);
+    // fewer cells to a chunk where 128 would leave warps without one (one PU50
+    // event 24 -> 16 us, 50 helices 18 -> 12)
+    const int warps = gridDim.x * kCaWarps;
+    const int rounds = (int)min((int64_t)kCaChunk, max((n_cells + 32 * warps - 1) / (32 * warps), (int64_t)1));
+    const int per = 32 * rounds;
+    const int n_chunks = (int)((n_cells + per - 1) / per);
     // the warps take the chunks in order from a queue: the chunks in flight
     // are neighbours, and so are the middle hits whose sorted cells they read
     for (;;) {
@@ -313,7 +318,7 @@ __global__ void __launch_bounds__(32 * kCaWarps, 12) k_connect(Params p) {
         if (lane == 0) ch = atomicAdd(p.counters + C_CA_NEXT, 1);
         ch = __shfl_sync(0xffffffffu, ch, 0);
         if (ch >= n_chunks) break;
-        const int64_t x0 = (int64_t)ch * kCaPer;
+        const int64_t x0 = (int64_t)ch * per, x1 = min(x0 + per, n_cells);
         // 1) the live cells whose inner hit can have cells ending on it (no
         //    cell ends on a layer that is the outer layer of no pair; most
         //    cells start on BPix1: no edge range is written for them, and the
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(32 * kCaWarps, 12) k_connect(Params p) {
         for (int it = 0; it < kCaChunk; it++) {
             const int pos = it * 32 + lane;
             const int64_t x = x0 + pos;
-            const bool need = x < n_cells && p.cell_alive[x] && s_inner_is_outer[p.cell_pair[x]];
+            const bool need = x < x1 && p.cell_alive[x] && s_inner_is_outer[p.cell_pair[x]];
             const unsigned m = __ballot_sync(0xffffffffu, need);
             if (need) {
                 const int i = nlist + __popc(m & below);
