@@ -268,7 +268,7 @@ STAGE_KERNELS = {
     "a5_cleaning": ("k_clean_max", "k_clean_keep"),
     "a6_fit": ("k_count_tracks", "k_select_tracks", "k_fit<3>", "k_fit<4>", "k_fit<5>", "k_fit<6..8>"),
 }
-FB_CLASS_MAX = {"k_fishbone_small": 192, "k_fishbone_medium": 320, "k_fishbone_large": 512}
+FB_CLASS_MAX = {"k_fishbone_small": 128, "k_fishbone_medium": 288, "k_fishbone_large": 512}
 
 
 def stage_bytes(H, D, E, T, K_by_n):

@@ -60,7 +60,7 @@ namespace ptk {
 constexpr int kCaWarps = 4;
 constexpr int kCaChunk = 4;         // rounds of 32 cells per edge reservation
 constexpr int kCaPer = 32 * kCaChunk;
-constexpr int kCaAcc = 160;         // edges a warp remembers
+constexpr int kCaQueue = 160;         // edges a warp remembers
 
 // The predicate chain: 1 connects, 0 does not; with kExact = false, 2 when
 // a float32 filter cannot decide and none fails.
@@ -194,8 +194,8 @@ struct __align__(16) CaWarp {
     int32_t cand[3][64];             // candidates that passed the window: entry, inner hit, search
     int32_t b[kCaPer], c[kCaPer];    // cells to search: inner and outer hit,
     uint8_t pos[kCaPer];             //   position in the chunk
-    uint8_t acc_pos[kCaAcc];         // edges found, by position: position of the cell,
-    int32_t acc[kCaAcc];             //   entry of the inner cell
+    uint8_t acc_pos[kCaQueue];         // edges found, by position: position of the cell,
+    int32_t acc[kCaQueue];             //   entry of the inner cell
     uint32_t und[kCaChunk];          // positions left to the exact pass
 };
 
@@ -229,7 +229,7 @@ __device__ __noinline__ int write_edges(const Params &p, CaWarp &sm, int64_t x0,
         for (int i = lane; i < na; i += 32) stay += sm.acc_pos[i] == pos;
         stay = __reduce_add_sync(0xffffffffu, stay);
         if (stay == na) {
-            if (na + 32 <= kCaAcc) return na;
+            if (na + 32 <= kCaQueue) return na;
             __syncwarp();
             if (lane == 0) sm.und[pos >> 5] |= 1u << (pos & 31);
             __syncwarp();
@@ -273,7 +273,7 @@ __device__ __noinline__ int write_edges(const Params &p, CaWarp &sm, int64_t x0,
 // the predicates on candidates 0..n-1 <= 32, a lane each; those that connect
 // join the edges found
 __device__ __forceinline__ int test_candidates(const Params &p, CaWarp &sm, int64_t x0, int n, int na, int lane) {
-    while (na + 32 > kCaAcc) na = write_edges(p, sm, x0, na, false, lane);
+    while (na + 32 > kCaQueue) na = write_edges(p, sm, x0, na, false, lane);
     int v = 0, k = 0, pos = 0;
     if (lane < n) {
         const int i = sm.cand[2][lane];
