@@ -42,14 +42,14 @@
 // hit takes.  Most outer hits have few cells, so three launches share the
 // work: one warp per hit up to 128 cells (256 buckets, 40 warps per SM),
 // taking chunks of outer hits from a queue and listing the others for two
-// warps (up to 288 cells, 40 warps per SM) and four warps per hit (up to 512,
-// 36); an exact pass of eight takes the rest (undecided tests, more
+// warps (up to 288 cells, 42 warps per SM) and four warps per hit (up to 512,
+// 44); an exact pass of eight takes the rest (undecided tests, more
 // cells), sorted in shared memory like the others up to 1024 cells, which
 // pT > 0.3 GeV events reach (0.2% of their hits), with a pairwise loop over
 // global memory beyond.  With one warp per hit throughout (up to 184, 320 and
 // 512 cells; 32, 24 and 12 warps per SM) the four kernels took 2.25 + 0.79 +
-// 0.05 + 0.04 ms for 64 PU200 events, now 1.21 + 1.41 + 0.05 + 0.02; 0.68 + 0.93
-// + 0.36 + 0.07 for 24 events with pT > 0.3 GeV, now 0.42 + 0.76 + 0.37 + 0.02;
+// 0.05 + 0.04 ms for 64 PU200 events, now 1.20 + 1.38 + 0.05 + 0.02; 0.68 + 0.93
+// + 0.36 + 0.07 for 24 events with pT > 0.3 GeV, now 0.42 + 0.75 + 0.35 + 0.02;
 // 62 + 57 + 42 + 17 us for one PU200 event, whose few large hits are a wait for
 // the slowest team, now 47 + 48 + 19 + 13; 158 us for 32 PU50 events, now 146.
 // Limits of 64 or 96 cells for one warp take 8% and 3% longer in all; 256 or 320
@@ -421,8 +421,8 @@ __device__ __forceinline__ void add_alive(const Params &p, int v) {
 // warps busy (454 -> 75 us with chunks by size; a PU50 event 158 -> 19 us, a
 // batch of 32 of them 279 -> 194 us).
 constexpr int kFbSmallMax = 128, kFbSmallBlocks = 5;
-constexpr int kFbMidMax = 288, kFbMidWarps = 2, kFbMidBlocks = 20;
-constexpr int kFbMaxWarps = 4, kFbMaxBlocks = 9;
+constexpr int kFbMidMax = 288, kFbMidWarps = 2, kFbMidBlocks = 21;
+constexpr int kFbMaxWarps = 4, kFbMaxBlocks = 11;
 constexpr int kFbExactWarps = 8;
 
 template <int W, int M, int NB, int kMinBlocks>
