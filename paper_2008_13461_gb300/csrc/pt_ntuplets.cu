@@ -94,11 +94,21 @@ __device__ __forceinline__ void dfs_emit(const Params &p, DfsHold &hold, const D
     }
 }
 
+// How many n-tuplets the warp has found (whole warp; every lane gets the same
+// number).  The lanes meet once more after the read: one that went on to the
+// next edges and counted there before another had read would leave the two
+// with different numbers, and with them in different collectives.
+__device__ __forceinline__ int dfs_held(const DfsHold &hold) {
+    __syncwarp();
+    const int n = hold.count[threadIdx.x >> 5];
+    __syncwarp();
+    return n;
+}
+
 // writes the warp's held n-tuplets (whole warp)
 __device__ __forceinline__ void dfs_flush(const Params &p, DfsHold &hold) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncwarp();
-    const int n = min(hold.count[w], kDfsHold);
+    const int n = min(dfs_held(hold), kDfsHold);
     int t0 = 0;
     if (lane == 0 && n > 0) t0 = atomicAdd(p.counters + C_TUPLES, n);
     t0 = __shfl_sync(0xffffffffu, t0, 0);
@@ -164,8 +174,7 @@ __global__ void __launch_bounds__(kThreads) k_dfs(Params p) {
             pa.hit[1] = r.w;
             dfs_level<1>(p, hold, pa, r.y, r.z, p.perm[p.cell_outer[c]]);
         }
-        __syncwarp();
-        if (hold.count[w] >= kDfsHold / 2) dfs_flush(p, hold);
+        if (dfs_held(hold) >= kDfsHold / 2) dfs_flush(p, hold);
     }
     dfs_flush(p, hold);
 }
