@@ -213,6 +213,7 @@ __device__ __noinline__ int write_edges(const Params &p, CaWarp &sm, int64_t x0,
             const int pos = i < na ? sm.acc_pos[i] : 0, k = i < na ? sm.acc[i] : 0;
             const bool keep = i < na && !((sm.und[pos >> 5] >> (pos & 31)) & 1);
             const unsigned m = __ballot_sync(0xffffffffu, keep);
+            __syncwarp();            // all have read what some now write over (a ballot alone orders no memory)
             if (keep) {
                 sm.acc_pos[n + __popc(m & below)] = (uint8_t)pos;
                 sm.acc[n + __popc(m & below)] = k;
