@@ -247,7 +247,9 @@ class Pipeline:
 
     def result(self, bufs: Buffers, counts: L.Counts, x, y, z, r, module, ev_off) -> Result:
         nc, ne, nt, nk = counts.n_cells, counts.n_edges, counts.n_tuples, counts.n_tracks
-        rows = lambda t, n, w: t.as_strided((n, w), (w, 1))        # one view each: small events notice
+        # one view each (small events notice), of no more rows than the buffer
+        # has: after an overflow the counts go beyond it
+        rows = lambda t, n, w: t.as_strided((min(n, t.numel() // w), w), (w, 1))
         return Result(
             counts=counts,
             cells=dict(inner=bufs.cell_inner[:nc], outer=bufs.cell_outer[:nc], pair=bufs.cell_pair[:nc],
