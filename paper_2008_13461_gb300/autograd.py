@@ -12,6 +12,7 @@ from __future__ import annotations
 import torch
 
 from . import _lib as L
+from .pipeline import own
 
 
 class _Fit(torch.autograd.Function):
@@ -106,7 +107,7 @@ class DifferentiableFit:
         dev = x.device
         gp = (gparams if gparams is not None else torch.zeros(0, 5, device=dev)).to(torch.float32).contiguous()
         gc = None if gchi2 is None else gchi2.to(torch.float32).contiguous()
-        gx, gy, gz = torch.zeros((3,) + x.shape, dtype=x.dtype, device=dev).unbind()
+        gx, gy, gz = own(torch.zeros((3,) + x.shape, dtype=x.dtype, device=dev))
         if gparams is None:
             k = int(gc.numel()) if gc is not None else 0
             gp = torch.zeros(k, 5, device=dev)
@@ -137,10 +138,9 @@ class DifferentiableFit:
         gxo, gyo, gzo = ((g if g is not None else torch.zeros_like(x)).contiguous() for g in (gxo, gyo, gzo))
         nm = self.centres.shape[0]
         want_hits = any(needs[:3])
-        gx, gy, gz = (torch.zeros((3,) + x.shape, dtype=x.dtype, device=x.device).unbind() if want_hits
+        gx, gy, gz = (own(torch.zeros((3,) + x.shape, dtype=x.dtype, device=x.device)) if want_hits
                       else (None, None, None))
-        gsr = torch.zeros(2, nm, 3, device=x.device)
-        gs, gr = (g if need else None for g, need in zip(gsr.unbind(), needs[3:5]))
+        gs, gr = (g if need else None for g, need in zip(own(torch.zeros(2, nm, 3, device=x.device)), needs[3:5]))
         ptr = lambda t: None if t is None else t.data_ptr()
         L.align_hits_grad(x.numel(), x.data_ptr(), y.data_ptr(), z.data_ptr(), self.module.data_ptr(), nm,
                           self.centres.data_ptr(), rot.data_ptr(), gxo.data_ptr(), gyo.data_ptr(), gzo.data_ptr(),

@@ -28,6 +28,14 @@ def _ptr(t: torch.Tensor | None) -> int | None:
     return None if t is None else t.data_ptr()
 
 
+def own(parts) -> list:
+    """Views of one allocation as tensors of their own, which share only its
+    memory: autograd lets each be changed in place, and counts the changes of
+    each apart (views of one tensor have one version, and the parts of an
+    unbind or a split may not be changed in place with a gradient)."""
+    return [t.data for t in parts]
+
+
 @dataclasses.dataclass
 class Buffers:
     n_hits: int
@@ -81,9 +89,9 @@ def find_vertices(ev, z0, ez0, pt, nhits, keep, n_events: int, cuts: dict | None
     E, M = n_events, max_vertices
     # the call is short, so it allocates twice, not once per output (the
     # library clears the status itself)
-    res = dict(zip(("n", "track_vertex", "status", "ndf", "ntracks"),
-                   torch.empty(E + k + 1 + 2 * E * M, dtype=torch.int32, device=dev).split((E, k, 1, E * M, E * M))))
-    res.update(zip(("z", "ez", "chi2", "sumpt2"), torch.empty(4, E, M, dtype=torch.float32, device=dev).unbind()))
+    ints = torch.empty(E + k + 1 + 2 * E * M, dtype=torch.int32, device=dev)
+    res = dict(zip(("n", "track_vertex", "status", "ndf", "ntracks"), own(ints.split((E, k, 1, E * M, E * M)))))
+    res.update(zip(("z", "ez", "chi2", "sumpt2"), own(torch.empty(4, E, M, dtype=torch.float32, device=dev))))
     res["ndf"], res["ntracks"] = res["ndf"].view(E, M), res["ntracks"].view(E, M)
     nbytes = L.vertex_scratch_size(k, E)
     scratch = torch.empty(2 * ((nbytes + 15) // 16), dtype=torch.int64, device=dev)     # 16-byte units
@@ -282,7 +290,7 @@ class Pipeline:
         ev, z0, ez0, pt, nhits (device tensors of n_tracks)."""
         s = (stream or torch.cuda.current_stream(self.device)).cuda_stream
         k = counts.n_tracks
-        o = dict(zip(("z0", "ez0", "pt"), torch.empty(3, max(1, k), dtype=torch.float32, device=self.device).unbind()),
+        o = dict(zip(("z0", "ez0", "pt"), own(torch.empty(3, max(1, k), dtype=torch.float32, device=self.device))),
                  ev=torch.empty(max(1, k), dtype=torch.int32, device=self.device),
                  nhits=torch.empty(max(1, k), dtype=torch.uint8, device=self.device))
         _, _, tuples, tracks = bufs.structs()
