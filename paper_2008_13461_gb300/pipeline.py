@@ -86,7 +86,7 @@ def find_vertices(ev, z0, ez0, pt, nhits, keep, n_events: int, cuts: dict | None
             raise ValueError("find_vertices: per-track tensors must be contiguous, of equal length and dtypes "
                              "int32 / float32 x3 / uint8 / uint8")
     s = (stream or torch.cuda.current_stream(dev)).cuda_stream
-    E, M = n_events, max_vertices
+    E, M = max(0, n_events), max(0, max_vertices)              # (the library refuses what is below)
     # the call is short, so it allocates twice, not once per output (the
     # library clears the status itself)
     ints = torch.empty(E + k + 1 + 2 * E * M, dtype=torch.int32, device=dev)
@@ -102,7 +102,8 @@ def find_vertices(ev, z0, ez0, pt, nhits, keep, n_events: int, cuts: dict | None
                       int(c["min_tracks"]))
     vo = L.Vertices(*(res[n].data_ptr() for n in ("n", "z", "ez", "chi2", "sumpt2", "ndf", "ntracks",
                                                     "track_vertex", "status")))
-    L.find_vertices(trk, k, E, vc, M, scratch.data_ptr(), scratch.numel() * scratch.element_size(), vo, s)
+    L.find_vertices(trk, k, n_events, vc, max_vertices, scratch.data_ptr(),
+                    scratch.numel() * scratch.element_size(), vo, s)
     if stream is not None:
         scratch.record_stream(stream)
     res["scratch"] = scratch                                   # kept alive until the stream has used it
