@@ -50,8 +50,10 @@
  *    that run are then incomplete and must be discarded.
  *  - Inputs must satisfy the exactness contract: every hit coordinate
  *    (x, y, z, r) is a float32 multiple of 2^-14 cm with magnitude below
- *    64 cm, and each hit lies inside the envelope of its layer.  Violations
- *    set PT_FLAG_INPUT.  Under the contract every doublet / cell / n-tuplet
+ *    64 cm, and each hit lies inside the envelope of its layer (its r and z;
+ *    r is expected to be the hypotenuse of x and y to 2^-13 cm, but need not
+ *    be: the search of a batch that holds any hit of which that is not so is
+ *    slower, and as exact).  Violations set PT_FLAG_INPUT.  Under the contract every doublet / cell / n-tuplet
  *    decision is the sign of an integer polynomial in the hit coordinates and
  *    the exact binary values of the float32 cut constants, and is decided
  *    exactly (a float32 evaluation with a proven error bound, falling back to

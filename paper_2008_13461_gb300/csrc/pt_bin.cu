@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_count(Params p) {
             if (bad) {
                 set_flag(p.counters, PT_FLAG_INPUT);
             } else {
+                if (!on_radius(x, y, r)) p.counters[C_OFF_RADIUS] = 1;
                 // event of hit h: ev_off[e] <= h < ev_off[e+1]
                 int lo = 0, hi = p.n_events - 1;
                 while (lo < hi) {

@@ -20,6 +20,7 @@ constexpr int kCounters = kHot + 6 * 32;
 enum Counter {
     C_CELLS = kHot, C_EDGES = kHot + 32, C_TUPLES = kHot + 64, C_TRACKS = 3, C_FLAGS = 4, C_FALLBACK = 5,
     C_ALIVE_CELLS = 6, C_ALIVE_TUPLES = 7,
+    C_OFF_RADIUS = 8,     // not 0: some hit's r is not the hypotenuse of x and y (on_radius)
     C_FB_NEXT = kHot + 96,     // Fishbone: next chunk of outer hits to take
     C_FB_BIG = 10,        // Fishbone: outer hits listed for the large warps
     C_FB_BIG_NEXT = 11,   // Fishbone: next listed outer hit to take
@@ -117,7 +118,7 @@ struct Params {
     float pair_pt_a[PT_MAX_PAIRS];       // 1 / (2 R) of the PT cut's minimum circumradius R (0: no cut)
     float pair_tan[PT_MAX_PAIRS];        // sqrt(tan2_dphi)
     float pair_err_zip[PT_MAX_PAIRS];    // rounding bounds of the doublet filter (pt_doublets.cu) over the
-    float pair_err_phi[PT_MAX_PAIRS];    //   pair's envelopes: of ZIP, of PhiW
+    float pair_err_phi[PT_MAX_PAIRS];    //   pair's envelopes (hits on their radius): of ZIP, of PhiW
     float pair_err_c[PT_MAX_PAIRS];      //   and of the cross product i x o
     int32_t n_pairs;
     int8_t pairs_by_outer[PT_N_LAYERS][kMaxPairsPerLayer];
@@ -161,6 +162,14 @@ __device__ __forceinline__ long long grid_int(float v) {
 __device__ __forceinline__ int phi_tile(float phi, int n_phi) {
     int b = __float2int_rd((phi + 3.14159265f) * (n_phi * 0.159154943f));
     return min(max(b, 0), n_phi - 1);
+}
+
+// r is the hypotenuse of x and y to 2^-13 (two grid steps; x, y and r rounded
+// each for itself are off by 1.3).  What searches less or computes with smaller bounds because of it
+// (the doublets) asks C_OFF_RADIUS first.  The squares' rounding, below 3u
+// (x^2 + y^2 + r^2), is at most a tenth of the bound.
+__device__ __forceinline__ bool on_radius(float x, float y, float r) {
+    return fabsf(fmaf(x, x, y * y) - r * r) <= 2.44140625e-4f * fabsf(r) + 1.5e-8f;
 }
 
 __device__ __forceinline__ float t_scale(float tmin, float tmax, int n_t) { return n_t / (tmax - tmin); }

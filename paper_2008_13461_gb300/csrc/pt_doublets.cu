@@ -57,18 +57,32 @@ struct PairWin {
     int32_t inner;                                   // inner layer, -1 - layer for a disk
 };
 
+// While every hit's r is the hypotenuse of its x and y (on_radius), |x|, |y|
+// and so the filter's errors are bounded over the layers' envelopes, and the
+// azimuth window may be narrowed by the radius.  With a hit off its radius in
+// the batch, x and y are bounded by the grid alone (64 cm), and no window is
+// narrowed: more candidates go to the sharper filters, which take their bounds
+// from the operands.
+constexpr float kGridXY = 64.0f * 64.0f;
+
 __device__ __forceinline__ void load_windows(const Params &p, PairWin *win) {
     const int k = threadIdx.x;
+    const bool off = p.counters[C_OFF_RADIUS] != 0;
     if (k < p.n_pairs) {
         const pt_pair_cuts pc = p.pair[k];
         const pt_layer li = p.layer[pc.inner];
         const bool barrel = li.kind == PT_LAYER_BARREL;
         PairWin w;
         w.zlo = pc.zlo, w.zhi = pc.zhi, w.zmax = pc.zmax, w.k_pt = pc.k_pt;
-        w.tan = p.pair_tan[k], w.ez = p.pair_err_zip[k], w.ep = p.pair_err_phi[k], w.ec = p.pair_err_c[k];
+        w.tan = p.pair_tan[k], w.ez = p.pair_err_zip[k];
+        w.ep = off ? 8.0f * kU * kGridXY * (1.0f + w.tan) : p.pair_err_phi[k];
+        w.ec = off ? 4.0f * kU * kGridXY : p.pair_err_c[k];
         w.dphi = p.pair_dphi[k];
+        // (an error of 2^-13 in each radius moves the arcsines' difference by
+        // less than 6e-5 while 2R >= 10 cm and the radii are below 0.9 of it,
+        // which is inside the margin of 1e-4)
         const float pa = p.pair_pt_a[k];
-        w.pa = pa > 0.f && li.rmax * pa < 1.f ? pa : 0.f;
+        w.pa = pa > 0.f && pa <= 0.1f && li.rmax * pa < 0.9f && !off ? pa : 0.f;
         w.si = asinf(li.rmin * w.pa), w.sx = asinf(li.rmax * w.pa);
         w.rmin = li.rmin, w.rmax = li.rmax;
         w.za = barrel ? li.zmin : fmaxf(li.zmin, pc.zlo);
@@ -116,15 +130,16 @@ __device__ __forceinline__ void t_window(const PairWin &w, float ro, float iro, 
 // about twice the operations (k_doublets 1721 -> 1652 us for 64 PU200 events),
 // so the cuts are taken in forms with few operations and bounds that are
 // constants of the pair; one candidate in ~10^5 lies within them and goes to
-// the sharper filters.  With u = 2^-24, hits within their layers' envelopes (checked on
-// input) and every rounding at most u relative:
+// the sharper filters.  With u = 2^-24, hits within their layers' envelopes and on
+// their radius (both checked on input; load_windows says what is taken if a hit is off
+// it) and every rounding at most u relative:
 //  ZIP   F = (zmax ro - zmax ri) - |zi ro - zo ri|, each product and sum
 //        rounded at most twice: off by less than 3u (|zo| ri + |zi| ro +
 //        2 zmax (ro + ri)); taken as 8u with the layers' largest values.  F >
 //        0 implies ro > ri.
 //  PhiW  the condition is tan Dt - |C| >= 0 (Dt > 0 follows): |C| and Dt are
 //        off by 2u ri ro, tan by 2u relative: less than 5u ri ro (1 + tan),
-//        taken as 8u; |x|, |y| <= r + 2^-14.
+//        taken as 8u; |x|, |y| <= r + 2^-13.
 //  PT    H = |o-i|^2 |i|^2 - k C^2 with k = k_pt / |o|^2: the first term and k
 //        are off by 7u relative (differences of grid values are exact, sums of
 //        squares 3u, the product and the quotient the rest), C by c = 2u ri ro
@@ -210,7 +225,7 @@ __device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane,
         // inner layer's radii with a margin far above the rounding of the
         // float32 arcsines, narrows the window to this outer hit.
         float dphi = w.dphi;
-        if (w.pa > 0.f && ro * w.pa < 1.f) {
+        if (w.pa > 0.f && ro * w.pa < 0.9f) {
             const float so = window_asin(ro * w.pa);
             if (kPi - so - w.sx > dphi + 1e-3f) dphi = fminf(dphi, fmaxf(so - w.si, w.sx - so) + 1e-4f);
         }
