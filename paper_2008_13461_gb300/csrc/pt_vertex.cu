@@ -240,14 +240,6 @@ struct Members {
     }
 };
 
-// (float)(1 / sqrt(s)): by one Newton step from a float32 seed where s is
-// well inside its range (relative error ~1e-14 before the rounding)
-__device__ __forceinline__ float error_of_weight(double s) {
-    if (!(s > 1e-30 && s < 1e30)) return (float)(1.0 / sqrt(s));
-    const double y = (double)rsqrtf((float)s);
-    return (float)(y * (1.5 - 0.5 * s * y * y));
-}
-
 // sort element: z0 and record, in order of (z0, track index)
 struct ZRec {
     float z;
@@ -718,14 +710,13 @@ __global__ void __launch_bounds__(32 * kFitWarps) k_vtx_fit(VtxArgs a) {
     for (int part = 0; part < (split ? 2 : 1); part++) {
         const double zv = part ? z1 : z0, sw = part ? s.sw1 : s.sw0;
         if (split) m.chi2_pt2(part, zv, pt, chi2, pt2);
-        const float ez = error_of_weight(sw);
         int v = 0;
         if (lane == 0) {
             v = atomicAdd(a.nv + e, 1);
             if (v < kVtxCap) {
                 const int o = e * kVtxCap + v;
                 a.vz[o] = zv;
-                a.vez[o] = ez;
+                a.vez[o] = (float)(1.0 / sqrt(sw));
                 a.vc2[o] = (float)chi2;
                 a.vnt[o] = split ? (part ? s.n1 : n - s.n1) : n;
                 a.vsp[o] = pt2;
