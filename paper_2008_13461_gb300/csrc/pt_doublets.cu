@@ -21,33 +21,12 @@ namespace ptk {
 constexpr float kTwoPiInv = 0.159154943f;
 constexpr float kPi = 3.14159265f;
 
-// Angles for the windows, whose margins are 1e-4: arctangent and arcsine by the
-// polynomials 4.4.49 (below 1e-5 rad) and 4.4.46 (2e-8) of Abramowitz and Stegun,
-// Handbook of Mathematical Functions.
-__device__ __forceinline__ float window_atan2(float y, float x) {
-    const float ax = fabsf(x), ay = fabsf(y), hi = fmaxf(ax, ay);
-    const float q = hi > 0.f ? __fdividef(fminf(ax, ay), hi) : 0.f, q2 = q * q;
-    float a = q * fmaf(q2, fmaf(q2, fmaf(q2, fmaf(q2, 0.0208351f, -0.0851330f), 0.1801410f), -0.3302995f), 0.9998660f);
-    a = ay > ax ? 0.5f * kPi - a : a;
-    a = x < 0.f ? kPi - a : a;
-    return copysignf(a, y);
-}
-__device__ __forceinline__ float window_asin(float x) {   // 0 <= x < 1
-    float c = fmaf(x, -0.0012624911f, 0.0066700901f);
-    c = fmaf(x, c, -0.0170881256f);
-    c = fmaf(x, c, 0.0308918810f);
-    c = fmaf(x, c, -0.0501743046f);
-    c = fmaf(x, c, 0.0889789874f);
-    c = fmaf(x, c, -0.2145988016f);
-    c = fmaf(x, c, 1.5707963050f);
-    const float d = 1.0f - x;
-    return 0.5f * kPi - d * rsqrtf(d) * c;
-}
-
 // What a sweep needs of a layer pair, in shared memory (a lane-wise index
 // into the kernel's parameters serialises, and what does not depend on the
 // outer hit is worked out once: 1623 -> 1544 us for 64 PU200 events, 105 -> 97
-// for 32 PU50 events; the polynomials above 1535 -> 1494 and 99 -> 95).
+// for 32 PU50 events).  The angles and quotients of a window are those of CUDA's
+// float32 functions: polynomials of 1e-5 for the angles gave 3 to 4% of the
+// kernel, and other rows of tiles where a window ends within 1e-5 of an edge.
 struct PairWin {
     float zlo, zhi, zmax, tan, k_pt, ez, ep, ec;     // cuts, and the filter's bounds
     float dphi;                                      // azimuthal half window of PhiW
@@ -95,13 +74,11 @@ __device__ __forceinline__ void load_windows(const Params &p, PairWin *win) {
 }
 
 // Conservative window of the inner hit's t coordinate for a pair, from ZIP
-// (z-intercept within +-zmax) and ZW, over the inner layer's envelope; iro =
-// 1 / ro.  The quotients are good to a few ulp: below 3e-5 cm at the largest
-// z, inside the sweep's margin.
-__device__ __forceinline__ void t_window(const PairWin &w, float ro, float iro, float zo, float &tlo, float &thi) {
+// (z-intercept within +-zmax) and ZW, over the inner layer's envelope.
+__device__ __forceinline__ void t_window(const PairWin &w, float ro, float zo, float &tlo, float &thi) {
     const float zm = w.zmax;
     if (w.inner >= 0) {
-        float f0 = w.rmin * iro, f1 = w.rmax * iro;
+        float f0 = w.rmin / ro, f1 = w.rmax / ro;
         float c0 = -zm + (zo + zm) * f0, c1 = -zm + (zo + zm) * f1;
         float c2 = zm + (zo - zm) * f0, c3 = zm + (zo - zm) * f1;
         tlo = fmaxf(fminf(fminf(c0, c1), fminf(c2, c3)), w.zlo);
@@ -110,9 +87,9 @@ __device__ __forceinline__ void t_window(const PairWin &w, float ro, float iro, 
     } else {
         const float za = w.za, zb = w.zb;
         if (fabsf(zo) > zm * 1.001f + 0.01f && za <= zb) {
-            const float q0 = __fdividef(ro, zo + zm), q1 = __fdividef(ro, zo - zm);   // same sign
-            float c0 = q0 * (za + zm), c1 = q0 * (zb + zm);
-            float c2 = q1 * (za - zm), c3 = q1 * (zb - zm);
+            const float d0 = zo + zm, d1 = zo - zm;   // same sign
+            float c0 = ro * (za + zm) / d0, c1 = ro * (zb + zm) / d0;
+            float c2 = ro * (za - zm) / d1, c3 = ro * (zb - zm) / d1;
             tlo = fminf(fminf(c0, c1), fminf(c2, c3));
             thi = fminf(fmaxf(fmaxf(c0, c1), fmaxf(c2, c3)), ro);
             if (tlo > thi) tlo = thi = 0.5f * (tlo + thi);
@@ -140,9 +117,10 @@ __device__ __forceinline__ void t_window(const PairWin &w, float ro, float iro, 
 //  PhiW  the condition is tan Dt - |C| >= 0 (Dt > 0 follows): |C| and Dt are
 //        off by 2u ri ro, tan by 2u relative: less than 5u ri ro (1 + tan),
 //        taken as 8u; |x|, |y| <= r + 2^-13.
-//  PT    H = |o-i|^2 |i|^2 - k C^2 with k = k_pt / |o|^2: the first term and k
-//        are off by 7u relative (differences of grid values are exact, sums of
-//        squares 3u, the product and the quotient the rest), C by c = 2u ri ro
+//  PT    H = |o-i|^2 |i|^2 - k C^2 with k = k_pt / |o|^2: the first term is off
+//        by 7u relative (differences of grid values are exact, sums of squares
+//        3u), k by 8u (the quotient 4u) and its product with C^2 by two more,
+//        C by c = 2u ri ro
 //        (taken as 4u) and so k C^2 by k (2 |C| c + c^2) besides; taken as
 //        16u (P + k C^2) + k (4 |C| c + 2 c^2).
 struct PairFilter {
@@ -194,8 +172,8 @@ __device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane,
     const float4 ho = __ldg(p.bh + o);
     const float xo = ho.x, yo = ho.y, zo = ho.z, ro = ho.w;
     const int Lo = p.blayer[o], ev = p.bev[o];
-    const float phio = window_atan2(yo, xo);
-    const float io2 = __fdividef(1.0f, fmaf(xo, xo, yo * yo)), iro = __fdividef(1.0f, ro);
+    const float phio = atan2f(yo, xo);
+    const float io2 = __fdividef(1.0f, fmaf(xo, xo, yo * yo));
     const unsigned lanes = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     const unsigned below = (1u << lane) - 1u;
     int count = 0;
@@ -204,7 +182,7 @@ __device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane,
         const int pi = p.pairs_by_outer[Lo][k];
         const PairWin &w = win[pi];
         float tlo, thi;
-        t_window(w, ro, iro, zo, tlo, thi);
+        t_window(w, ro, zo, tlo, thi);
         const float tmin = w.inner >= 0 ? w.za : w.rmin;
         // Tile ranges: the t window's float32 bounds are within ~1e-5 cm of
         // the exact ones, so a margin of 1e-4 cm keeps every accepted hit
@@ -226,7 +204,7 @@ __device__ int sweep_outer(const Params &p, const PairWin *win, int o, int lane,
         // float32 arcsines, narrows the window to this outer hit.
         float dphi = w.dphi;
         if (w.pa > 0.f && ro * w.pa < 0.9f) {
-            const float so = window_asin(ro * w.pa);
+            const float so = asinf(ro * w.pa);
             if (kPi - so - w.sx > dphi + 1e-3f) dphi = fminf(dphi, fmaxf(so - w.si, w.sx - so) + 1e-4f);
         }
         int f0 = __float2int_rd((phio - dphi + kPi) * (p.n_phi * kTwoPiInv));
