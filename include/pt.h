@@ -163,7 +163,10 @@ typedef struct {
     int32_t doublet_lanes;  /* lanes per outer hit: 4, 8, 16 or 32 (for few hits more are used) */
     int32_t connect_lanes;  /* reserved (4, 8, 16 or 32 accepted); the CA
                                connection runs one warp per middle hit */
-    int32_t blocks_per_sm;  /* persistent grid size factor, 1..32 */
+    int32_t blocks_per_sm;  /* 1..32: at most so many blocks of 256 threads per SM in
+                               every persistent kernel (of 128 in the Fishbone's two-warp
+                               teams and the fit's adjoint); each takes no more than is
+                               useful to it, so from 14 on all grids are the largest */
 } pt_tuning;
 
 typedef struct {

@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(128) k_connect_exact(Params p) {
 void launch_connect(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_connect", s);
-        launch_pdl(k_connect, g.blocks(12), 32 * kCaWarps, 0, s, p);
+        launch_pdl(k_connect, g.blocks(12, 2), 32 * kCaWarps, 0, s, p);
     }
     KernelTimer t("k_connect_exact", s);
     launch_pdl(k_connect_exact, g.blocks(4), 128, 0, s, p);

@@ -539,7 +539,7 @@ void launch_fishbone(const Params &p, float unit_thr, float du, const Grid &g, c
     }
     {
         KernelTimer t("k_fishbone_medium", s);
-        launch_pdl(k_fishbone_large<kFbMidWarps, kFbMidMax, 512, false, kFbMidBlocks>, g.blocks(kFbMidBlocks),
+        launch_pdl(k_fishbone_large<kFbMidWarps, kFbMidMax, 512, false, kFbMidBlocks>, g.blocks(kFbMidBlocks, 2),
                    32 * kFbMidWarps, 0, s, p, unit_thr, du);
     }
     {

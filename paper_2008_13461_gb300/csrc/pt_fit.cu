@@ -534,18 +534,18 @@ template <typename R>
 void launch_fit_r(const Params &p, const Grid &g, cudaStream_t s) {
     {
         KernelTimer t("k_fit<3>", s);
-        launch_pdl(k_fit<3, R>, g.sms * 56, kFitThreads, 0, s, p);
+        launch_pdl(k_fit<3, R>, g.blocks(56, 4), kFitThreads, 0, s, p);
     }
     {
         KernelTimer t("k_fit<4>", s);
-        launch_pdl(k_fit<4, R>, g.sms * 44, kFitThreads, 0, s, p);
+        launch_pdl(k_fit<4, R>, g.blocks(44, 4), kFitThreads, 0, s, p);
     }
     {
         KernelTimer t("k_fit<5>", s);
-        launch_pdl(k_fit<5, R>, g.sms * 16, kFitThreads, 0, s, p);
+        launch_pdl(k_fit<5, R>, g.blocks(16, 4), kFitThreads, 0, s, p);
     }
     KernelTimer t("k_fit<6..8>", s);
-    launch_pdl(k_fit<6, R>, g.sms * 4, kFitThreads, 0, s, p);
+    launch_pdl(k_fit<6, R>, g.blocks(4, 4), kFitThreads, 0, s, p);
 }
 
 void launch_fit(const Params &p, const Grid &g, cudaStream_t s) {

@@ -715,18 +715,18 @@ void launch_fit_grad(const Params &p, const float *gpar, const float *gchi, floa
                      cudaStream_t s) {
     {
         KernelTimer t("k_fit_grad<3>", s);
-        launch_pdl(k_fit_grad<3>, g.sms * 20, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<3>, g.blocks(20, 2), kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<4>", s);
-        launch_pdl(k_fit_grad<4>, g.sms * 16, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<4>, g.blocks(16, 2), kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     {
         KernelTimer t("k_fit_grad<5>", s);
-        launch_pdl(k_fit_grad<5>, g.sms * 8, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
+        launch_pdl(k_fit_grad<5>, g.blocks(8, 2), kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
     }
     KernelTimer t("k_fit_grad<6..8>", s);
-    launch_pdl(k_fit_grad<6>, g.sms * 4, kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
+    launch_pdl(k_fit_grad<6>, g.blocks(4, 2), kGradThreads, 0, s, p, gpar, gchi, gx, gy, gz);
 }
 
 void launch_align(int n, const float *x, const float *y, const float *z, const int32_t *module, const float *centre,

@@ -45,13 +45,16 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, int block, size_t smem, 
 }
 
 // Size of a persistent grid: `resident` blocks per SM (what the kernel's
-// registers and shared memory let an SM hold), or the tuning's factor when
-// that is smaller.  More blocks than are resident only start, find the queue
+// registers and shared memory let an SM hold), or what the tuning's factor
+// allows when that is smaller: `per` blocks for each unit of it, a unit being 256 threads
+// (128 in the Fishbone's two-warp teams and in the adjoint), so that a caller who
+// lowers the factor to leave room on the SMs gets that from every kernel.  More
+// blocks than are resident only start, find the queue
 // or the range used up, and end: 5-10 us of empty waves per kernel in the
 // smallest events with a grid of 24 blocks per SM whatever the kernel.
 struct Grid {
     int sms, factor;
-    int blocks(int resident) const { return sms * (factor < resident ? factor : resident); }
+    int blocks(int resident, int per = 1) const { return sms * (factor * per < resident ? factor * per : resident); }
 };
 
 void launch_scan(int32_t *a, int64_t n, int32_t *part, cudaStream_t s);
