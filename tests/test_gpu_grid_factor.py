@@ -101,6 +101,12 @@ def test_the_default_and_the_largest_factor_launch_the_same():
     assert grids(24) == grids(32)
 
 
+def test_the_tuner_tries_no_two_factors_that_launch_the_same():
+    from paper_2008_13461_gb300.autotune import SPACE
+    tried = [grids(f) for f in dict(SPACE)["blocks_per_sm"]]
+    assert all(tried[i] != tried[j] for i in range(len(tried)) for j in range(i))
+
+
 def test_results_do_not_depend_on_the_factor():
     from parity import compare_sets, compare_tracks, gpu_run, oracle_run
     b = E.make_batch("barrel-50-helices", n_events=1)
