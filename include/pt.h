@@ -161,8 +161,8 @@ typedef struct {
     int32_t n_phi_bins;     /* azimuthal tiles per layer, 16..1024 */
     int32_t n_t_bins;       /* tiles along z (barrel) or r (disks), 1..64 */
     int32_t doublet_lanes;  /* lanes per outer hit: 4, 8, 16 or 32 (for few hits more are used) */
-    int32_t connect_lanes;  /* reserved (4, 8, 16 or 32 accepted); the CA
-                               connection runs one warp per middle hit */
+    int32_t connect_lanes;  /* reserved (4, 8, 16 or 32 accepted): the warps of the
+                               CA connection take chunks of up to 128 cells */
     int32_t blocks_per_sm;  /* 1..32: at most so many blocks of 256 threads per SM in
                                every persistent kernel (of 128 in the Fishbone's two-warp
                                teams and the fit's adjoint); each takes no more than is

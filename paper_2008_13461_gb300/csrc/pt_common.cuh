@@ -10,7 +10,7 @@
 
 namespace ptk {
 
-constexpr int kThreads = 256;            // threads per block of every kernel
+constexpr int kThreads = 256;            // threads per block, unless a kernel says otherwise
 constexpr int kMaxPairsPerLayer = 8;
 // workspace counters (int32 slots at the start of ws).  The ones every warp
 // of a kernel adds to have 128 bytes to themselves: an L2 slice takes about
@@ -49,7 +49,7 @@ __device__ __forceinline__ int sk_bucket(float key, float k0, float iw, int nb) 
 
 // The ends of those buckets, for the connection to start at: one per 1 << sk_end_shift
 // buckets, as many as leave no more of them than cells (a power of
-// two), for hits of up to kSkEnds cells (what a warp of the Fishbone sorts).
+// two), for hits of up to kSkEnds cells (what a team of the Fishbone sorts).
 constexpr int kSkEnds = 1024;
 __device__ __forceinline__ int sk_ends(int n) { return 1 << (31 - __clz(n)); }
 __device__ __forceinline__ int sk_end_shift(int n) { return max(5, 32 - __clz(n - 1)) - (31 - __clz(n)); }

@@ -11,7 +11,7 @@
 // window; the Fishbone also leaves the ends of the buckets, so the run is
 // found with two loads (a binary search took about seven one after the
 // other: 2167 -> 1970 us for 64 PU200 events, and the ends cost the Fishbone 55).
-// Longer lists than a warp of the Fishbone sorts are searched.
+// Lists that are longer than a team of the Fishbone sorts are searched.
 //
 // The R-z cut is very tight, so it is first used as a window on the slope
 // key.  For a barrel b, with key = dz/dr of a segment,

@@ -43,7 +43,8 @@ template <int M>
 __device__ __forceinline__ int pidx(int r, int c) { return r * (r + 1) / 2 + c; }
 
 // 1/sqrt(s) and 1/d in the solve's precision R.  Double: from a float32
-// seed and one Newton step (relative error 1e-7 -> ~1e-14), to keep the slow
+// seed and one Newton step (relative error up to 2.7e-7 -> 1.1e-13 for the
+// root, 1.2e-7 -> 1.4e-14 for the reciprocal), to keep the slow
 // FP64 pipe to a few multiply-adds; float: IEEE square root and division.
 __device__ __forceinline__ double rsqrt_r(double s) {
     const double y = (double)rsqrtf((float)s);

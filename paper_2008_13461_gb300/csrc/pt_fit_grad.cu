@@ -30,7 +30,8 @@ template <int M>
 __device__ __forceinline__ int pk(int r, int c) { return r >= c ? r * (r + 1) / 2 + c : c * (c + 1) / 2 + r; }
 
 // Reciprocal, reciprocal square root and square root from a float32 seed and
-// one Newton step (relative error about 1e-14): a few FP64 multiply-adds
+// one Newton step (relative error up to 1.4e-14 for the reciprocal, 1.1e-13 for
+// the roots, whose seed may be two units off): a few FP64 multiply-adds
 // instead of the full IEEE sequences on the slow FP64 pipe.  Used where the
 // argument is nonzero and well inside the float32 range (lengths, weights,
 // variances); sqrt_d(0) = 0.

@@ -28,7 +28,10 @@
 // memory, so that every track's compatible tracks lie in a window around it;
 // densities and links come from window scans (two threads per track, one to
 // each side), roots from pointer jumping, candidates from a counting sort of
-// the tracks by root.  The sort by z0 is a counting sort too (by z0 tile, a
+// the tracks by root.  With few tracks per event that block does all of it
+// (k_vtx_group); with many on average the window scans of all events run
+// over every SM in between (k_vtx_sort, k_vtx_density, k_vtx_link,
+// k_vtx_roots).  The sort by z0 is a counting sort too (by z0 tile, a
 // tile's few entries ranked by comparing them with each other); where a tile
 // is crowded a bitonic sort takes over.  The candidates' fits and 2-means splits, the
 // float64 part, then run one warp per candidate over the candidates of all
@@ -607,7 +610,7 @@ __global__ void __launch_bounds__(kVtxThreads, 1) k_vtx_group(VtxArgs a) {
 // events).  What bounds it is the float64 pipe and the longest split: with a
 // butterfly per sum, a division per centre, the members read again in every
 // round and the outputs summed anew, 24 PU200 events (194 vertices of 25
-// tracks each, up to 192) took 122 us; 66 us now.
+// tracks each, up to 192) took 122 us; 70 us now.
 constexpr int kFitWarps = 8;
 
 __global__ void __launch_bounds__(32 * kFitWarps) k_vtx_fit(VtxArgs a) {
@@ -892,8 +895,10 @@ pt_status launch_vertices(const pt_vertex_tracks &in, int32_t n_tracks, int32_t 
     // summaries of which a third are eligible, one block against four kernels
     // measured 35 / 49 us at 3400 tracks per event, 50 / 57 us at 5100 and
     // 67 / 62 us at 6800; for fitted PU200 events (48,600 tracks, a tenth
-    // eligible) 225 / 106 us.  The line lies between, where either costs the
-    // other at most ~15 us.
+    // eligible) 225 / 106 us.  For events of like size the line lies where
+    // either costs at most ~15 us more than the other.  The host knows only the
+    // mean: one large event among many small ones is left to its block, at up
+    // to the 225 us above.
     const bool split = n_tracks / n_events > kVtxSplit;
     // per device and call (cheap; no shared state between threads or devices)
     auto big_smem = [](void (*k)(VtxArgs)) {
