@@ -1,8 +1,9 @@
-"""Hits whose r is not the hypotenuse of x and y.  The contract ties r to its
-layer's envelope only, and every predicate reads r or (x, y), so the cells
-are exact whatever the two say of each other: pairs within rounding of the
-azimuth and curvature cuts where x and y are far larger than r, and pairs
-beyond the azimuth window that r alone would suggest."""
+"""Decisions within rounding of the doublet cuts, and hits whose r is not the
+hypotenuse of x and y.  The contract ties r to its layer's envelope only, and
+every predicate reads r or (x, y), so the cells are exact whatever the two
+say of each other: pairs next to the azimuth and curvature cuts where x and y
+are far larger than r, next to the intercept cut over whole envelopes, and
+pairs beyond the azimuth window that r alone would suggest."""
 import numpy as np
 import pytest
 
@@ -77,6 +78,38 @@ def _near_the_cut(cut: str, far, seed: int, n: int):
 @pytest.mark.parametrize("far", [(3.0, 7.0), (20.0, 30.0), (40.0, 45.0)])
 def test_pairs_within_rounding_of_a_cut(cut, far):
     pairs, cuts = _near_the_cut(cut, far, 3, 4000)
+    kept = _compare(pairs, cuts)
+    assert 0.1 * len(pairs) < kept < 0.9 * len(pairs)
+
+
+def _near_the_intercept(inner: int, outer: int, seed: int, n: int):
+    """Pairs on one azimuth within 2e-7 of the ZIP cut (relative to its
+    terms), over the whole of both layers' envelopes."""
+    rng = np.random.default_rng(seed)
+    li, lo, zmax = LAYERS[inner], LAYERS[outer], 12.0
+    out = []
+    while len(out) < n:
+        m = 200000
+        ri, zi, zo = (_snap(rng.uniform(a + 0.01, b - 0.01, m))
+                      for a, b in ((li.rmin, li.rmax), (li.zmin, li.zmax), (lo.zmin, lo.zmax)))
+        side = rng.choice([-zmax, zmax], m)
+        ro = _snap(ri * (zo - side) / np.where(zi == side, np.nan, zi - side))
+        left, right = np.abs(zi * ro - zo * ri), zmax * (ro - ri)
+        near = (ro > lo.rmin) & (ro < lo.rmax) & (ro > ri) & (np.abs(left - right) <= 2e-7 * (left + right))
+        phi = rng.uniform(-np.pi, np.pi, m)
+        for k in np.nonzero(near)[0]:
+            xy = [(float(_snap(r * np.cos(phi[k]))), float(_snap(r * np.sin(phi[k])))) for r in (ri[k], ro[k])]
+            out.append(((*xy[0], zi[k], ri[k], inner), (*xy[1], zo[k], ro[k], outer)))
+    cuts = CU.make_cuts(pt_min=0.5)
+    for pc in cuts["pairs"]:
+        pc["zmax"], pc["zlo"], pc["zhi"] = zmax, -60.0, 60.0
+    return out[:n], cuts
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("inner,outer", [(0, 1), (2, 3), (0, 4), (1, 7), (4, 6), (8, 9)])
+def test_pairs_within_rounding_of_the_intercept(inner, outer):
+    pairs, cuts = _near_the_intercept(inner, outer, 8, 2000)
     kept = _compare(pairs, cuts)
     assert 0.1 * len(pairs) < kept < 0.9 * len(pairs)
 
